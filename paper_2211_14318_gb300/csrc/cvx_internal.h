@@ -40,13 +40,32 @@ struct ItemCands {
     int n, flags, pad;
 };
 
+// Constants of a queued node that its line scan needs, written by k_nodes
+// before the scan, one thread per node: in FP64 they take four exponentials
+// and logarithms, which on one lane of a scanning warp cost as much as on 32
+// (the FP64 pipe has 2 lanes per SM and clock; of 133 ms for 1,048,576 points,
+// 16^2 directions, L = 201, this was 22 ms).
+struct ScanConsts {
+    float C, sa, cb, w0;  // sample shift, tangent-slope constants, FP32 centre sample
+    // centre expansion of the line function for the no-split certificate:
+    // d0 = d(0), B1p = B1 + 2 B2 lg0 (lg0 = log2 J0), gp = dv/dd at d0,
+    // k1e = K1 2^{-d0} (d0 > 0, else 0), invJ0 = 1 / J0
+    float d0, B1p, gp, k1e, invJ0;
+    float d0abs;  // |A0| + |lg0| (|B1| + B2 |lg0|): magnitude of the terms of d0
+    int e;        // the node's window exponent (line spacing h 2^e)
+};
+
 struct NodeCands {
-    int dir[kNodeCand];
+    // the scan's constants until k_select reads its results, then the candidates
+    union {
+        int dir[kNodeCand];
+        ScanConsts sc;
+    };
     int ab[kNodeCand];  // FP32 bridge pair hint per candidate (as in ItemCands), -1 if unknown
     int n, flags;
     float qcut;  // smallest FP32 q of a direction not refined (sample units)
     float eps;   // FP32 error bound used at this node (sample units)
-    // node constants for the FP64 refinement, computed once per node
+    // node constants of the scan and of the FP64 refinement, written by k_nodes
     NodeLine nl;  // FP32 line constants (make_node_line)
     double ek;    // exp(-beta_k / D_0)
     double shift; // sample shift C in FP64 (line_shift)

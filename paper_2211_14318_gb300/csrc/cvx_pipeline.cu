@@ -2,6 +2,7 @@
 // of problems (convexify_points is a batch of one).
 //
 // Per lamination level (Eq. 3.3, top-down):
+//   k_nodes   per queued node: its line constants (FP64, rounded to FP32)
 //   k_scan    FP32 screening: every direction's line is sampled (Eq. 4.4),
 //             bounds on its hull value at t = 0 (Algorithm 1 read at t = 0)
 //             are found and the best directions kept per work item -- the hot
@@ -124,6 +125,47 @@ __global__ void k_init(const Pipe P) {
 }
 
 // -------------------------------------------------------------------------
+// k_nodes: one thread per queued node, before the scan: the node's FP32 line
+// constants and FP64 history terms (scan, selection and refinement read
+// them), and the node's upper-bound word.
+// -------------------------------------------------------------------------
+__global__ void k_nodes(const Pipe P, int level) {
+    const int qi = blockIdx.x * blockDim.x + threadIdx.x;
+    if (qi >= P.cnt[level]) return;
+    const int p = P.qp[level][qi];
+    const ProbDesc &pd = P.probs[P.pid[p]];
+    const cvx_node *nd = node_ptr(pd, p, P.qh[level][qi]);
+    const double F[4] = {nd->F[0], nd->F[1], nd->F[2], nd->F[3]};
+    const double beta = pd.beta[p - pd.point_off];
+    NodeCands &nc = P.cands[qi];
+    const NodeLine nl = make_node_line(F, beta, pd.mat);
+    const double shift = line_shift(pd.mat, beta);
+    nc.nl = nl;
+    nc.ek = exp(-beta / pd.mat.D0);
+    nc.shift = shift;
+    P.node_u[qi] = 0x7f7f7f7f;  // the node's upper bound starts at a huge finite key
+    if (P.energy != CVX_ENERGY_NH_DAMAGE) return;
+    ScanConsts c;
+    c.C = (float)shift;
+    c.e = nd->window_exp;
+    center_slope_consts(nl, scaled_line(pd.line, c.e).h64, c.sa, c.cb);
+    DirLine d0;
+    d0.A1 = d0.A2 = d0.cJ = 0.0f;
+    d0.J0 = nl.J0;
+    c.w0 = sample_w<CVX_ENERGY_NH_DAMAGE>(nl, d0, 0.0f);
+    const double J0 = nl.J0, lg0 = J0 > 0.0 ? log2(J0) : 0.0;
+    const double dc = (double)nl.A0 + lg0 * ((double)nl.B1 + (double)nl.B2 * lg0);
+    const double e2 = exp2(-dc);
+    c.d0 = (float)dc;
+    c.B1p = (float)((double)nl.B1 + 2.0 * (double)nl.B2 * lg0);
+    c.gp = (float)(dc < 0.0 ? 1.0 + (double)nl.K2 : 1.0 + (double)nl.K1 * kLn2d * e2);
+    c.k1e = dc > 0.0 ? (float)((double)nl.K1 * e2) : 0.0f;
+    c.invJ0 = J0 > 0.0 ? (float)(1.0 / J0) : 0.0f;
+    c.d0abs = (float)(fabs((double)nl.A0) + fabs(lg0) * (fabs((double)nl.B1) + (double)nl.B2 * fabs(lg0)));
+    nc.sc = c;
+}
+
+// -------------------------------------------------------------------------
 // k_scan: persistent CTAs take work items (node, block of directions) from an
 // atomic counter.  Each warp scans a contiguous run of directions,
 // warm-starting every hull search from the previous direction's bridge, and
@@ -180,15 +222,15 @@ __global__ void __launch_bounds__(32 * kScanWarps, CVX_SCAN_MIN_BLOCKS) k_scan(c
                 s_pd = P.probs[P.pid[p]];
                 if (win) s_c = P.center[qi];
                 if (ch < pass_chunks(s_pd, P.pass)) {
-                    const cvx_node *nd = node_ptr(s_pd, p, hi);
-                    double F[4] = {nd->F[0], nd->F[1], nd->F[2], nd->F[3]};
-                    const double beta = s_pd.beta[p - s_pd.point_off];
-                    s_nl = make_node_line(F, beta, s_pd.mat);
-                    s_shift = (float)line_shift(s_pd.mat, beta);
+                    const NodeCands &nc = P.cands[qi];
+                    s_nl = nc.nl;
+                    s_shift = (float)nc.shift;
                     s_ukey = f2key(INFINITY);
-                    s_e = nd->window_exp;
-                    if (EK == CVX_ENERGY_NH_DAMAGE)
-                        center_slope_consts(s_nl, scaled_line(s_pd.line, s_e).h64, s_sa, s_cb);
+                    s_e = node_ptr(s_pd, p, hi)->window_exp;
+                    if (EK == CVX_ENERGY_NH_DAMAGE) {
+                        s_sa = nc.sc.sa;
+                        s_cb = nc.sc.cb;
+                    }
                 }
             }
         }
@@ -496,10 +538,11 @@ __global__ void k_select(const Pipe P, int level) {
         U = fminf(U, r[c].qhi_min);
         fl |= r[c].flags;
     }
-    NodeCands nc;
-    nc.n = 0;
+    NodeCands &nc = P.cands[qi];  // (the scan is done with the constants in nc.sc)
+    const double shift64 = nc.shift;
+    int n = 0;
     float cq[kNodeCand];  // the candidates' FP32 lower bounds
-    const float shift = (float)line_shift(pd.mat, pd.beta[P.qp[level][qi] - pd.point_off]);
+    const float shift = (float)shift64;
     const float kap = pd.kappa_f;
     // a direction is a candidate iff q - eps(q) <= m + eps(m), m = min(W(F), U)
     const float mref = fminf(w0, U);
@@ -520,43 +563,34 @@ __global__ void k_select(const Pipe P, int level) {
             }
             if (bc < 0) break;
             const float q = r[bc].q[pos[bc]];
-            if (!(q - eps32_at(q, kap, shift) <= R) || nc.n == kNodeCand) {
+            if (!(q - eps32_at(q, kap, shift) <= R) || n == kNodeCand) {
                 qcut = fminf(qcut, q);
                 break;
             }
-            cq[nc.n] = q;
-            nc.dir[nc.n] = r[bc].dir[pos[bc]];
-            nc.ab[nc.n++] = r[bc].ab[pos[bc]];
+            cq[n] = q;
+            nc.dir[n] = r[bc].dir[pos[bc]];
+            nc.ab[n++] = r[bc].ab[pos[bc]];
             ++pos[bc];
         }
         for (int c = nch; c < chunks; ++c) qcut = fminf(qcut, r[c].q[0]);
     } else {
         qcut = fminf(qcut, qmin);
     }
+    nc.n = n;
     nc.qcut = qcut;
     nc.eps = qcut < INFINITY ? eps32_at(qcut, kap, shift) : 0.0f;
     nc.flags = fl;
-    if (nc.n) {
-        // node constants of the FP64 refinement, once per node
-        const cvx_node *nd = node_ptr(pd, P.qp[level][qi], P.qh[level][qi]);
-        const double F[4] = {nd->F[0], nd->F[1], nd->F[2], nd->F[3]};
-        const double beta = pd.beta[P.qp[level][qi] - pd.point_off];
-        nc.nl = make_node_line(F, beta, pd.mat);
-        nc.ek = exp(-beta / pd.mat.D0);
-        nc.shift = line_shift(pd.mat, beta);
-    }
-    P.cands[qi] = nc;
-    if (nc.n) {
-        const int pos = atomicAdd(P.cnt + (P.K + 1) + level, nc.n);
-        for (int c = 0; c < nc.n; ++c) P.work[pos + c] = make_int2(qi, c);
+    if (n) {
+        const int pos = atomicAdd(P.cnt + (P.K + 1) + level, n);
+        for (int c = 0; c < n; ++c) P.work[pos + c] = make_int2(qi, c);
         // per candidate, a lower bound of its FP64 value in W units (as for
         // qcut in k_commit): (q - eps(q) + C) / kappa'; k_refine's second
         // phase skips a candidate whose bound exceeds the first one's value
         RefineOut *ro = P.refined + (long long)qi * kNodeCand;
-        for (int c = 0; c < nc.n; ++c) {
+        for (int c = 0; c < n; ++c) {
             const float q = cq[c];
             RefineOut o;
-            o.q = ((double)q - (double)eps32_at(q, kap, shift) + nc.shift) / pd.kappa;
+            o.q = ((double)q - (double)eps32_at(q, kap, shift) + shift64) / pd.kappa;
             o.a = o.b = -1;
             o.ok = 0;
             o.pad = kScreened;
@@ -1113,8 +1147,7 @@ __global__ void k_commit(const Pipe P, int level) {
     // FP64 node value among the refined directions; an unrefined direction
     // (FP32 q >= qcut) could only win if qcut - eps reached it
     const double V = (bc >= 0 && ro[bc].q < nd.w) ? ro[bc].q : nd.w;
-    const double shift = line_shift(pd.mat, pd.beta[p - pd.point_off]);
-    const bool overflow = !(((double)nc.qcut - (double)nc.eps + shift) / pd.kappa > V);
+    const bool overflow = !(((double)nc.qcut - (double)nc.eps + nc.shift) / pd.kappa > V);
     // the node's decision: the best refined direction, or (mirror stage) the
     // main window's when that one holds the lower value
     const bool split = bc >= 0 && ro[bc].q < nd.w;
@@ -1631,11 +1664,9 @@ cudaError_t pipe_level(const Pipe &p, int l, int warps, int grid, cudaStream_t s
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const long long max_nodes = p.N << l;
-    if (p.lanes) {
-        // the node bounds start at +inf (a huge finite key); reset outside the timed region
-        if ((e = cudaMemsetAsync(p.node_u, 0x7f, sizeof(int) * (size_t)max_nodes, s)) != cudaSuccess)
-            return e;
-    }
+    const unsigned nb = (unsigned)((max_nodes + 127) / 128);
+    k_nodes<<<nb, 128, 0, s>>>(p, l);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
     if (ev && (e = cudaEventRecord(ev[0], s)) != cudaSuccess) return e;
     if (p.lanes)
         e = launch_scan_lanes(p, l, sms, s);
@@ -1645,7 +1676,6 @@ cudaError_t pipe_level(const Pipe &p, int l, int warps, int grid, cudaStream_t s
                 : launch_scan_t<CVX_ENERGY_DOUBLE_WELL>(p, l, warps, grid, s);
     if (e != cudaSuccess) return e;
     if (ev && (e = cudaEventRecord(ev[1], s)) != cudaSuccess) return e;
-    const unsigned nb = (unsigned)((max_nodes + 127) / 128);
     k_select<<<nb, 128, 0, s>>>(p, l);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     const long long want = (max_nodes * kNodeCand + 3) / 4;

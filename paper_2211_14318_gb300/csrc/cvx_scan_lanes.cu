@@ -4,8 +4,9 @@
 // hull.
 //
 // A warp takes a work item (a node and up to 256 of its directions) and each
-// lane samples its own line, two samples per paired FP32 instruction, without
-// storing it.  For the hull at t = 0 of the left set {x < 0} and the right set
+// lane takes its own line, two samples per paired FP32 instruction, without
+// storing it, and without taking the samples that a bound of v'' shows to lie
+// above the minimum looked for (bb_pass).  For the hull at t = 0 of the left set {x < 0} and the right set
 // {x > 0} of the samples (x = m - m0) the pass at a slope s yields
 //   e_L = min over the left of (v - s x),  e_R = min over the right,
 // and their minimisers a < 0 < b.  For any s, min(e_L, e_R) is a lower bound
@@ -57,22 +58,13 @@ struct LaneState {
 };
 
 // Node constants of a warp's item.
-struct LaneNode {
+struct LaneNode : ScanConsts {
     NodeLine nl;
-    float C, sa, cb, w0;  // sample shift, tangent-slope constants, FP32 centre sample
-    // centre expansion of the line function for the no-split certificate:
-    // d0 = d(0), B1p = B1 + 2 B2 lg0 (lg0 = log2 J0), gp = dv/dd at d0,
-    // k1e = K1 2^{-d0} (d0 > 0, else 0), invJ0 = 1 / J0
-    float d0, B1p, gp, k1e, invJ0;
-    float d0abs;  // |A0| + |lg0| (|B1| + B2 |lg0|): magnitude of the terms of d0
-    int e;        // the node's window exponent (line spacing h 2^e)
 };
 
 struct SideMin {
-    float eL, eR;    // minima of v - s x over the left and the right samples
-    int kL, kR;      // pair index of each minimum, -1 if the side has no finite sample
-    float eLf, eRf;  // the same minima over the far samples only (outside the near
-                     // region [2 kf - m0, 2 kn], see line_pass)
+    float eL, eR;  // minima of v - s x over the left and the right samples
+    int kL, kR;    // pair index of each minimum, -1 if the side has no finite sample
 };
 
 __device__ __forceinline__ void side_update(f32x2 B, int k, float &e, int &kk) {
@@ -85,16 +77,15 @@ __device__ __forceinline__ void side_update(f32x2 B, int k, float &e, int &kk) {
     }
 }
 
-// Pass over a line at slope s = -ns.  Pairs (x, x + 1): left x = 2k - m0,
-// right x = 2k + 1, for k = k0, k0 + kstep, ... < m0 / 2; with m0 odd the
-// lane with k0 = 0 also takes the sample next to the centre on the left
-// (x = -1) and the last one on the right (x = m0) as pair m0 / 2.  The
-// samples are those of sample_w (each half of a paired instruction rounds
-// as the scalar one), at t = fl(x h).  Left pairs k >= kf and right pairs
-// k < kn form the near region (x in [2 kf - m0, -1] and [1, 2 kn]); the far
-// minima leave it out.
+// Full pass over a line at slope s = -ns, the pairs k0, k0 + kstep, ...: the
+// whole warp's pass over one line (k0 = lane, kstep = 32).  Pairs (x, x + 1):
+// left x = 2k - m0, right x = 2k + 1, k < m0 / 2; with m0 odd the lane with
+// k0 = 0 also takes the sample next to the centre on the left (x = -1) and
+// the last one on the right (x = m0) as pair m0 / 2.  The samples are those
+// of sample_w (each half of a paired instruction rounds as the scalar one),
+// at t = fl(x h).
 __device__ __forceinline__ SideMin line_pass(const NHPair &c, f32x2 H, float ns, int m0, int k0,
-                                             int kstep, int kf = 0, int kn = 0) {
+                                             int kstep) {
     SideMin r;
     r.eL = r.eR = INFINITY;
     r.kL = r.kR = -1;
@@ -103,42 +94,218 @@ __device__ __forceinline__ SideMin line_pass(const NHPair &c, f32x2 H, float ns,
     const float st = 2.0f * (float)kstep;
     const f32x2 STEP = pk2(st, st);
     f32x2 X = pk2((float)(2 * k0 - m0), (float)(2 * k0 - m0 + 1));
-    int k = k0;
 #pragma unroll 2
-    for (; k < kf; k += kstep) {
-        side_update(fma2(NS, X, sample_nh2(c, mul2(X, H))), k, r.eL, r.kL);
-        X = add2(X, STEP);
-    }
-    r.eLf = r.eL;
-#pragma unroll 2
-    for (; k < np; k += kstep) {
+    for (int k = k0; k < np; k += kstep) {
         side_update(fma2(NS, X, sample_nh2(c, mul2(X, H))), k, r.eL, r.kL);
         X = add2(X, STEP);
     }
     X = pk2((float)(2 * k0 + 1), (float)(2 * k0 + 2));
-    k = k0;
 #pragma unroll 2
-    for (; k < kn; k += kstep) {
+    for (int k = k0; k < np; k += kstep) {
         side_update(fma2(NS, X, sample_nh2(c, mul2(X, H))), k, r.eR, r.kR);
-        X = add2(X, STEP);
-    }
-    float ef = INFINITY;
-    int kk = -1;
-#pragma unroll 2
-    for (; k < np; k += kstep) {
-        side_update(fma2(NS, X, sample_nh2(c, mul2(X, H))), k, ef, kk);
         X = add2(X, STEP);
     }
     if ((m0 & 1) && k0 == 0) {
         X = pk2(-1.0f, -1.0f);
         side_update(fma2(NS, X, sample_nh2(c, mul2(X, H))), np, r.eL, r.kL);
         X = pk2((float)m0, (float)m0);
-        side_update(fma2(NS, X, sample_nh2(c, mul2(X, H))), np, ef, kk);
+        side_update(fma2(NS, X, sample_nh2(c, mul2(X, H))), np, r.eR, r.kR);
     }
-    r.eRf = ef;
-    if (ef < r.eR) {
-        r.eR = ef;
-        r.kR = kk;
+    return r;
+}
+
+// ---- the lane's own pass over a line: the same minima (bit for bit, lowest
+// pair on equal values) without sampling the whole line.
+//
+// A side is cut into intervals of 2 PP samples.  Only their end points are
+// sampled first.  Inside an interval of length delta in t the function
+// g = v - s x lies at most M delta^2 / 8 below the lower of its end values,
+// M any upper bound of v'' there, so an interval whose bound exceeds the
+// smallest sample seen so far cannot hold the side's minimum and is never
+// sampled.  The others (the interval of the minimum and its neighbours as a
+// rule) are sampled in full.
+//
+// Bound of v'': v = phi(d(t)) with phi' = 1 + K2' 2^{-max(d, 0)} (C ln 2 = K2')
+// positive and nonincreasing, phi'' <= 0, so v'' <= phi'(min d) max(d'', 0);
+//   d'' = 2 A2 + (cJ / J)^2 (c0 - c1 log2 J),
+//   c0 = 2 B2 / ln2^2 - B1 / ln2, c1 = 2 B2 / ln2,
+// whose positive part falls with J, so its maximum over eight intervals is
+// taken at their smallest J, and d lies at most eta = max(d'') delta^2 / 8
+// below its end values, which raises 2^{-d} by at most 2^eta <= 1 + eta
+// (eta <= 1).  Intervals that reach J <= 0 are always sampled; eight
+// intervals with J <= 0 throughout hold no finite sample.
+// The rounding of the samples (kEps32 max(kappa', |v| + C) bounds it, with
+// |v| <= |g| + |s| m0) is covered four times over: by `base` and by the term
+// in |e| of the comparison.
+// What bounds it: instruction issue (79 % of the slots at L = 201).  Taking
+// every sample instead: 3,001 load-path points, 128^2 directions, L = 2049,
+// depth 3: 326.9 ms of line scan, 70.9 ms with the intervals; 16,384 mesh
+// points, 64^2, L = 1025: 227.9 -> 70 ms; 1,048,576 points, 16^2, L = 201:
+// 86.9 -> 51 ms.  2.5 to 4.0 intervals are sampled per line, both sides
+// together.
+struct BBGeom {
+    float h, q8;  // sample spacing, delta^2 / 8
+    float rPP;    // 1 / PP
+    int m0, PP;   // samples per side, pairs per interval
+};
+
+// Pairs per interval on a side of m0 samples: about sqrt(m0) samples (an end
+// costs about two samples, one to two intervals per side are sampled), at
+// most 32 intervals per side (one mask bit each).  0.4 and 0.7 in place of
+// 0.5 measured 4 % slower at L = 201, 7 % slower and 2 % faster at L = 1025.
+constexpr float kBBScale = 0.5f;
+__device__ __forceinline__ BBGeom bb_geom(float h, int m0) {
+    BBGeom g;
+    g.h = h;
+    g.m0 = m0;
+    g.PP = max(max(((m0 >> 1) + 31) >> 5, (int)(kBBScale * sqrtf((float)m0) + 0.5f)), 1);
+    g.rPP = 1.0f / (float)g.PP;
+    g.q8 = 0.5f * (float)(g.PP * g.PP) * h * h;
+    return g;
+}
+
+__device__ __forceinline__ float bb_base(float kap, float C, float s, int m0) {
+    return 4.0f * kEps32 * (kap + C + fabsf(s) * (float)m0);
+}
+
+// g = v - s x at two samples, and 2^{-max(d, 0)} there.
+__device__ __forceinline__ void bb_eval(const NHPair &c, f32x2 H, f32x2 NS, f32x2 X, float &g0,
+                                        float &g1, float &E0, float &E1) {
+    const f32x2 T = mul2(X, H);
+    const f32x2 P = fma2(T, fma2(T, c.A2, c.A1), c.A0);
+    float j0, j1, d0, d1;
+    upk2(fma2(T, c.CJ, c.J0), j0, j1);
+    const f32x2 LG = pk2(lg2_approx(j0), lg2_approx(j1));
+    const f32x2 D = fma2(LG, fma2(LG, c.B2, c.B1), P);
+    upk2(D, d0, d1);
+    E0 = ex2_approx(-fmaxf(d0, 0.0f));
+    E1 = ex2_approx(-fmaxf(d1, 0.0f));
+    const f32x2 W = fma2(c.K2, pk2(fminf(d0, 0.0f), fminf(d1, 0.0f)), D);
+    upk2(fma2(NS, X, fma2(c.NK1, pk2(E0, E1), W)), g0, g1);
+}
+
+// The lane's pass at slope s = -ns over the left samples -m0 .. xlL (the
+// pairs k < kl, and x = -1 if that is a pair of its own) and the right pairs
+// k >= kr with the last sample m0 (kl = m0 / 2, xlL = -1, kr = 0: the whole
+// line).  xsL, xsR: samples of the two regions taken first (a neighbouring
+// line's minimisers).  Not inlined: three call sites share one copy, which
+// keeps the kernel in the instruction cache (inlined copies left the warps
+// waiting for instructions 6.4 cycles per issue).
+__device__ __noinline__ SideMin bb_pass(const LaneNode &N, const BBGeom &G, float A1, float A2,
+                                        float cJ, float ns, float base, int kl, int xlL, int kr,
+                                        int xsL, int xsR) {
+    const int m0 = G.m0, PP = G.PP, np = m0 >> 1;
+    const float h = G.h;
+    const f32x2 H = pk2(h, h), NS = pk2(ns, ns);
+    NHPair c = nh_pair_node(N.nl);
+    c.A1 = pk2(A1, A1);
+    c.A2 = pk2(A2, A2);
+    c.CJ = pk2(cJ, cJ);
+    const float J0 = N.nl.J0, K2 = N.nl.K2;
+    c.J0 = pk2(J0, J0);
+    const float c1 = 2.0f * N.nl.B2 * (1.0f / kLn2), c0 = (c1 - N.nl.B1) * (1.0f / kLn2);
+    const float fS = 2.0f * (float)PP;
+    float gs0, gs1, eu0, eu1;
+    bb_eval(c, H, NS, pk2((float)xsL, (float)xsR), gs0, gs1, eu0, eu1);
+    unsigned mL = 0, mR = 0;
+    float lastL = INFINITY, lastR = INFINITY;
+#pragma unroll 1
+    for (int side = 0; side < 2; ++side) {
+        const int xb = side ? 2 * kr + 1 : -m0;
+        const int xl = side ? m0 : xlL;
+        const int npr = side ? np - kr : kl;
+        if (xl < xb) continue;
+        const float fl = (float)xl;
+        float ga, g1, Ea, E1;
+        bb_eval(c, H, NS, pk2((float)xb, fl), ga, g1, Ea, E1);
+        float e = fmin3(side ? gs1 : gs0, ga, g1);
+        if (side) lastR = g1;
+        else lastL = g1;
+        const int NI = (int)(((float)(npr + PP - 1) + 0.5f) * G.rPP);
+        unsigned mask = 0;
+        float xa = (float)xb;  // the left end of the next interval
+#pragma unroll 1
+        for (int i0 = 0; i0 < NI; i0 += 8) {
+            // the largest d'' over the eight intervals
+            const float xe = fminf(__fmaf_rn(8.0f, fS, xa), fl);
+            const float Ja = __fmaf_rn(xa * h, cJ, J0), Je = __fmaf_rn(xe * h, cJ, J0);
+            const float Jm = fminf(Ja, Je);
+            if (!(fmaxf(Ja, Je) > 0.0f)) {
+                ga = INFINITY;
+                xa = xe;
+                continue;
+            }
+            const float r = __fdividef(cJ, Jm);
+            const float dd = __fmaf_rn(r * r, fmaxf(__fmaf_rn(-c1, lg2_approx(Jm), c0), 0.0f), 2.0f * A2);
+            float eta = dd * G.q8;
+            if (!(Jm > 0.0f) || !(eta < 1e30f)) eta = INFINITY;
+            const float up = eta <= 1.0f ? 1.0f + eta : INFINITY;
+            const float etc = 1.0001f * eta;
+            unsigned bit = 1u << i0;
+            const int ie = min(i0 + 8, NI);
+#pragma unroll 1
+            for (int i = i0; i < ie; i += 2, bit <<= 2) {
+                const float x0 = fminf(xa + fS, fl), x1 = fminf(__fmaf_rn(2.0f, fS, xa), fl);
+                float p0, p1, E0, E1b;
+                bb_eval(c, H, NS, pk2(x0, x1), p0, p1, E0, E1b);
+                e = fmin3(e, p0, p1);
+                // (Ea * up is NaN only where both are 0 and inf: fminf takes 1)
+                const float En = fminf(fmaxf(Ea, fmaxf(E0, E1b)) * up, 1.0f);
+                const float thr = __fmaf_rn(etc, __fmaf_rn(K2, En, 1.0f), base) +
+                                  __fmaf_rn(4.0f * kEps32, fabsf(e), e);
+                if (!(fminf(ga, p0) > thr)) mask |= bit;
+                if (!(fminf(p0, p1) > thr)) mask |= bit << 1;
+                ga = p1;
+                Ea = E1b;
+                xa = x1;
+            }
+        }
+        mask &= NI >= 32 ? 0xffffffffu : (1u << NI) - 1u;
+        if (side) mR = mask;
+        else mL = mask;
+    }
+    SideMin r;
+    r.eL = r.eR = INFINITY;
+    r.kL = r.kR = -1;
+    const f32x2 TWO = pk2(2.0f, 2.0f);
+#pragma unroll 1
+    while (mL | mR) {
+        const bool left = mL != 0;
+        const unsigned m = left ? mL : mR;
+        const int ka = (__ffs(m) - 1) * PP;
+        const int kb = min(left ? kl : np - kr, ka + PP);
+        float e = left ? r.eL : r.eR;
+        int kk = -1;
+        const float x = (float)((left ? -m0 : 2 * kr + 1) + 2 * ka);
+        f32x2 X = pk2(x, x + 1.0f);
+#pragma unroll 2
+        for (int k = ka; k < kb; ++k) {
+            float b0, b1;
+            upk2(fma2(NS, X, sample_nh2(c, mul2(X, H))), b0, b1);
+            const float en = fmin3(e, b0, b1);
+            if (en < e) kk = k;
+            e = en;
+            X = add2(X, TWO);
+        }
+        if (left) {
+            mL = m & (m - 1);
+            r.eL = e;
+            r.kL = kk >= 0 ? kk : r.kL;
+        } else {
+            mR = m & (m - 1);
+            r.eR = e;
+            r.kR = kk >= 0 ? kk + kr : r.kR;
+        }
+    }
+    // the last sample of a side with an odd number of them is a pair of its own
+    // (elsewhere it lies in the last pair)
+    if (lastL < r.eL) {
+        r.eL = lastL;
+        r.kL = np;
+    }
+    if (lastR < r.eR) {
+        r.eR = lastR;
+        r.kR = np;
     }
     return r;
 }
@@ -336,16 +503,14 @@ __device__ __forceinline__ int lane_window_dir(const ProbDesc &pd, int2 c, int j
 __global__ void __launch_bounds__(32 * kLaneWarps, CVX_LANE_MIN_BLOCKS)
     k_scan_lanes(const Pipe P, int level) {
     __shared__ LaneState s_st[kLaneWarps][kLaneItemMax];
-    __shared__ float s_ef[kLaneWarps][kLaneItemMax];  // far minimum of the first pass
     __shared__ unsigned short s_live[kLaneWarps][kLaneItemMax];
     __shared__ LaneNode s_nd[kLaneWarps];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const bool win = P.pass == PASS_WINDOW;
     const int n_nodes = P.cnt[level];
     const long long n_items = (long long)n_nodes * P.C;
-    const int32_t *qp = P.qp[level], *qh = P.qh[level];
+    const int32_t *qp = P.qp[level];
     LaneState *st = s_st[warp];
-    float *efl = s_ef[warp];
     unsigned short *live = s_live[warp];
     LaneNode &N = s_nd[warp];
     unsigned long long n_valid = 0;
@@ -361,30 +526,14 @@ __global__ void __launch_bounds__(32 * kLaneWarps, CVX_LANE_MIN_BLOCKS)
         const ProbDesc &pd = P.probs[P.pid[p]];
         const int chunks = win ? pd.wchunks : pd.chunks;
         if (ch >= chunks) continue;
-        if (lane == 0) {
-            const cvx_node *nd = node_ptr(pd, p, qh[qi]);
-            const double F[4] = {nd->F[0], nd->F[1], nd->F[2], nd->F[3]};
-            const double beta = pd.beta[p - pd.point_off];
-            N.nl = make_node_line(F, beta, pd.mat);
-            N.C = (float)line_shift(pd.mat, beta);
-            N.e = nd->window_exp;
-            center_slope_consts(N.nl, scaled_line(pd.line, N.e).h64, N.sa, N.cb);
-            DirLine d0;
-            d0.A1 = d0.A2 = d0.cJ = 0.0f;
-            d0.J0 = N.nl.J0;
-            N.w0 = sample_w<CVX_ENERGY_NH_DAMAGE>(N.nl, d0, 0.0f);
-            {
-                const double J0 = N.nl.J0, lg0 = J0 > 0.0 ? log2(J0) : 0.0;
-                const double dc = (double)N.nl.A0 + lg0 * ((double)N.nl.B1 + (double)N.nl.B2 * lg0);
-                const double e2 = exp2(-dc);
-                N.d0 = (float)dc;
-                N.B1p = (float)((double)N.nl.B1 + 2.0 * (double)N.nl.B2 * lg0);
-                N.gp = (float)(dc < 0.0 ? 1.0 + (double)N.nl.K2 : 1.0 + (double)N.nl.K1 * kLn2d * e2);
-                N.k1e = dc > 0.0 ? (float)((double)N.nl.K1 * e2) : 0.0f;
-                N.invJ0 = J0 > 0.0 ? (float)(1.0 / J0) : 0.0f;
-                N.d0abs = (float)(fabs((double)N.nl.A0) +
-                                  fabs(lg0) * (fabs((double)N.nl.B1) + (double)N.nl.B2 * fabs(lg0)));
-            }
+        {
+            constexpr int kW = sizeof(NodeLine) / 4, kS = sizeof(ScanConsts) / 4;
+            static_assert(kW + kS <= 32, "one word per lane");
+            const NodeCands &nc = P.cands[qi];
+            if (lane < kW) reinterpret_cast<int *>(&N.nl)[lane] = reinterpret_cast<const int *>(&nc.nl)[lane];
+            else if (lane < kW + kS)
+                reinterpret_cast<int *>(static_cast<ScanConsts *>(&N))[lane - kW] =
+                    reinterpret_cast<const int *>(&nc.sc)[lane - kW];
         }
         __syncwarp();
         const LineSpec ln = scaled_line(pd.line, N.e);
@@ -399,6 +548,7 @@ __global__ void __launch_bounds__(32 * kLaneWarps, CVX_LANE_MIN_BLOCKS)
             return win ? lane_window_dir(pd, cen, d0 + blk + j) : d0 + blk + j;
         };
         const f32x2 H = pk2(ln.h32, ln.h32);
+        const BBGeom G = bb_geom(ln.h32, m0);
         NHPair node = nh_pair_node(N.nl);
         node.J0 = pk2(N.nl.J0, N.nl.J0);
         // the item's best directions so far: lane i < kItemTop holds entry i
@@ -416,6 +566,7 @@ __global__ void __launch_bounds__(32 * kLaneWarps, CVX_LANE_MIN_BLOCKS)
             const int Pn = (nb + 31) >> 5;
             float umin = INFINITY, s_prev = 0.0f;
             bool warm = false;
+            int xsL = -1, xsR = 1;  // the previous line's minimisers
             // near region of the no-split certificate: |x| up to Xn samples
             // (even, at most 0.04 in t and 32 samples)
             const int np = m0 >> 1;
@@ -429,7 +580,8 @@ __global__ void __launch_bounds__(32 * kLaneWarps, CVX_LANE_MIN_BLOCKS)
                 const NHPair c = line_pair(node, dl);
                 const bool tangent = !warm;
                 const float s0 = warm ? s_prev : sa * __fmaf_rn(cb, dl.cJ, dl.A1);
-                const SideMin sm = line_pass(c, H, -s0, m0, 0, 1, kf, kn);
+                const SideMin sm = bb_pass(N, G, dl.A1, dl.A2, dl.cJ, -s0, bb_base(kap, C, s0, m0),
+                                           np, -1, 0, xsL, xsR);
                 const Bounds b = pass_bounds(c, H, s0, m0, sm);
                 LaneState t;
                 t.q_lo = b.q_lo;
@@ -439,9 +591,10 @@ __global__ void __launch_bounds__(32 * kLaneWarps, CVX_LANE_MIN_BLOCKS)
                 if (b.q_hi - b.q_lo <= 0.25f * eps32_at(b.q_lo, kap, C)) t.ab |= kConv;
                 if (tangent) t.ab |= kTan;
                 st[j] = t;
-                efl[j] = fminf(sm.eLf, sm.eRf);
                 umin = fminf(umin, b.q_hi);
                 warm = b.a >= 0 && b.q_hi < w0 - epsc;
+                xsL = b.a >= 0 ? b.a - m0 : -1;
+                xsR = b.a >= 0 ? b.b - m0 : 1;
                 s_prev = b.s;
                 n_valid += valid_samples(dl, ln, CVX_ENERGY_NH_DAMAGE);
             }
@@ -484,7 +637,11 @@ __global__ void __launch_bounds__(32 * kLaneWarps, CVX_LANE_MIN_BLOCKS)
                             make_dir_line<CVX_ENERGY_NH_DAMAGE>(N.nl, P.dir32[doff + gdir(blk, j)]);
                         const NHPair c = line_pair(node, dl);
                         LaneState t = st[j];
-                        const Bounds b = pass_bounds(c, H, t.s, m0, line_pass(c, H, -t.s, m0, 0, 1));
+                        const int a0 = t.ab & 0xfff, b0 = (t.ab >> 12) & 0xfff;
+                        const SideMin sm = bb_pass(N, G, dl.A1, dl.A2, dl.cJ, -t.s,
+                                                   bb_base(kap, C, t.s, m0), np, -1, 0, a0 - m0,
+                                                   b0 - m0);
+                        const Bounds b = pass_bounds(c, H, t.s, m0, sm);
                         const int ab = enc_ab(b.a, b.b);
                         const bool same = ab == (t.ab & ~kTan);
                         t.q_lo = fmaxf(t.q_lo, b.q_lo);
@@ -559,7 +716,13 @@ __global__ void __launch_bounds__(32 * kLaneWarps, CVX_LANE_MIN_BLOCKS)
                     const float4 d32 = P.dir32[doff + gdir(blk, j)];
                     const DirLine dl = make_dir_line<CVX_ENERGY_NH_DAMAGE>(N.nl, d32);
                     const float s0 = sa * __fmaf_rn(cb, dl.cJ, dl.A1);
-                    if (flat_certificate(N, dl, d32, ln.h32, m0, 2 * kf - m0, 2 * kn, s0, efl[j], kap))
+                    // the smallest v - s0 x over the far samples (left pairs k < kf,
+                    // right pairs k >= kn, and the last sample if m0 is odd)
+                    const int xlL = 2 * kf - 1 - m0;
+                    const SideMin sf = bb_pass(N, G, dl.A1, dl.A2, dl.cJ, -s0, bb_base(kap, C, s0, m0),
+                                               kf, xlL, kn, xlL, min(2 * kn + 1, m0));
+                    const float ef = fminf(sf.eL, sf.eR);
+                    if (flat_certificate(N, dl, d32, ln.h32, m0, 2 * kf - m0, 2 * kn, s0, ef, kap))
                         st[j].ab |= kCert;
                 }
                 __syncwarp();
