@@ -243,6 +243,9 @@ int scan_max_blocks_per_sm(int energy, int warps, int stride);
 bool lane_scan_enabled(int energy);
 int lane_scan_blocks_per_sm();
 cudaError_t launch_scan_lanes(const Pipe &p, int level, int sms, cudaStream_t s);
+// FP64 refinement after it (cvx_refine_lanes.cu), phase 0 or 1.
+cudaError_t launch_refine_lanes(const Pipe &p, int level, int phase, int sms, long long max_work,
+                                cudaStream_t s);
 // Directions per work item of the lane-per-line scan: whole nodes (a warp
 // takes them in blocks of kLaneItemMax lines), smaller items (multiples of
 // 32) when the nodes are too few for every warp of the grid to get two items.

@@ -1,0 +1,149 @@
+// cvx_intervals.cuh -- which parts of a rank-one line of the damage energy can
+// hold a sample at or below a given level of v - s x, from the samples at the
+// ends of its intervals and an upper bound of v'' (used by the lane-per-line
+// scan and by the FP64 refinement's certificate).
+#pragma once
+
+#include "cvx_internal.h"
+
+namespace cvx {
+
+// A side of a line (its samples left or right of the centre) is cut into
+// intervals of 2 PP samples.  Only their end points are sampled first.
+// Inside an interval of length delta in t the function g = v - s x lies at
+// most M delta^2 / 8 below the lower of its end values, M any upper bound of
+// v'' there, so an interval whose bound exceeds a level holds no sample at or
+// below it.
+//
+// Bound of v'': v = phi(d(t)) with phi' = 1 + K2' 2^{-max(d, 0)} (C ln 2 = K2')
+// positive and nonincreasing, phi'' <= 0, so v'' <= phi'(min d) max(d'', 0);
+//   d'' = 2 A2 + (cJ / J)^2 (c0 - c1 log2 J),
+//   c0 = 2 B2 / ln2^2 - B1 / ln2, c1 = 2 B2 / ln2,
+// whose positive part falls with J, so its maximum over eight intervals is
+// taken at their smallest J, and d lies at most eta = max(d'') delta^2 / 8
+// below its end values, which raises 2^{-d} by at most 2^eta <= 1 + eta
+// (eta <= 1).  Intervals that reach J <= 0 are always kept; eight intervals
+// with J <= 0 throughout hold no finite sample.
+// The rounding of the samples (kEps32 max(kappa', |v| + C) bounds it, with
+// |v| <= |g| + |s| m0) is covered four times over: by `base` (iv_base) and by
+// the term in |e| of the comparison.
+struct IvGeom {
+    float h, q8;  // sample spacing, delta^2 / 8
+    float rPP;    // 1 / PP
+    int m0, PP;   // samples per side, pairs per interval
+};
+
+// Pairs per interval on a side of m0 samples: about sqrt(m0) samples (an end
+// costs about two samples, one to two intervals per side are sampled), at
+// most 32 intervals per side (one mask bit each).  0.4 and 0.7 in place of
+// 0.5 measured 4 % slower at L = 201, 7 % slower and 2 % faster at L = 1025.
+constexpr float kIvScale = 0.5f;
+
+__device__ __forceinline__ IvGeom iv_geom(float h, int m0) {
+    IvGeom g;
+    g.h = h;
+    g.m0 = m0;
+    g.PP = max(max(((m0 >> 1) + 31) >> 5, (int)(kIvScale * sqrtf((float)m0) + 0.5f)), 1);
+    g.rPP = 1.0f / (float)g.PP;
+    g.q8 = 0.5f * (float)(g.PP * g.PP) * h * h;
+    return g;
+}
+
+// Intervals of a region of npr pairs: ceil(npr / PP).
+__device__ __forceinline__ int iv_count(const IvGeom &g, int npr) {
+    return (int)(((float)(npr + g.PP - 1) + 0.5f) * g.rPP);
+}
+
+__device__ __forceinline__ float iv_base(float kap, float C, float s, int m0) {
+    return 4.0f * kEps32 * (kap + C + fabsf(s) * (float)m0);
+}
+
+// The constants of a line: sample_nh2's, and those of d''.
+struct IvLine {
+    NHPair c;
+    float A2, cJ, J0, K2, c0, c1;
+};
+
+__device__ __forceinline__ IvLine iv_line(const NodeLine &nl, float A1, float A2, float cJ) {
+    IvLine l;
+    l.c = nh_pair_node(nl);
+    l.c.A1 = pk2(A1, A1);
+    l.c.A2 = pk2(A2, A2);
+    l.c.CJ = pk2(cJ, cJ);
+    l.J0 = nl.J0;
+    l.c.J0 = pk2(l.J0, l.J0);
+    l.A2 = A2;
+    l.cJ = cJ;
+    l.K2 = nl.K2;
+    l.c1 = 2.0f * nl.B2 * (1.0f / kLn2);
+    l.c0 = (l.c1 - nl.B1) * (1.0f / kLn2);
+    return l;
+}
+
+// g = v - s x at two samples, and 2^{-max(d, 0)} there.
+__device__ __forceinline__ void iv_eval(const NHPair &c, f32x2 H, f32x2 NS, f32x2 X, float &g0,
+                                        float &g1, float &E0, float &E1) {
+    const f32x2 T = mul2(X, H);
+    const f32x2 P = fma2(T, fma2(T, c.A2, c.A1), c.A0);
+    float j0, j1, d0, d1;
+    upk2(fma2(T, c.CJ, c.J0), j0, j1);
+    const f32x2 LG = pk2(lg2_approx(j0), lg2_approx(j1));
+    const f32x2 D = fma2(LG, fma2(LG, c.B2, c.B1), P);
+    upk2(D, d0, d1);
+    E0 = ex2_approx(-fmaxf(d0, 0.0f));
+    E1 = ex2_approx(-fmaxf(d1, 0.0f));
+    const f32x2 W = fma2(c.K2, pk2(fminf(d0, 0.0f), fminf(d1, 0.0f)), D);
+    upk2(fma2(NS, X, fma2(c.NK1, pk2(E0, E1), W)), g0, g1);
+}
+
+// Intervals (a mask) of the region from sample xb (value ga, Ea) to fl with
+// NI intervals that can hold a sample with v - s x <= e.  kLower: e follows
+// the smallest end value seen (the search for the minimum), else it is fixed.
+template <bool kLower>
+__device__ __forceinline__ unsigned iv_sweep(const IvLine &l, const IvGeom &G, f32x2 H, f32x2 NS,
+                                             float base, int xb, float fl, int NI, float ga,
+                                             float Ea, float &e) {
+    const float h = G.h, fS = 2.0f * (float)G.PP;
+    unsigned mask = 0;
+    float xa = (float)xb;  // the left end of the next interval
+#pragma unroll 1
+    for (int i0 = 0; i0 < NI; i0 += 8) {
+        // the largest d'' over the eight intervals
+        const float xe = fminf(__fmaf_rn(8.0f, fS, xa), fl);
+        const float Ja = __fmaf_rn(xa * h, l.cJ, l.J0), Je = __fmaf_rn(xe * h, l.cJ, l.J0);
+        const float Jm = fminf(Ja, Je);
+        if (!(fmaxf(Ja, Je) > 0.0f)) {
+            ga = INFINITY;
+            xa = xe;
+            continue;
+        }
+        const float r = __fdividef(l.cJ, Jm);
+        const float dd =
+            __fmaf_rn(r * r, fmaxf(__fmaf_rn(-l.c1, lg2_approx(Jm), l.c0), 0.0f), 2.0f * l.A2);
+        float eta = dd * G.q8;
+        if (!(Jm > 0.0f) || !(eta < 1e30f)) eta = INFINITY;
+        const float up = eta <= 1.0f ? 1.0f + eta : INFINITY;
+        const float etc = 1.0001f * eta;
+        unsigned bit = 1u << i0;
+        const int ie = min(i0 + 8, NI);
+#pragma unroll 1
+        for (int i = i0; i < ie; i += 2, bit <<= 2) {
+            const float x0 = fminf(xa + fS, fl), x1 = fminf(__fmaf_rn(2.0f, fS, xa), fl);
+            float p0, p1, E0, E1;
+            iv_eval(l.c, H, NS, pk2(x0, x1), p0, p1, E0, E1);
+            if (kLower) e = fmin3(e, p0, p1);
+            // (Ea * up is NaN only where both are 0 and inf: fminf takes 1)
+            const float En = fminf(fmaxf(Ea, fmaxf(E0, E1)) * up, 1.0f);
+            const float thr = __fmaf_rn(etc, __fmaf_rn(l.K2, En, 1.0f), base) +
+                              __fmaf_rn(4.0f * kEps32, fabsf(e), e);
+            if (!(fminf(ga, p0) > thr)) mask |= bit;
+            if (!(fminf(p0, p1) > thr)) mask |= bit << 1;
+            ga = p1;
+            Ea = E1;
+            xa = x1;
+        }
+    }
+    return mask & (NI >= 32 ? 0xffffffffu : (1u << NI) - 1u);
+}
+
+}  // namespace cvx

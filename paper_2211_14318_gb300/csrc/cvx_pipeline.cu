@@ -21,6 +21,7 @@
 #include <limits.h>
 
 #include "cvx_line.cuh"
+#include "cvx_refine.cuh"
 
 namespace cvx {
 
@@ -603,36 +604,7 @@ __global__ void k_select(const Pipe P, int level) {
 // FP64 bridge of the left and right sets of one line held in shared memory:
 // supporting-slope iteration with full passes; ties go to the outermost sample
 // (Algorithm 1 keeps the outermost of collinear points).
-//
-// The minima of v - s x are compared as order-preserving integer keys of the
-// doubles, so that the comparisons run on the integer pipe: the FP64 pipe
-// (2 lanes per SM per clock) is what bounds the refinement, and a key compares
-// exactly as its double does.
 // -------------------------------------------------------------------------
-
-// Integer key of a double that is not NaN: x < y iff dkey(x) < dkey(y), and
-// x == y iff the keys are equal (-0 and +0 share the key 0).
-__device__ __forceinline__ long long dkey(double x) {
-    const long long b = __double_as_longlong(x);
-    return b >= 0 ? b : -(b & 0x7fffffffffffffffLL);
-}
-
-constexpr long long kKeyInf = 0x7ff0000000000000LL;  // dkey(+inf)
-
-// Warp-wide minimum of (key, sample index); ties to the lower index if
-// prefer_low, else to the higher.
-__device__ __forceinline__ void warp_min_key(long long &v, int &k, bool prefer_low) {
-#pragma unroll
-    for (int o = 16; o; o >>= 1) {
-        const long long v2 = __shfl_xor_sync(kFull, v, o);
-        const int k2 = __shfl_xor_sync(kFull, k, o);
-        if (v2 < v || (v2 == v && (prefer_low ? k2 < k : k2 > k))) {
-            v = v2;
-            k = k2;
-        }
-    }
-}
-
 __device__ void bridge64(const double *sw, int L, int m0, int lane, int &a, int &b) {
     double s = 0.0;
     a = b = -1;
@@ -692,188 +664,12 @@ __device__ bool window_bridge64(double vA, double vB, int kA, int kB, int m0, in
     return false;
 }
 
-// Half-warp minimum with the sample index (lanes 0-15 and 16-31 reduce
-// separately); ties to the lower index if prefer_low, else to the higher.
-__device__ __forceinline__ void half_min_key(long long &v, int &k, bool prefer_low) {
-#pragma unroll
-    for (int o = 8; o; o >>= 1) {
-        const long long v2 = __shfl_xor_sync(kFull, v, o);
-        const int k2 = __shfl_xor_sync(kFull, k, o);
-        if (v2 < v || (v2 == v && (prefer_low ? k2 < k : k2 > k))) {
-            v = v2;
-            k = k2;
-        }
-    }
-}
-
-// FP64 bridge from the line scan's FP32 pair (a, b) (damage energy): the
-// supporting-slope iteration over FP64 samples in two windows around a and
-// b (16 samples each, one per lane, for L <= 513; 32 each, two per lane,
-// above), then a certificate over the whole line that every sample outside
-// the windows lies strictly above the FP64 chord.  Each such sample is first
-// tested on its FP32 value, computed on the fly: its FP32 sample less the
-// FP32 error bound kEps32 max(kappa', |v| + C) and the rounding bound of the
-// chord evaluated in FP32 sample units lies above the chord.  Where that test
-// is inconclusive (near the tangent points, or det near 0) the sample is
-// taken in FP64 and compared with the chord exactly.  An FP64 sample on or
-// below the chord moves the pair to the lowest such sample of its side (at
-// the chord's slope) and the windows are taken around the new pair, at most
-// 4 times.  Returns false if that does not settle (the caller resamples the
-// whole line in FP64); n64 counts the FP64 spot samples.
-// Lines up to this many samples take FP64 windows of 16 samples per side in
-// the refinement (one sample per lane), longer lines 32 per side (two per
-// lane).  A window that misses a tangent point only costs a further round:
-// the certificate over the whole line moves it.
-#ifndef CVX_REFINE_NARROW_MAX_L
-#define CVX_REFINE_NARROW_MAX_L 513
-#endif
-
-__device__ bool refine_hinted(const double F[4], const double R[4], double beta, const NodeCands &nc,
-                              const ProbDesc &pd, const LineSpec &ln, float4 d32, int hab, int lane,
-                              int &a, int &b, double &wa, double &wb, unsigned &n64,
-                              int *spot_q) {
-    const int m0 = ln.m0, L = ln.L;
-    const double ek = nc.ek;
-    a = hab & 0xffff;
-    b = hab >> 16;
-    if (!(a >= 0 && a < m0 && b > m0 && b < L)) return false;
-    const bool narrow = L <= CVX_REFINE_NARROW_MAX_L;
-    const int W = narrow ? 16 : 32;
-    const double kap = pd.kappa, C = nc.shift;
-    const float kapf = pd.kappa_f, Cf = (float)C;
-    const DirLine dl = make_dir_line<CVX_ENERGY_NH_DAMAGE>(nc.nl, d32);
-    for (int round = 0; round < 4; ++round) {
-        const int loA = max(0, min(a - W / 2, m0 - W));
-        const int loB = max(m0 + 1, min(b - (W / 2 - 1), L - W));
-        // window samples: narrow, lane l < 16 holds left loA + l and lane
-        // l >= 16 right loB + l - 16; wide, every lane holds left loA + l and
-        // right loB + l
-        const int kA = narrow ? loA + (lane & 15) : loA + lane;
-        const int kB = narrow ? loB + (lane & 15) : loB + lane;
-        const bool hasA = narrow ? lane < 16 : true, hasB = narrow ? lane >= 16 : true;
-        double vA = INFINITY, vB = INFINITY;
-        if (hasA && kA < m0) {
-            const double v = sample_w64_ek(F, R, kA, m0, ln.h64, beta, ek, pd.mat);
-            vA = v == v ? v : INFINITY;
-        }
-        if (hasB && kB < L) {
-            const double v = sample_w64_ek(F, R, kB, m0, ln.h64, beta, ek, pd.mat);
-            vB = v == v ? v : INFINITY;
-        }
-        auto valA = [&](int k) { return __shfl_sync(kFull, vA, k - loA); };
-        auto valB = [&](int k) { return __shfl_sync(kFull, vB, narrow ? 16 + k - loB : k - loB); };
-        wa = valA(a);
-        wb = valB(b);
-        if (!(wa < INFINITY && wb < INFINITY)) return false;
-        bool settled = false;
-        // per round: which window samples count, and their abscissae
-        const bool left = lane < 16;
-        const double vN = left ? vA : vB;
-        const int kN = left ? kA : kB;
-        const bool okA = vA < INFINITY, okB = vB < INFINITY, okN = vN < INFINITY;
-        const double xA = (double)(kA - m0), xB = (double)(kB - m0), xN = (double)(kN - m0);
-        for (int it = 0; it < 64 && !settled; ++it) {
-            const double s = (wb - wa) / (double)(b - a);
-            int na, nb;
-            if (narrow) {
-                long long e = okN ? dkey(vN - s * xN) : kKeyInf;
-                int kk = okN ? kN : (left ? INT_MAX : -1);
-                half_min_key(e, kk, left);
-                na = __shfl_sync(kFull, kk, 0);
-                nb = __shfl_sync(kFull, kk, 16);
-            } else {
-                long long eA = okA ? dkey(vA - s * xA) : kKeyInf;
-                long long eB = okB ? dkey(vB - s * xB) : kKeyInf;
-                int ka = okA ? kA : INT_MAX, kb = okB ? kB : -1;
-                warp_min_key(eA, ka, true);
-                warp_min_key(eB, kb, false);
-                na = ka;
-                nb = kb;
-            }
-            if (na == INT_MAX || nb < 0) return false;
-            settled = na == a && nb == b;
-            a = na;
-            b = nb;
-            wa = valA(a);
-            wb = valB(b);
-        }
-        if (!settled) return false;
-        // certificate over the samples outside the windows and the centre
-        const double s = (wb - wa) / (double)(b - a);
-        const float la = (float)(kap * wa - C), ls = (float)(kap * s);
-        const int hiA = min(loA + W, m0), hiB = min(loB + W, L);
-        long long eL = kKeyInf, eR = kKeyInf;  // lowest v - s x of FP64 samples on or below
-        int kL = INT_MAX, kR = -1;              // the chord, per side (keys)
-        unsigned c64 = 0;
-        // FP64 spot sample k, compared with the chord exactly
-        auto spot = [&](int k) {
-            ++c64;
-            const double v = sample_w64_ek(F, R, k, m0, ln.h64, beta, ek, pd.mat);
-            if (!(v == v)) return;  // det <= 0: excluded
-            const double line = wa + s * (double)(k - a);
-            if (v > line + 1e-14 * fabs(line)) return;
-            const long long e = dkey(v - s * (double)(k - m0));
-            if (k < m0) {
-                if (e < eL || (e == eL && k < kL)) {
-                    eL = e;
-                    kL = k;
-                }
-            } else if (e < eR || (e == eR && k > kR)) {
-                eR = e;
-                kR = k;
-            }
-        };
-        // samples whose FP32 test is inconclusive queue up in the warp's
-        // shared-memory buffer and are taken in FP64 32 at a time, one per
-        // lane, so that a few scattered ones do not each cost the whole warp
-        // an FP64 sample; the minima do not depend on the order
-        int nq = 0;
-        for (int base = 0; base < L; base += 32) {
-            const int k = base + lane;
-            bool need = false;
-            if (k < L && k != m0 && !(k >= loA && k < hiA) && !(k >= loB && k < hiB)) {
-                const float v32 =
-                    sample_w<CVX_ENERGY_NH_DAMAGE>(nc.nl, dl, __fmul_rn((float)(k - m0), ln.h32));
-                need = true;
-                if (v32 < INFINITY && v32 > -INFINITY) {
-                    const float x = (float)(k - a);
-                    const float Lv = __fmaf_rn(ls, x, la);
-                    const float err = 2.0f * kU32 * (fabsf(la) + fabsf(ls * x) + fabsf(Lv)) +
-                                      kEps32 * fmaxf(kapf, fabsf(v32) + Cf) + 1e-30f;
-                    need = !(__fsub_rn(v32, Lv) > 1.001f * err);  // else above the chord
-                }
-            }
-            const unsigned bal = __ballot_sync(kFull, need);
-            if (need) spot_q[nq + __popc(bal & ((1u << lane) - 1u))] = k;
-            nq += __popc(bal);
-            __syncwarp();
-            if (nq >= 32) {
-                spot(spot_q[lane]);
-                const int rest = nq - 32;
-                __syncwarp();
-                if (lane < rest) spot_q[lane] = spot_q[32 + lane];
-                nq = rest;
-                __syncwarp();
-            }
-        }
-        if (lane < nq) spot(spot_q[lane]);
-        __syncwarp();
-        n64 += c64;
-        warp_min_key(eL, kL, true);
-        warp_min_key(eR, kR, false);
-        if (kL == INT_MAX && kR < 0) return true;  // certified
-        if (kL != INT_MAX) a = kL;
-        if (kR >= 0) b = kR;
-    }
-    return false;
-}
-
 // The FP64 refinement of candidate c of queued node qi (one warp): writes
 // P.refined[qi][c].
 template <int EK>
 __device__ __forceinline__ void refine_one(const Pipe &P, int level, int qi, int c, int lane,
                                            double *sw, HullCounters &hc,
-                                           unsigned long long &n_full, unsigned &n_spot) {
+                                           unsigned long long &n_full) {
     float *sw32 = reinterpret_cast<float *>(sw);
     const int32_t *qp = P.qp[level], *qh = P.qh[level];
     const int p = qp[qi], hi = qh[qi];
@@ -887,43 +683,6 @@ __device__ __forceinline__ void refine_one(const Pipe &P, int level, int qi, int
     const double R[4] = {__dmul_rn(d[0], d[2]), __dmul_rn(d[0], d[3]), __dmul_rn(d[1], d[2]),
                          __dmul_rn(d[1], d[3])};
     const double beta = pd.beta[p - pd.point_off];
-    const int hab = P.cands[qi].ab[c];
-    if (EK == CVX_ENERGY_NH_DAMAGE && hab >= 0) {
-        // the scan's FP32 pair as the start, windows in FP64, FP32 certificate
-        int a, b;
-        double wa = 0.0, wb = 0.0;
-        bool ok = refine_hinted(F, R, beta, P.cands[qi], pd, ln, P.dir32[pd.dir_off + dir], hab,
-                                lane, a, b, wa, wb, n_spot, reinterpret_cast<int *>(sw));
-        if (!ok) {
-            ++n_full;
-            const double ek = P.cands[qi].ek;
-            for (int k = lane; k < ln.L; k += 32)
-                sw[k] = sample_w64_ek(F, R, k, m0, ln.h64, beta, ek, pd.mat);
-            __syncwarp();
-            bridge64(sw, ln.L, m0, lane, a, b);
-            if (a >= 0) {
-                wa = sw[a];
-                wb = sw[b];
-            }
-        }
-        if (lane == 0) {
-            RefineOut o;
-            o.a = a;
-            o.b = b;
-            o.pad = 0;
-            if (a >= 0) {
-                const double xa = (double)(a - m0), xb = (double)(b - m0);
-                o.q = (xb * wa - xa * wb) / (xb - xa);
-                o.ok = 1;
-            } else {
-                o.q = INFINITY;
-                o.ok = 0;
-            }
-            P.refined[(long long)qi * kNodeCand + c] = o;
-        }
-        __syncwarp();
-        return;
-    }
     // FP32 line and its approximate bridge
     const NodeLine nl = P.cands[qi].nl;
     const DirLine dl = make_dir_line<EK>(nl, P.dir32[pd.dir_off + dir]);
@@ -1008,7 +767,8 @@ __device__ __forceinline__ void refine_one(const Pipe &P, int level, int qi, int
     __syncwarp();
 }
 
-// k_refine: one warp per screened (node, direction).  The FP64 bridge of the
+// k_refine: one warp per screened (node, direction), after the warp-per-line
+// scan (k_refine_lanes serves the lane-per-line scan).  The FP64 bridge of the
 // left and right sample sets is searched in two 32-sample FP64 windows around
 // the FP32 bridge and certified against the whole line with the FP32 samples:
 // every sample m outside the windows must satisfy
@@ -1035,7 +795,6 @@ __global__ void __launch_bounds__(128) k_refine(const Pipe P, int level, int pha
     __syncwarp();
     HullCounters hc{s_hc[warp]};
     unsigned long long n_full = 0, n_ref = 0;
-    unsigned n_spot = 0;  // FP64 spot samples of the certificates (per lane)
     const int nwarps = gridDim.x * (blockDim.x >> 5);
     const int gw = blockIdx.x * (blockDim.x >> 5) + warp;
     // the warp's next (node, candidate): phase 0 takes 32 nodes per step and
@@ -1071,13 +830,11 @@ __global__ void __launch_bounds__(128) k_refine(const Pipe P, int level, int pha
             }
             if (qi < 0) break;
         }
-        refine_one<EK>(P, level, qi, c, lane, sw, hc, n_full, n_spot);
+        refine_one<EK>(P, level, qi, c, lane, sw, hc, n_full);
         ++n_ref;
     }
     if (lane == 0) add_counter(P.counters, C_REFFULL, n_full);
     if (lane == 0) add_counter(P.counters, C_REFINED, n_ref);
-    n_spot = __reduce_add_sync(kFull, n_spot);
-    if (lane == 0) add_counter(P.counters, C_FP64, n_spot);
 }
 
 // Offset of grid index i from the centre c on a periodic axis of N cells, in
@@ -1678,18 +1435,24 @@ cudaError_t pipe_level(const Pipe &p, int l, int warps, int grid, cudaStream_t s
     if (ev && (e = cudaEventRecord(ev[1], s)) != cudaSuccess) return e;
     k_select<<<nb, 128, 0, s>>>(p, l);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    const long long want = (max_nodes * kNodeCand + 3) / 4;
-    const unsigned rg = (unsigned)(want < (long long)sms * 8 ? want : (long long)sms * 8);
-    const size_t rsm = (size_t)4 * p.stride64 * sizeof(double);
-    auto kr = p.energy == CVX_ENERGY_NH_DAMAGE ? k_refine<CVX_ENERGY_NH_DAMAGE>
-                                               : k_refine<CVX_ENERGY_DOUBLE_WELL>;
-    if ((e = cudaFuncSetAttribute(kr, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)rsm)) !=
-        cudaSuccess)
-        return e;
-    kr<<<rg, 128, rsm, s>>>(p, l, 0);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    kr<<<rg, 128, rsm, s>>>(p, l, 1);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    if (p.lanes) {
+        for (int phase = 0; phase < 2; ++phase)
+            if ((e = launch_refine_lanes(p, l, phase, sms, max_nodes * kNodeCand, s)) != cudaSuccess)
+                return e;
+    } else {
+        const long long want = (max_nodes * kNodeCand + 3) / 4;
+        const unsigned rg = (unsigned)(want < (long long)sms * 8 ? want : (long long)sms * 8);
+        const size_t rsm = (size_t)4 * p.stride64 * sizeof(double);
+        auto kr = p.energy == CVX_ENERGY_NH_DAMAGE ? k_refine<CVX_ENERGY_NH_DAMAGE>
+                                                   : k_refine<CVX_ENERGY_DOUBLE_WELL>;
+        if ((e = cudaFuncSetAttribute(kr, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)rsm)) !=
+            cudaSuccess)
+            return e;
+        kr<<<rg, 128, rsm, s>>>(p, l, 0);
+        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+        kr<<<rg, 128, rsm, s>>>(p, l, 1);
+        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    }
     k_commit<<<nb, 128, 0, s>>>(p, l);
     return cudaGetLastError();
 }

@@ -6,7 +6,7 @@
 // A warp takes a work item (a node and up to 256 of its directions) and each
 // lane takes its own line, two samples per paired FP32 instruction, without
 // storing it, and without taking the samples that a bound of v'' shows to lie
-// above the minimum looked for (bb_pass).  For the hull at t = 0 of the left set {x < 0} and the right set
+// above the minimum looked for (lane_pass).  For the hull at t = 0 of the left set {x < 0} and the right set
 // {x > 0} of the samples (x = m - m0) the pass at a slope s yields
 //   e_L = min over the left of (v - s x),  e_R = min over the right,
 // and their minimisers a < 0 < b.  For any s, min(e_L, e_R) is a lower bound
@@ -28,6 +28,7 @@
 #include <stdlib.h>
 #include <string.h>
 
+#include "cvx_intervals.cuh"
 #include "cvx_line.cuh"
 
 namespace cvx {
@@ -115,98 +116,33 @@ __device__ __forceinline__ SideMin line_pass(const NHPair &c, f32x2 H, float ns,
 }
 
 // ---- the lane's own pass over a line: the same minima (bit for bit, lowest
-// pair on equal values) without sampling the whole line.
-//
-// A side is cut into intervals of 2 PP samples.  Only their end points are
-// sampled first.  Inside an interval of length delta in t the function
-// g = v - s x lies at most M delta^2 / 8 below the lower of its end values,
-// M any upper bound of v'' there, so an interval whose bound exceeds the
-// smallest sample seen so far cannot hold the side's minimum and is never
-// sampled.  The others (the interval of the minimum and its neighbours as a
-// rule) are sampled in full.
-//
-// Bound of v'': v = phi(d(t)) with phi' = 1 + K2' 2^{-max(d, 0)} (C ln 2 = K2')
-// positive and nonincreasing, phi'' <= 0, so v'' <= phi'(min d) max(d'', 0);
-//   d'' = 2 A2 + (cJ / J)^2 (c0 - c1 log2 J),
-//   c0 = 2 B2 / ln2^2 - B1 / ln2, c1 = 2 B2 / ln2,
-// whose positive part falls with J, so its maximum over eight intervals is
-// taken at their smallest J, and d lies at most eta = max(d'') delta^2 / 8
-// below its end values, which raises 2^{-d} by at most 2^eta <= 1 + eta
-// (eta <= 1).  Intervals that reach J <= 0 are always sampled; eight
-// intervals with J <= 0 throughout hold no finite sample.
-// The rounding of the samples (kEps32 max(kappa', |v| + C) bounds it, with
-// |v| <= |g| + |s| m0) is covered four times over: by `base` and by the term
-// in |e| of the comparison.
+// pair on equal values) without sampling the whole line.  The ends of the
+// intervals (cvx_intervals.cuh) are sampled first; an interval whose bound
+// exceeds the smallest sample seen so far cannot hold the side's minimum and
+// is never sampled, the others (the interval of the minimum and its
+// neighbours as a rule) are sampled in full.
 // What bounds it: instruction issue (79 % of the slots at L = 201).  Taking
 // every sample instead: 3,001 load-path points, 128^2 directions, L = 2049,
 // depth 3: 326.9 ms of line scan, 70.9 ms with the intervals; 16,384 mesh
 // points, 64^2, L = 1025: 227.9 -> 70 ms; 1,048,576 points, 16^2, L = 201:
 // 86.9 -> 51 ms.  2.5 to 4.0 intervals are sampled per line, both sides
 // together.
-struct BBGeom {
-    float h, q8;  // sample spacing, delta^2 / 8
-    float rPP;    // 1 / PP
-    int m0, PP;   // samples per side, pairs per interval
-};
-
-// Pairs per interval on a side of m0 samples: about sqrt(m0) samples (an end
-// costs about two samples, one to two intervals per side are sampled), at
-// most 32 intervals per side (one mask bit each).  0.4 and 0.7 in place of
-// 0.5 measured 4 % slower at L = 201, 7 % slower and 2 % faster at L = 1025.
-constexpr float kBBScale = 0.5f;
-__device__ __forceinline__ BBGeom bb_geom(float h, int m0) {
-    BBGeom g;
-    g.h = h;
-    g.m0 = m0;
-    g.PP = max(max(((m0 >> 1) + 31) >> 5, (int)(kBBScale * sqrtf((float)m0) + 0.5f)), 1);
-    g.rPP = 1.0f / (float)g.PP;
-    g.q8 = 0.5f * (float)(g.PP * g.PP) * h * h;
-    return g;
-}
-
-__device__ __forceinline__ float bb_base(float kap, float C, float s, int m0) {
-    return 4.0f * kEps32 * (kap + C + fabsf(s) * (float)m0);
-}
-
-// g = v - s x at two samples, and 2^{-max(d, 0)} there.
-__device__ __forceinline__ void bb_eval(const NHPair &c, f32x2 H, f32x2 NS, f32x2 X, float &g0,
-                                        float &g1, float &E0, float &E1) {
-    const f32x2 T = mul2(X, H);
-    const f32x2 P = fma2(T, fma2(T, c.A2, c.A1), c.A0);
-    float j0, j1, d0, d1;
-    upk2(fma2(T, c.CJ, c.J0), j0, j1);
-    const f32x2 LG = pk2(lg2_approx(j0), lg2_approx(j1));
-    const f32x2 D = fma2(LG, fma2(LG, c.B2, c.B1), P);
-    upk2(D, d0, d1);
-    E0 = ex2_approx(-fmaxf(d0, 0.0f));
-    E1 = ex2_approx(-fmaxf(d1, 0.0f));
-    const f32x2 W = fma2(c.K2, pk2(fminf(d0, 0.0f), fminf(d1, 0.0f)), D);
-    upk2(fma2(NS, X, fma2(c.NK1, pk2(E0, E1), W)), g0, g1);
-}
-
-// The lane's pass at slope s = -ns over the left samples -m0 .. xlL (the
-// pairs k < kl, and x = -1 if that is a pair of its own) and the right pairs
+//
+// The pass at slope s = -ns over the left samples -m0 .. xlL (the pairs
+// k < kl, and x = -1 if that is a pair of its own) and the right pairs
 // k >= kr with the last sample m0 (kl = m0 / 2, xlL = -1, kr = 0: the whole
 // line).  xsL, xsR: samples of the two regions taken first (a neighbouring
 // line's minimisers).  Not inlined: three call sites share one copy, which
 // keeps the kernel in the instruction cache (inlined copies left the warps
 // waiting for instructions 6.4 cycles per issue).
-__device__ __noinline__ SideMin bb_pass(const LaneNode &N, const BBGeom &G, float A1, float A2,
-                                        float cJ, float ns, float base, int kl, int xlL, int kr,
-                                        int xsL, int xsR) {
+__device__ __noinline__ SideMin lane_pass(const LaneNode &N, const IvGeom &G, float A1, float A2,
+                                          float cJ, float ns, float base, int kl, int xlL, int kr,
+                                          int xsL, int xsR) {
     const int m0 = G.m0, PP = G.PP, np = m0 >> 1;
-    const float h = G.h;
-    const f32x2 H = pk2(h, h), NS = pk2(ns, ns);
-    NHPair c = nh_pair_node(N.nl);
-    c.A1 = pk2(A1, A1);
-    c.A2 = pk2(A2, A2);
-    c.CJ = pk2(cJ, cJ);
-    const float J0 = N.nl.J0, K2 = N.nl.K2;
-    c.J0 = pk2(J0, J0);
-    const float c1 = 2.0f * N.nl.B2 * (1.0f / kLn2), c0 = (c1 - N.nl.B1) * (1.0f / kLn2);
-    const float fS = 2.0f * (float)PP;
+    const f32x2 H = pk2(G.h, G.h), NS = pk2(ns, ns);
+    const IvLine l = iv_line(N.nl, A1, A2, cJ);
     float gs0, gs1, eu0, eu1;
-    bb_eval(c, H, NS, pk2((float)xsL, (float)xsR), gs0, gs1, eu0, eu1);
+    iv_eval(l.c, H, NS, pk2((float)xsL, (float)xsR), gs0, gs1, eu0, eu1);
     unsigned mL = 0, mR = 0;
     float lastL = INFINITY, lastR = INFINITY;
 #pragma unroll 1
@@ -215,52 +151,13 @@ __device__ __noinline__ SideMin bb_pass(const LaneNode &N, const BBGeom &G, floa
         const int xl = side ? m0 : xlL;
         const int npr = side ? np - kr : kl;
         if (xl < xb) continue;
-        const float fl = (float)xl;
         float ga, g1, Ea, E1;
-        bb_eval(c, H, NS, pk2((float)xb, fl), ga, g1, Ea, E1);
+        iv_eval(l.c, H, NS, pk2((float)xb, (float)xl), ga, g1, Ea, E1);
         float e = fmin3(side ? gs1 : gs0, ga, g1);
         if (side) lastR = g1;
         else lastL = g1;
-        const int NI = (int)(((float)(npr + PP - 1) + 0.5f) * G.rPP);
-        unsigned mask = 0;
-        float xa = (float)xb;  // the left end of the next interval
-#pragma unroll 1
-        for (int i0 = 0; i0 < NI; i0 += 8) {
-            // the largest d'' over the eight intervals
-            const float xe = fminf(__fmaf_rn(8.0f, fS, xa), fl);
-            const float Ja = __fmaf_rn(xa * h, cJ, J0), Je = __fmaf_rn(xe * h, cJ, J0);
-            const float Jm = fminf(Ja, Je);
-            if (!(fmaxf(Ja, Je) > 0.0f)) {
-                ga = INFINITY;
-                xa = xe;
-                continue;
-            }
-            const float r = __fdividef(cJ, Jm);
-            const float dd = __fmaf_rn(r * r, fmaxf(__fmaf_rn(-c1, lg2_approx(Jm), c0), 0.0f), 2.0f * A2);
-            float eta = dd * G.q8;
-            if (!(Jm > 0.0f) || !(eta < 1e30f)) eta = INFINITY;
-            const float up = eta <= 1.0f ? 1.0f + eta : INFINITY;
-            const float etc = 1.0001f * eta;
-            unsigned bit = 1u << i0;
-            const int ie = min(i0 + 8, NI);
-#pragma unroll 1
-            for (int i = i0; i < ie; i += 2, bit <<= 2) {
-                const float x0 = fminf(xa + fS, fl), x1 = fminf(__fmaf_rn(2.0f, fS, xa), fl);
-                float p0, p1, E0, E1b;
-                bb_eval(c, H, NS, pk2(x0, x1), p0, p1, E0, E1b);
-                e = fmin3(e, p0, p1);
-                // (Ea * up is NaN only where both are 0 and inf: fminf takes 1)
-                const float En = fminf(fmaxf(Ea, fmaxf(E0, E1b)) * up, 1.0f);
-                const float thr = __fmaf_rn(etc, __fmaf_rn(K2, En, 1.0f), base) +
-                                  __fmaf_rn(4.0f * kEps32, fabsf(e), e);
-                if (!(fminf(ga, p0) > thr)) mask |= bit;
-                if (!(fminf(p0, p1) > thr)) mask |= bit << 1;
-                ga = p1;
-                Ea = E1b;
-                xa = x1;
-            }
-        }
-        mask &= NI >= 32 ? 0xffffffffu : (1u << NI) - 1u;
+        const unsigned mask =
+            iv_sweep<true>(l, G, H, NS, base, xb, (float)xl, iv_count(G, npr), ga, Ea, e);
         if (side) mR = mask;
         else mL = mask;
     }
@@ -281,7 +178,7 @@ __device__ __noinline__ SideMin bb_pass(const LaneNode &N, const BBGeom &G, floa
 #pragma unroll 2
         for (int k = ka; k < kb; ++k) {
             float b0, b1;
-            upk2(fma2(NS, X, sample_nh2(c, mul2(X, H))), b0, b1);
+            upk2(fma2(NS, X, sample_nh2(l.c, mul2(X, H))), b0, b1);
             const float en = fmin3(e, b0, b1);
             if (en < e) kk = k;
             e = en;
@@ -548,7 +445,7 @@ __global__ void __launch_bounds__(32 * kLaneWarps, CVX_LANE_MIN_BLOCKS)
             return win ? lane_window_dir(pd, cen, d0 + blk + j) : d0 + blk + j;
         };
         const f32x2 H = pk2(ln.h32, ln.h32);
-        const BBGeom G = bb_geom(ln.h32, m0);
+        const IvGeom G = iv_geom(ln.h32, m0);
         NHPair node = nh_pair_node(N.nl);
         node.J0 = pk2(N.nl.J0, N.nl.J0);
         // the item's best directions so far: lane i < kItemTop holds entry i
@@ -580,7 +477,7 @@ __global__ void __launch_bounds__(32 * kLaneWarps, CVX_LANE_MIN_BLOCKS)
                 const NHPair c = line_pair(node, dl);
                 const bool tangent = !warm;
                 const float s0 = warm ? s_prev : sa * __fmaf_rn(cb, dl.cJ, dl.A1);
-                const SideMin sm = bb_pass(N, G, dl.A1, dl.A2, dl.cJ, -s0, bb_base(kap, C, s0, m0),
+                const SideMin sm = lane_pass(N, G, dl.A1, dl.A2, dl.cJ, -s0, iv_base(kap, C, s0, m0),
                                            np, -1, 0, xsL, xsR);
                 const Bounds b = pass_bounds(c, H, s0, m0, sm);
                 LaneState t;
@@ -638,8 +535,8 @@ __global__ void __launch_bounds__(32 * kLaneWarps, CVX_LANE_MIN_BLOCKS)
                         const NHPair c = line_pair(node, dl);
                         LaneState t = st[j];
                         const int a0 = t.ab & 0xfff, b0 = (t.ab >> 12) & 0xfff;
-                        const SideMin sm = bb_pass(N, G, dl.A1, dl.A2, dl.cJ, -t.s,
-                                                   bb_base(kap, C, t.s, m0), np, -1, 0, a0 - m0,
+                        const SideMin sm = lane_pass(N, G, dl.A1, dl.A2, dl.cJ, -t.s,
+                                                   iv_base(kap, C, t.s, m0), np, -1, 0, a0 - m0,
                                                    b0 - m0);
                         const Bounds b = pass_bounds(c, H, t.s, m0, sm);
                         const int ab = enc_ab(b.a, b.b);
@@ -719,7 +616,7 @@ __global__ void __launch_bounds__(32 * kLaneWarps, CVX_LANE_MIN_BLOCKS)
                     // the smallest v - s0 x over the far samples (left pairs k < kf,
                     // right pairs k >= kn, and the last sample if m0 is odd)
                     const int xlL = 2 * kf - 1 - m0;
-                    const SideMin sf = bb_pass(N, G, dl.A1, dl.A2, dl.cJ, -s0, bb_base(kap, C, s0, m0),
+                    const SideMin sf = lane_pass(N, G, dl.A1, dl.A2, dl.cJ, -s0, iv_base(kap, C, s0, m0),
                                                kf, xlL, kn, xlL, min(2 * kn + 1, m0));
                     const float ef = fminf(sf.eL, sf.eR);
                     if (flat_certificate(N, dl, d32, ln.h32, m0, 2 * kf - m0, 2 * kn, s0, ef, kap))
