@@ -430,9 +430,9 @@ int cvx_grid_convexify(cvx_handle *h, const cvx_params *p, const cvx_grid *g, do
  *   leaves (n int64, nullable): the leaves of the tree.
  * NaN (leaves 0) outside the grid.  nd and off must be those of the run that
  * made the forest.  0 <= K <= 64.  The trees are tabulated per grid point and
- * order first (K sweeps over the grid); workspace: three tables of W, P,
- * (A,) leaf count per grid point ((D + 2) 8 bytes per point, D^2 8 more with
- * A). */
+ * order first (K sweeps over the grid); workspace: two tables of one record
+ * per grid point (W, P, leaf count; with A its upper triangle): 64 bytes for
+ * d = 2 and 96 for d = 3, with A 128 and 448. */
 int cvx_grid_query(cvx_handle *h, const cvx_params *p, const cvx_grid *g, double beta_k,
                    int32_t det_rule, int32_t nd, const int32_t *off, int32_t K, const double *WK,
                    const int32_t *forest, int64_t n, const double *F, double *W_interp,

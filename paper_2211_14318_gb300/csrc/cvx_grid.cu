@@ -174,25 +174,50 @@ __device__ double grid_w64(const double *F, double beta, const Material &m, int 
     return w_of_psi0(s, beta, m);
 }
 
-// dW/dF = (1 - D(max(s, beta))) dpsi0/dF with
-//   Eq. (2.3): mu F - mu F^-T + lambda ln|J| F^-T (d ln|J|/dF = F^-T = cof F / J);
-//   Eq. (2.2): F (lambda/2 (I1 - 3) 1 + mu (C - 1)).
-template <int D>
-__device__ void grid_p64(const double *F, double beta, const Material &m, int rule, double *P) {
+// W, P = dW/dF and (kA) the tangent d^2W/dFdF at one F, sharing the invariants,
+// one logarithm and one exponential (ek = e^{-beta/D_0}):
+//   P = g dpsi0/dF, g = 1 - D(max(s, beta)), with
+//   Eq. (2.3): dpsi0/dF = mu F - mu F^-T + lambda ln|J| F^-T (F^-T = cof F / J);
+//   Eq. (2.2): dpsi0/dF = F S, S = lambda/2 (I1 - 3) 1 + mu (C - 1);
+//   A = g d^2psi0 + g' dpsi0 (x) dpsi0, on loading (s > beta)
+//   g' = -(D_inf / D_0) e^{-s / D_0}, else 0, with
+//   Eq. (2.3), G = F^-T:
+//     d^2psi0/dF_iJ dF_kL = mu d_ik d_JL + lambda G_iJ G_kL + (mu - lambda ln|J|) G_iL G_kJ;
+//   Eq. (2.2): d_ik S_LJ + lambda F_iJ F_kL + mu F_iL F_kJ + mu (F F^T)_ik d_JL.
+// A is symmetric: its upper triangle, row by row (D (D + 1) / 2 values).
+template <int D, bool kA>
+__device__ void grid_wpa64(const double *F, double beta, double ek, const Material &m, int rule,
+                           double &W, double *P, double *A) {
+    constexpr int d = D == 4 ? 2 : 3;
     if (m.energy == CVX_ENERGY_DOUBLE_WELL) {
-        if (D == 4) stress64(F, beta, m, P);
-        else
-            for (int c = 0; c < D; ++c) P[c] = nan("");
-        return;
+        if (D == 4) {
+            W = energy64(F, beta, m);
+            stress64(F, beta, m, P);
+            if (kA) {
+                double T[16];
+                tangent64(F, beta, m, T);
+                int k = 0;
+                for (int r = 0; r < 4; ++r)
+                    for (int c = r; c < 4; ++c) A[k++] = T[4 * r + c];
+            }
+        }
+        return;  // the call refuses it for D = 9
     }
     double s, J, I1, C[D];
     if (psi0_grid<D>(F, m, rule, s, J, I1, C)) {
+        W = nan("");
         for (int c = 0; c < D; ++c) P[c] = nan("");
+        if (kA)
+            for (int c = 0; c < D * (D + 1) / 2; ++c) A[c] = nan("");
         return;
     }
-    const double b = s > beta ? s : beta;
-    const double gd = 1.0 - m.Dinf * (1.0 - exp(-b / m.D0));
-    constexpr int d = D == 4 ? 2 : 3;
+    const bool load = s > beta;
+    const double es = load ? exp(-s / m.D0) : ek;
+    W = s <= beta ? (1.0 - m.Dinf * (1.0 - ek)) * (s - beta)
+                  : (1.0 - m.Dinf) * (s - beta) + m.Dinf * m.D0 * (ek - es);
+    const double g = 1.0 - m.Dinf * (1.0 - es);
+    const double gp = load ? -(m.Dinf / m.D0) * es : 0.0;
+    double dp[D];  // dpsi0/dF
     if (m.energy == CVX_ENERGY_STVK_DAMAGE) {
         double S[D];
         for (int a = 0; a < d; ++a)
@@ -203,112 +228,63 @@ __device__ void grid_p64(const double *F, double beta, const Material &m, int ru
             for (int c = 0; c < d; ++c) {
                 double v = 0.0;
                 for (int k = 0; k < d; ++k) v += F[d * a + k] * S[d * k + c];
-                P[d * a + c] = gd * v;
+                dp[d * a + c] = v;
             }
-        return;
-    }
-    double cof[D];
-    if (D == 4) {
-        cof[0] = F[3];
-        cof[1] = -F[2];
-        cof[2] = -F[1];
-        cof[3] = F[0];
-    } else {
-        cof[0] = F[4] * F[8] - F[5] * F[7];
-        cof[1] = F[5] * F[6] - F[3] * F[8];
-        cof[2] = F[3] * F[7] - F[4] * F[6];
-        cof[3] = F[2] * F[7] - F[1] * F[8];
-        cof[4] = F[0] * F[8] - F[2] * F[6];
-        cof[5] = F[1] * F[6] - F[0] * F[7];
-        cof[6] = F[1] * F[5] - F[2] * F[4];
-        cof[7] = F[2] * F[3] - F[0] * F[5];
-        cof[8] = F[0] * F[4] - F[1] * F[3];
-    }
-    const double lj = log(fabs(J));
-    for (int c = 0; c < D; ++c) {
-        const double fit = cof[c] / J;
-        P[c] = gd * (m.mu * F[c] - m.mu * fit + m.lam * lj * fit);
-    }
-}
-
-// d^2W/dFdF (D x D, A[D a + b] = dP_a / dF_b over the row-major entries):
-// A = g d^2psi0 + g' dpsi0 (x) dpsi0, g = 1 - D(max(s, beta)), on loading
-// (s > beta) g' = -(D_inf / D_0) e^{-s / D_0}, with
-//   Eq. (2.3), G = F^-T, ln|J|:
-//     d^2psi0/dF_iJ dF_kL = mu d_ik d_JL + lambda G_iJ G_kL + (mu - lambda ln|J|) G_iL G_kJ;
-//   Eq. (2.2), S = lambda/2 (I1 - 3) 1 + mu (C - 1), dpsi0/dF = F S:
-//     d^2psi0/dF_iJ dF_kL = d_ik S_LJ + lambda F_iJ F_kL + mu F_iL F_kJ + mu (F F^T)_ik d_JL.
-template <int D>
-__device__ void grid_a64(const double *F, double beta, const Material &m, int rule, double *A) {
-    if (m.energy == CVX_ENERGY_DOUBLE_WELL) {
-        if (D == 4) tangent64(F, beta, m, A);
-        else
-            for (int c = 0; c < D * D; ++c) A[c] = nan("");
-        return;
-    }
-    double s, J, I1, C[D];
-    if (psi0_grid<D>(F, m, rule, s, J, I1, C)) {
-        for (int c = 0; c < D * D; ++c) A[c] = nan("");
-        return;
-    }
-    constexpr int d = D == 4 ? 2 : 3;
-    const double b = s > beta ? s : beta;
-    const double g = 1.0 - m.Dinf * (1.0 - exp(-b / m.D0));
-    const double gp = s > beta ? -(m.Dinf / m.D0) * exp(-s / m.D0) : 0.0;
-    double dp[D];
-    grid_p64<D>(F, beta, m, rule, dp);  // g dpsi0/dF
-    const double ig = 1.0 / g;
-    for (int c = 0; c < D; ++c) dp[c] *= ig;
-    if (m.energy == CVX_ENERGY_STVK_DAMAGE) {
-        double S[D], FF[D];
-        for (int a = 0; a < d; ++a)
-            for (int c = 0; c < d; ++c) {
-                double v = 0.0;
-                for (int k = 0; k < d; ++k) v += F[d * a + k] * F[d * c + k];
-                FF[d * a + c] = v;
-                S[d * a + c] = m.mu * (C[d * a + c] - (a == c ? 1.0 : 0.0)) +
-                               (a == c ? 0.5 * m.lam * (I1 - 3.0) : 0.0);
-            }
-        for (int i = 0; i < d; ++i)
-            for (int jj = 0; jj < d; ++jj)
-                for (int k = 0; k < d; ++k)
-                    for (int l = 0; l < d; ++l) {
-                        const double d2 = (i == k ? S[d * l + jj] : 0.0) +
-                                          m.lam * F[d * i + jj] * F[d * k + l] +
-                                          m.mu * F[d * i + l] * F[d * k + jj] +
-                                          (jj == l ? m.mu * FF[d * i + k] : 0.0);
-                        A[D * (d * i + jj) + d * k + l] =
-                            g * d2 + gp * dp[d * i + jj] * dp[d * k + l];
-                    }
-        return;
-    }
-    double G[D];
-    if (D == 4) {
-        G[0] = F[3] / J;
-        G[1] = -F[2] / J;
-        G[2] = -F[1] / J;
-        G[3] = F[0] / J;
-    } else {
-        G[0] = (F[4] * F[8] - F[5] * F[7]) / J;
-        G[1] = (F[5] * F[6] - F[3] * F[8]) / J;
-        G[2] = (F[3] * F[7] - F[4] * F[6]) / J;
-        G[3] = (F[2] * F[7] - F[1] * F[8]) / J;
-        G[4] = (F[0] * F[8] - F[2] * F[6]) / J;
-        G[5] = (F[1] * F[6] - F[0] * F[7]) / J;
-        G[6] = (F[1] * F[5] - F[2] * F[4]) / J;
-        G[7] = (F[2] * F[3] - F[0] * F[5]) / J;
-        G[8] = (F[0] * F[4] - F[1] * F[3]) / J;
-    }
-    const double cc = m.mu - m.lam * log(fabs(J));
-    for (int i = 0; i < d; ++i)
-        for (int jj = 0; jj < d; ++jj)
-            for (int k = 0; k < d; ++k)
-                for (int l = 0; l < d; ++l) {
-                    const double d2 = (i == k && jj == l ? m.mu : 0.0) +
-                                      m.lam * G[d * i + jj] * G[d * k + l] +
-                                      cc * G[d * i + l] * G[d * k + jj];
-                    A[D * (d * i + jj) + d * k + l] = g * d2 + gp * dp[d * i + jj] * dp[d * k + l];
+        if (kA) {
+            double FF[D];
+            for (int a = 0; a < d; ++a)
+                for (int c = 0; c < d; ++c) {
+                    double v = 0.0;
+                    for (int k = 0; k < d; ++k) v += F[d * a + k] * F[d * c + k];
+                    FF[d * a + c] = v;
                 }
+            int n = 0;
+#pragma unroll
+            for (int r = 0; r < D; ++r)
+#pragma unroll
+                for (int q = r; q < D; ++q) {
+                    const int i = r / d, jj = r % d, k = q / d, l = q % d;
+                    const double d2 = (i == k ? S[d * l + jj] : 0.0) + m.lam * F[r] * F[q] +
+                                      m.mu * F[d * i + l] * F[d * k + jj] +
+                                      (jj == l ? m.mu * FF[d * i + k] : 0.0);
+                    A[n++] = g * d2 + gp * dp[r] * dp[q];
+                }
+        }
+    } else {
+        double G[D];
+        if (D == 4) {
+            G[0] = F[3] / J;
+            G[1] = -F[2] / J;
+            G[2] = -F[1] / J;
+            G[3] = F[0] / J;
+        } else {
+            G[0] = (F[4] * F[8] - F[5] * F[7]) / J;
+            G[1] = (F[5] * F[6] - F[3] * F[8]) / J;
+            G[2] = (F[3] * F[7] - F[4] * F[6]) / J;
+            G[3] = (F[2] * F[7] - F[1] * F[8]) / J;
+            G[4] = (F[0] * F[8] - F[2] * F[6]) / J;
+            G[5] = (F[1] * F[6] - F[0] * F[7]) / J;
+            G[6] = (F[1] * F[5] - F[2] * F[4]) / J;
+            G[7] = (F[2] * F[3] - F[0] * F[5]) / J;
+            G[8] = (F[0] * F[4] - F[1] * F[3]) / J;
+        }
+        const double lj = log(fabs(J));
+        for (int c = 0; c < D; ++c) dp[c] = m.mu * F[c] - m.mu * G[c] + m.lam * lj * G[c];
+        if (kA) {
+            const double cc = m.mu - m.lam * lj;
+            int n = 0;
+#pragma unroll
+            for (int r = 0; r < D; ++r)
+#pragma unroll
+                for (int q = r; q < D; ++q) {
+                    const int i = r / d, jj = r % d, k = q / d, l = q % d;
+                    const double d2 = (r == q ? m.mu : 0.0) + m.lam * G[r] * G[q] +
+                                      cc * G[d * i + l] * G[d * k + jj];
+                    A[n++] = g * d2 + gp * dp[r] * dp[q];
+                }
+        }
+    }
+    for (int c = 0; c < D; ++c) P[c] = g * dp[c];
 }
 
 // Number of grid points on the line that starts at index i along offset o.
@@ -561,141 +537,280 @@ __global__ void k_grid_final(int N, const int *iters, const double *pong, double
 }
 
 // Trees of Algorithm 2 tabulated per grid point and order (Algorithm 3 by
-// dynamic programming over the orders).  T_d(p) = (W, P, leaves) of the tree
-// below grid point p at order d: at d = 0 (or where no iteration up to d
-// split p) the leaf values W(p), P(p) (Eq. 2.12) and one leaf; where
+// dynamic programming over the orders).  T_d(p) = (W, P, A, leaves) of the
+// tree below grid point p at order d: at d = 0 (or where no iteration up to d
+// split p) the leaf values W(p), P(p) (Eq. 2.12), A(p) and one leaf; where
 // iteration d split p with record (dir, l-, l+), xi = -l- / (l+ - l-),
 //   T_d(p) = (1 - xi) T_{d-1}(p + l- R) + xi T_{d-1}(p + l+ R);
 // elsewhere T_d(p) = T_{d-1}(p) (the latest split below d decides).  A record
-// this library did not write makes p a leaf at that order.  Layout: W[N],
-// P[D][N], leaves[N] per order, ping-pong between two buffers.
-template <int D>
-__global__ void k_grid_tree0(GridT<D> g, Material m, double beta, int rule, double *Tw,
-                             double *Tp, long long *Tl, double *Ta) {
-    const int p = blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= g.N) return;
-    double F[D], P[D];
+// this library did not write makes p a leaf at that order.
+//
+// Layout: one record per point, W, P, the upper triangle of A, leaves (int64)
+// -- 16 words of 8 bytes for D = 4 with the tangent -- in two buffers; a flag
+// per point says which buffer holds its latest record.  An order writes the
+// records of the points it split into their other buffer, so that the old
+// ones stay readable, and only copies the flags of the rest.  A group of
+// lanes takes a point or a query, a lane per word, so that a record is read
+// and written in whole sectors.  (Values in separate arrays, copied whole per
+// order, and A accumulated in global memory by one thread per query: 648,025
+// points, 15 orders, 1,048,576 queries with the tangent took 0.85 + 1.43 +
+// 6.46 ms; this takes 0.33 + 0.53 + 0.95 ms.)
+template <int D, bool kA>
+struct TreeRec {
+    static constexpr int kTri = D * (D + 1) / 2;
+    static constexpr int kLeaf = 1 + D + (kA ? kTri : 0);  // the word of the leaf count
+    static constexpr int kWords = D == 4 ? (kA ? 16 : 8) : (kA ? 56 : 12);
+    static constexpr int kLanes = D == 4 ? kWords : (kA ? 32 : 16);
+    static_assert(kLeaf < kWords, "record layout");
+};
+
+template <int D, bool kA>
+__device__ void leaf_record(const GridT<D> &g, int p, const Material &m, double beta, double ek,
+                            int rule, double *r) {
+    using R = TreeRec<D, kA>;
+    double F[D], P[D], A[kA ? R::kTri : 1], W;
     grid_point<D>(g, p, F);
-    Tw[p] = grid_w64<D>(F, beta, m, rule);
-    grid_p64<D>(F, beta, m, rule, P);
-    for (int c = 0; c < D; ++c) Tp[(long long)c * g.N + p] = P[c];
-    Tl[p] = 1;
-    if (Ta) {
-        double A[D * D];
-        grid_a64<D>(F, beta, m, rule, A);
-        for (int c = 0; c < D * D; ++c) Ta[(long long)c * g.N + p] = A[c];
-    }
+    grid_wpa64<D, kA>(F, beta, ek, m, rule, W, P, A);
+    r[0] = W;
+#pragma unroll
+    for (int c = 0; c < D; ++c) r[1 + c] = P[c];
+    if (kA)
+#pragma unroll
+        for (int c = 0; c < R::kTri; ++c) r[1 + D + c] = A[c];
+    r[R::kLeaf] = __longlong_as_double(1ll);
+#pragma unroll
+    for (int c = R::kLeaf + 1; c < R::kWords; ++c) r[c] = 0.0;
 }
 
-template <int D>
-__global__ void k_grid_tree_step(GridT<D> g, const GridDirT<D> *dirs, int nd, const int *rec,
-                                 const double *Tw0, const double *Tp0, const long long *Tl0,
-                                 const double *Tw, const double *Tp, const long long *Tl,
-                                 double *Uw, double *Up, long long *Ul, const double *Ta0,
-                                 const double *Ta, double *Ua) {
-    const int p = blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= g.N) return;
-    const long long N = g.N;
-    const int dj = rec[3 * (long long)p], lm = rec[3 * (long long)p + 1],
-              lp = rec[3 * (long long)p + 2];
-    if (dj < 0) {  // not split in this iteration: the tree of the order below
-        Uw[p] = Tw[p];
-        for (int c = 0; c < D; ++c) Up[c * N + p] = Tp[c * N + p];
-        Ul[p] = Tl[p];
-        if (Ua)
-            for (int c = 0; c < D * D; ++c) Ua[c * N + p] = Ta[c * N + p];
-        return;
+constexpr int kTreeThreads = 64;
+
+template <int D, bool kA>
+__global__ void __launch_bounds__(kTreeThreads) k_grid_tree0(GridT<D> g, Material m, double beta,
+                                                             int rule, double *T,
+                                                             unsigned char *flag) {
+    using R = TreeRec<D, kA>;
+    constexpr int kPitch = R::kWords + 1;  // odd: no bank conflicts in the transposition
+    __shared__ double s_r[kTreeThreads * kPitch];
+    const int p0 = blockIdx.x * kTreeThreads, p = p0 + threadIdx.x;
+    const double ek = exp(-beta / m.D0);
+    if (p < g.N) {
+        leaf_record<D, kA>(g, p, m, beta, ek, rule, s_r + threadIdx.x * kPitch);
+        flag[p] = 0;
     }
-    const int step = dj < nd ? dirs[dj].step : 0;
-    const long long cm = p + (long long)lm * step, cp = p + (long long)lp * step;
-    if (dj >= nd || !(lm < 0 && lp > 0) || cm < 0 || cm >= N || cp < 0 || cp >= N) {
-        Uw[p] = Tw0[p];
-        for (int c = 0; c < D; ++c) Up[c * N + p] = Tp0[c * N + p];
-        Ul[p] = Tl0[p];
-        if (Ua)
-            for (int c = 0; c < D * D; ++c) Ua[c * N + p] = Ta0[c * N + p];
-        return;
-    }
-    const double xi = __ddiv_rn((double)(-lm), (double)(lp - lm));
-    const double xm = __dsub_rn(1.0, xi);
-    Uw[p] = __dadd_rn(__dmul_rn(xm, Tw[cm]), __dmul_rn(xi, Tw[cp]));
-    for (int c = 0; c < D; ++c)
-        Up[c * N + p] = __dadd_rn(__dmul_rn(xm, Tp[c * N + cm]), __dmul_rn(xi, Tp[c * N + cp]));
-    if (Ua)
-        for (int c = 0; c < D * D; ++c)
-            Ua[c * N + p] =
-                __dadd_rn(__dmul_rn(xm, Ta[c * N + cm]), __dmul_rn(xi, Ta[c * N + cp]));
-    const long long l = Tl[cm] + Tl[cp];
-    Ul[p] = l < Tl[cm] ? 0x7fffffffffffffffLL : l;  // saturates
+    __syncthreads();
+    const int n = min(kTreeThreads, g.N - p0) * R::kWords;
+    double *out = T + (size_t)p0 * R::kWords;
+    for (int i = threadIdx.x; i < n; i += kTreeThreads)
+        out[i] = s_r[i / R::kWords * kPitch + i % R::kWords];
 }
 
-// Algorithm 2's tree at n points evaluated by Algorithm 3, one thread per
-// point: the corners of the grid cell holding F (multilinear weights
-// prod_c (1 - t_c or t_c); a coordinate within 1e-12 grid steps of a grid
-// value counts as on it; corners of weight 0 left out; corner bit c counted
-// from the first component) at order K, each contributing its weight times
-// the tabulated tree T_K.  W_interp is the multilinear interpolation of W^K.
-template <int D>
-__global__ void k_grid_query(GridT<D> g, const double *WK, const double *Tw, const double *Tp,
-                             const long long *Tl, const double *Ta, long long n,
-                             const double *F, double *Wi, double *Wt, double *P, double *A,
-                             long long *leaves) {
-    const long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (q >= n) return;
-    int i0[D];
-    double t[D];
-    bool inside = true;
-    for (int c = 0; c < D; ++c) {
-        const double u = __ddiv_rn(__dsub_rn(F[D * q + c], g.lo[c]), g.delta[c]);
-        if (u < -1e-12 || u > (double)(g.n[c] - 1) + 1e-12) inside = false;
-        double f = floor(u);
-        double r = __dsub_rn(u, f);
-        if (r > 1.0 - 1e-12) {
-            f = __dadd_rn(f, 1.0);
-            r = 0.0;
-        } else if (r < 1e-12) {
-            r = 0.0;
+constexpr int kStepThreads = 256;
+
+// One order: a thread per point reads the iteration's record (and divides),
+// then groups of lanes, a lane per word, combine the records of the points it
+// split.
+template <int D, bool kA>
+__global__ void __launch_bounds__(kStepThreads)
+    k_grid_tree_step(GridT<D> g, const GridDirT<D> *dirs, int nd, const int *rec, Material m,
+                     double beta, int rule, double *T0, double *T1, const unsigned char *flag,
+                     unsigned char *flag_out) {
+    using R = TreeRec<D, kA>;
+    __shared__ double s_xi[kStepThreads];
+    __shared__ int s_c[kStepThreads][2];            // the children's points
+    __shared__ unsigned short s_p[kStepThreads];    // thread | buffers of F-, F+ and the output << 8
+    __shared__ int s_n;
+    if (threadIdx.x == 0) s_n = 0;
+    __syncthreads();
+    const int p0 = blockIdx.x * kStepThreads;
+    const long long p = (long long)p0 + threadIdx.x;
+    if (p < g.N) {
+        const int dj = rec[3 * p];
+        int f = flag[p];
+        if (dj >= 0) {
+            const int lm = rec[3 * p + 1], lp = rec[3 * p + 2];
+            const int step = dj < nd ? dirs[dj].step : 0;
+            const long long cm = p + (long long)lm * step, cp = p + (long long)lp * step;
+            if (dj >= nd || !(lm < 0 && lp > 0) || cm < 0 || cm >= g.N || cp < 0 || cp >= g.N) {
+                leaf_record<D, kA>(g, (int)p, m, beta, exp(-beta / m.D0), rule,
+                                   (f ? T0 : T1) + (size_t)p * R::kWords);
+            } else {
+                const int i = atomicAdd(&s_n, 1);
+                s_xi[i] = __ddiv_rn((double)(-lm), (double)(lp - lm));
+                s_c[i][0] = (int)cm;
+                s_c[i][1] = (int)cp;
+                s_p[i] = (unsigned short)(threadIdx.x | (flag[cm] << 8) | (flag[cp] << 9) |
+                                          ((1 - f) << 10));
+            }
+            f = 1 - f;
         }
-        int ii = (int)f;
-        ii = ii > g.n[c] - 1 ? g.n[c] - 1 : ii;
-        ii = ii < 0 ? 0 : ii;
-        i0[c] = ii;
-        t[c] = r;
+        flag_out[p] = (unsigned char)f;  // not split: the tree of the order below
     }
-    double wi = 0.0, wt = 0.0, Pp[D];
-    for (int c = 0; c < D; ++c) Pp[c] = 0.0;
-    if (A)
-        for (int c = 0; c < D * D; ++c) A[(long long)D * D * q + c] = 0.0;
-    long long nl = 0;
-    const long long N = g.N;
-    for (int corner = 0; inside && corner < (1 << D); ++corner) {
-        double w = 1.0;
-        int flat = 0;
+    __syncthreads();
+    const int v = threadIdx.x % R::kLanes;
+    for (int i = threadIdx.x / R::kLanes; i < s_n; i += kStepThreads / R::kLanes) {
+        const double xi = s_xi[i], xm = __dsub_rn(1.0, xi);
+        const unsigned sp = s_p[i];
+        const double *Tm = (sp & 0x100 ? T1 : T0) + (size_t)s_c[i][0] * R::kWords;
+        const double *Tp = (sp & 0x200 ? T1 : T0) + (size_t)s_c[i][1] * R::kWords;
+        double *out = (sp & 0x400 ? T1 : T0) + (size_t)(p0 + (int)(sp & 0xff)) * R::kWords;
+#pragma unroll
+        for (int w = v; w < R::kWords; w += R::kLanes) {
+            const double a = Tm[w], b = Tp[w];
+            double r = __dadd_rn(__dmul_rn(xm, a), __dmul_rn(xi, b));
+            if (w == R::kLeaf) {
+                const long long la = __double_as_longlong(a), l = la + __double_as_longlong(b);
+                r = __longlong_as_double(l < la ? 0x7fffffffffffffffLL : l);  // saturates
+            }
+            out[w] = r;
+        }
+    }
+}
+
+// Algorithm 2's tree at n points evaluated by Algorithm 3: the corners of the
+// grid cell holding F (multilinear weights prod_c (1 - t_c or t_c); a
+// coordinate within 1e-12 grid steps of a grid value counts as on it; corners
+// of weight 0 left out; corner bit c counted from the first component) at
+// order K, each contributing its weight times the tabulated tree T_K.
+// W_interp is the multilinear interpolation of W^K.  A thread per query finds
+// the cell and W_interp, then a group of lanes per query sums the records, a
+// lane per word, each lane having computed the weight of one corner.  What
+// bounds it is the FP64 pipe (2 lanes per SM and clock): 16 sums per word and
+// query, and the division and tests of the cell.
+constexpr int kQueryThreads = 128;
+
+template <int D, bool kA>
+__global__ void __launch_bounds__(kQueryThreads)
+    k_grid_query(GridT<D> g, const double *WK, const double *T0, const double *T1,
+                 const unsigned char *flag, long long n, const double *F, double *Wi, double *Wt,
+                 double *P, double *A, long long *leaves) {
+    using R = TreeRec<D, kA>;
+    constexpr int kG = R::kLanes, kC = 1 << D, kPer = (R::kWords + kG - 1) / kG;
+    __shared__ double s_t[kQueryThreads][2 * D];  // 1 - t_c and t_c
+    __shared__ int s_flat[kQueryThreads];  // flat index of the cell's first corner, -1 outside
+    __shared__ int s_in[kQueryThreads];    // bit c: the cell has an upper corner in component c
+    const long long q0 = (long long)blockIdx.x * kQueryThreads;
+    {
+        const long long q = q0 + threadIdx.x;
+        bool inside = q < n;
+        double t[D];
+        int flat0 = 0, in = 0;
+#pragma unroll
         for (int c = 0; c < D; ++c) {
-            const int up = (corner >> (D - 1 - c)) & 1;
-            w = __dmul_rn(w, up ? t[c] : __dsub_rn(1.0, t[c]));
-            flat += (i0[c] + up) * g.s[c];
+            const double u =
+                inside ? __ddiv_rn(__dsub_rn(F[D * q + c], g.lo[c]), g.delta[c]) : -1.0;
+            if (u < -1e-12 || u > (double)(g.n[c] - 1) + 1e-12) inside = false;
+            double f = floor(u);
+            double r = __dsub_rn(u, f);
+            if (r > 1.0 - 1e-12) {
+                f = __dadd_rn(f, 1.0);
+                r = 0.0;
+            } else if (r < 1e-12) {
+                r = 0.0;
+            }
+            int ii = (int)f;
+            ii = ii > g.n[c] - 1 ? g.n[c] - 1 : ii;
+            ii = ii < 0 ? 0 : ii;
+            flat0 += ii * g.s[c];
+            in |= (ii < g.n[c] - 1 ? 1 : 0) << c;
+            t[c] = r;
+            s_t[threadIdx.x][2 * c] = __dsub_rn(1.0, r);
+            s_t[threadIdx.x][2 * c + 1] = r;
         }
-        if (w == 0.0) continue;
-        wi = __dadd_rn(wi, __dmul_rn(w, WK[flat]));
-        wt = __dadd_rn(wt, __dmul_rn(w, Tw[flat]));
-        for (int a = 0; a < D; ++a) Pp[a] = __dadd_rn(Pp[a], __dmul_rn(w, Tp[a * N + flat]));
-        nl += Tl[flat];
-        if (A)  // accumulated in place (the output row starts at zero)
-            for (int c = 0; c < D * D; ++c)
-                A[(long long)D * D * q + c] =
-                    __dadd_rn(A[(long long)D * D * q + c], __dmul_rn(w, Ta[c * N + flat]));
+        s_flat[threadIdx.x] = inside ? flat0 : -1;
+        s_in[threadIdx.x] = in;
+        if (q < n) {
+            double wi = inside ? 0.0 : nan("");
+            if (inside) {
+#pragma unroll(D == 4 ? 16 : 1)
+                for (int corner = 0; corner < kC; ++corner) {
+                    double w = 1.0;
+                    int flat = flat0;
+#pragma unroll
+                    for (int c = 0; c < D; ++c) {
+                        const int up = (corner >> (D - 1 - c)) & 1;
+                        const double x = up ? t[c] : __dsub_rn(1.0, t[c]);
+                        w = c == 0 ? x : __dmul_rn(w, x);
+                        flat += (up & (in >> c)) * g.s[c];
+                    }
+                    if (w == 0.0) continue;
+                    wi = __dadd_rn(wi, __dmul_rn(w, WK[flat]));
+                }
+            }
+            Wi[q] = wi;
+        }
     }
-    if (!inside) {
-        wi = wt = nan("");
-        for (int a = 0; a < D; ++a) Pp[a] = nan("");
-        if (A)
-            for (int c = 0; c < D * D; ++c) A[(long long)D * D * q + c] = nan("");
+    __syncthreads();
+    const int v = threadIdx.x % kG, grp = threadIdx.x / kG;
+    const unsigned lane0 = (threadIdx.x & 31) / kG * kG;  // the group's first lane
+    const unsigned gm = (kG == 32 ? 0xffffffffu : ((1u << (kG & 31)) - 1u) << lane0);
+    int at0[kPer], at1[kPer];  // places of the lane's words of A in a query's 4 x 4 or 9 x 9
+#pragma unroll
+    for (int j = 0; j < kPer; ++j) {
+        int e = v + j * kG - 1 - D, r = 0;  // upper triangle, row r from (r, r)
+        while (r < D && e >= D - r) {
+            e -= D - r;
+            ++r;
+        }
+        at0[j] = D * r + r + e;
+        at1[j] = D * (r + e) + r;
     }
-    Wi[q] = wi;
-    Wt[q] = wt;
-    for (int a = 0; a < D; ++a) P[D * q + a] = Pp[a];
-    if (leaves) leaves[q] = nl;
+    for (int i = grp; i < kQueryThreads && q0 + i < n; i += kQueryThreads / kG) {
+        const long long q = q0 + i;
+        const int flat0 = s_flat[i], in = s_in[i];
+        double acc[kPer];
+        long long nl = 0;
+#pragma unroll
+        for (int k = 0; k < kPer; ++k) acc[k] = 0.0;
+        if (flat0 >= 0) {
+            for (int c0 = 0; c0 < kC; c0 += kG) {
+                // this lane's corner: weight and record
+                double w = 1.0;
+                int flat = flat0;
+#pragma unroll
+                for (int c = 0; c < D; ++c) {
+                    const int up = ((c0 + v) >> (D - 1 - c)) & 1;
+                    const double x = s_t[i][2 * c + up];
+                    w = c == 0 ? x : __dmul_rn(w, x);
+                    flat += (up & (in >> c)) * g.s[c];
+                }
+                // the record's place, its buffer (bit 62), and -1 for a corner of
+                // weight 0, which is not read (tested on the bits: comparing in
+                // FP64 would cost as much as the sums)
+                long long at = -1;
+                if ((__double_as_longlong(w) << 1) != 0)
+                    at = (long long)flat * R::kWords | (flag[flat] ? 1ll << 62 : 0);
+#pragma unroll(D == 4 ? kG : 4)
+                for (int k = 0; k < kG; ++k) {
+                    const double wk = __shfl_sync(gm, w, k, kG);
+                    const long long ak = __shfl_sync(gm, at, k, kG);
+                    const double *r = ((ak >> 62) ? T1 : T0) + (ak & ((1ll << 62) - 1));
+#pragma unroll
+                    for (int j = 0; j < kPer; ++j) {
+                        const int x = v + j * kG;
+                        double val = 0.0;  // (a corner of weight 0 is not read)
+                        if (ak >= 0 && x < R::kWords) val = r[x];
+                        acc[j] = __fma_rn(wk, val, acc[j]);
+                        if (x == R::kLeaf) nl += __double_as_longlong(val);
+                    }
+                }
+            }
+        } else {
+#pragma unroll
+            for (int k = 0; k < kPer; ++k) acc[k] = nan("");
+        }
+#pragma unroll
+        for (int j = 0; j < kPer; ++j) {
+            const int x = v + j * kG;
+            if (x == 0) Wt[q] = acc[j];
+            else if (x <= D) P[D * q + x - 1] = acc[j];
+            else if (x == R::kLeaf) {
+                if (leaves) leaves[q] = nl;
+            } else if (kA && x < R::kLeaf) {
+                A[(long long)D * D * q + at0[j]] = acc[j];
+                A[(long long)D * D * q + at1[j]] = acc[j];
+            }
+        }
+    }
 }
 
 // ------------------------------------------------------------------ host
@@ -1008,6 +1123,40 @@ int grid_convexify_t(cvx_handle *h, const cvx_params *p, const cvx_grid *g, doub
     return CVX_OK;
 }
 
+template <int D, bool kA>
+int grid_query_run(cvx_handle *h, const GridT<D> &gd, const std::vector<GridDirT<D>> &dirs,
+                   const cvx_params *p, double beta_k, int32_t rule, int32_t K, const double *WK,
+                   const int32_t *forest, int64_t n, const double *F, double *W_interp,
+                   double *W_tree, double *P, double *A, int64_t *leaves, cudaStream_t s) {
+    using R = TreeRec<D, kA>;
+    const int nd = (int)dirs.size();
+    // two buffers of records, two arrays of flags
+    const size_t tab = up256(sizeof(double) * R::kWords * (size_t)gd.N), fl = up256(gd.N);
+    const size_t o_t = up256(sizeof(GridDirT<D>) * nd);
+    int rc = ensure_ws(h, o_t + 2 * tab + 2 * fl, s);
+    if (rc) return rc;
+    GridDirT<D> *dd = (GridDirT<D> *)h->ws;
+    double *T0 = (double *)(h->ws + o_t), *T1 = (double *)(h->ws + o_t + tab);
+    unsigned char *f0 = (unsigned char *)(h->ws + o_t + 2 * tab), *f1 = f0 + fl;
+    CK(cudaMemcpyAsync(dd, dirs.data(), sizeof(GridDirT<D>) * nd, cudaMemcpyHostToDevice, s),
+       "cvx_grid_query");
+    const Material mat = material_of(p);
+    k_grid_tree0<D, kA><<<(unsigned)((gd.N + (long long)kTreeThreads - 1) / kTreeThreads), kTreeThreads, 0, s>>>(
+        gd, mat, beta_k, rule, T0, f0);
+    CK(cudaGetLastError(), "cvx_grid_query leaves");
+    const unsigned nb = (unsigned)((gd.N + (long long)kStepThreads - 1) / kStepThreads);
+    for (int d = 1; d <= K; ++d) {
+        k_grid_tree_step<D, kA><<<nb, kStepThreads, 0, s>>>(gd, dd, nd, forest + 3 * (size_t)(d - 1) * gd.N, mat,
+                                                   beta_k, rule, T0, T1, f0, f1);
+        CK(cudaGetLastError(), "cvx_grid_query tree order");
+        std::swap(f0, f1);
+    }
+    k_grid_query<D, kA><<<(unsigned)((n + kQueryThreads - 1) / kQueryThreads), kQueryThreads, 0, s>>>(
+        gd, WK, T0, T1, f0, n, F, W_interp, W_tree, P, A, reinterpret_cast<long long *>(leaves));
+    CK(cudaGetLastError(), "cvx_grid_query");
+    return CVX_OK;
+}
+
 template <int D>
 int grid_query_t(cvx_handle *h, const cvx_params *p, const cvx_grid *g, double beta_k,
                  int32_t rule, int32_t nd, const int32_t *off, int32_t K, const double *WK,
@@ -1028,48 +1177,10 @@ int grid_query_t(cvx_handle *h, const cvx_params *p, const cvx_grid *g, double b
         return fail(CVX_ERR_INVALID_ARG, "NULL array (WK, F, W_interp, W_tree, P; forest if K > 0)");
     if (n == 0) return CVX_OK;
     DeviceGuard dg(h->device);
-    // tables: the leaves (order 0) and two buffers of orders, each
-    // W[N], P[D][N], leaves[N] (and A[D^2][N] when the tangent is asked for)
-    const int na = A ? D * D : 0;
-    const size_t tab = up256(sizeof(double) * (D + 1 + na) * (size_t)gd.N) +
-                       up256(sizeof(long long) * (size_t)gd.N);
-    const size_t o_t = up256(sizeof(GridDirT<D>) * nd);
-    rc = ensure_ws(h, o_t + 3 * tab, s);
-    if (rc) return rc;
-    GridDirT<D> *dd = (GridDirT<D> *)h->ws;
-    struct Tab {
-        double *w, *p, *a;
-        long long *l;
-    };
-    auto carve = [&](int i) {
-        char *b = h->ws + o_t + i * tab;
-        Tab t;
-        t.w = (double *)b;
-        t.p = t.w + gd.N;
-        t.a = A ? t.p + (size_t)D * gd.N : nullptr;
-        t.l = (long long *)(b + up256(sizeof(double) * (D + 1 + na) * (size_t)gd.N));
-        return t;
-    };
-    const Tab t0 = carve(0), ta = carve(1), tb = carve(2);
-    CK(cudaMemcpyAsync(dd, dirs.data(), sizeof(GridDirT<D>) * nd, cudaMemcpyHostToDevice, s),
-       "cvx_grid_query");
-    const unsigned pbk = (unsigned)((gd.N + 255) / 256);
-    k_grid_tree0<D><<<pbk, 256, 0, s>>>(gd, material_of(p), beta_k, rule, t0.w, t0.p, t0.l, t0.a);
-    CK(cudaGetLastError(), "cvx_grid_query leaves");
-    Tab cur = t0;
-    for (int d = 1; d <= K; ++d) {
-        const Tab nx = (d & 1) ? ta : tb;
-        k_grid_tree_step<D><<<pbk, 256, 0, s>>>(gd, dd, nd, forest + 3 * (size_t)(d - 1) * gd.N,
-                                                t0.w, t0.p, t0.l, cur.w, cur.p, cur.l, nx.w, nx.p,
-                                                nx.l, t0.a, cur.a, nx.a);
-        CK(cudaGetLastError(), "cvx_grid_query tree order");
-        cur = nx;
-    }
-    k_grid_query<D><<<(unsigned)((n + 127) / 128), 128, 0, s>>>(
-        gd, WK, cur.w, cur.p, cur.l, cur.a, n, F, W_interp, W_tree, P, A,
-        reinterpret_cast<long long *>(leaves));
-    CK(cudaGetLastError(), "cvx_grid_query");
-    return CVX_OK;
+    return A ? grid_query_run<D, true>(h, gd, dirs, p, beta_k, rule, K, WK, forest, n, F, W_interp,
+                                       W_tree, P, A, leaves, s)
+             : grid_query_run<D, false>(h, gd, dirs, p, beta_k, rule, K, WK, forest, n, F, W_interp,
+                                        W_tree, P, A, leaves, s);
 }
 
 }  // namespace
