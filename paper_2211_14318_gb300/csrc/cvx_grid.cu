@@ -13,12 +13,11 @@
 // lower hull: the value of Eq. (4.3) at a point is the hull read at that
 // point.  So one thread builds Algorithm 1's hull of one (direction, line)
 // pair once (a stack in shared memory) and then walks the line again: a
-// point strictly inside a hull edge records the numerator of its chord value
-// and the edge's ends.  The per-point minimum over the directions (lowest
+// point strictly inside a hull edge records the edge's ends and an FP32 lower
+// bound of its chord value.  The per-point minimum over the directions (lowest
 // direction index on equal values, a strict decrease required) is a second
-// kernel over the points; it divides only where a direction can still win
-// (a product with the rounded reciprocal of the integer denominator bounds
-// the quotient from below first).  Predicates and chord values are the FP64
+// kernel over the points; it evaluates in FP64 only the directions whose bound
+// says that they can win.  Predicates and chord values are the FP64
 // expressions of the hull at the point with every operation rounded on its
 // own (no contraction into FMA): the hull's vertex set does not depend on
 // where the line is read, so each step is reproducible bit for bit.
@@ -67,6 +66,7 @@ template <int D>
 struct GridDirT {
     int o[D];  // grid-index offset of one step along the line
     int step;  // its flat-index step
+    unsigned pos, neg;  // bit c: o[c] > 0, o[c] < 0
 };
 
 __device__ __forceinline__ bool finite_bits(double x) {
@@ -93,6 +93,16 @@ __device__ __forceinline__ double exact_double(int v) {
     return __longlong_as_double((long long)bits);
 }
 
+// A double truncated to FP32 on the integer pipe (relative error below
+// 2^-23; magnitudes below 2^-126 give 0, above 2^127 infinity).
+__device__ __forceinline__ float trunc32(double x) {
+    const int hi = __double2hiint(x), lo = __double2loint(x);
+    const int m = (hi & 0x7fffffff) - (896 << 20);  // exponent rebiased, top 20 fraction bits
+    int b = (m << 3) | (int)((unsigned)lo >> 29);
+    b = m < (1 << 20) ? 0 : (m >= (254 << 20) ? 0x7f800000 : b);
+    return __int_as_float(b | (hi & 0x80000000));
+}
+
 template <int D>
 __device__ __forceinline__ void grid_index(const GridT<D> &g, int idx, int *i) {
 #pragma unroll
@@ -112,9 +122,8 @@ __device__ __forceinline__ void grid_point(const GridT<D> &g, int idx, double *F
 }
 
 // Eq. (2.9) in s = psi0: s <= beta: (1 - D(beta)) (s - beta); otherwise
-// (1 - D_inf)(s - beta) + D_inf D_0 (e^{-beta/D_0} - e^{-s/D_0}).
-__device__ __forceinline__ double w_of_psi0(double s, double beta, const Material &m) {
-    const double ek = exp(-beta / m.D0);
+// (1 - D_inf)(s - beta) + D_inf D_0 (e^{-beta/D_0} - e^{-s/D_0}); ek = e^{-beta/D_0}.
+__device__ __forceinline__ double w_of_psi0(double s, double beta, double ek, const Material &m) {
     if (s <= beta) return (1.0 - m.Dinf * (1.0 - ek)) * (s - beta);
     return (1.0 - m.Dinf) * (s - beta) + m.Dinf * m.D0 * (ek - exp(-s / m.D0));
 }
@@ -164,14 +173,6 @@ __device__ bool psi0_grid(const double *F, const Material &m, int rule, double &
     const double lj = log(aj);
     s = 0.5 * m.mu * (I1 - 3.0) - m.mu * lj + 0.5 * m.lam * lj * lj;
     return rule == 0 ? !(J > 0.0) : !(aj > 0.0);
-}
-
-template <int D>
-__device__ double grid_w64(const double *F, double beta, const Material &m, int rule) {
-    if (m.energy == CVX_ENERGY_DOUBLE_WELL) return D == 4 ? energy64(F, beta, m) : nan("");
-    double s, J, I1, C[D];
-    if (psi0_grid<D>(F, m, rule, s, J, I1, C)) return nan("");
-    return w_of_psi0(s, beta, m);
 }
 
 // W, P = dW/dF and (kA) the tangent d^2W/dFdF at one F, sharing the invariants,
@@ -301,30 +302,73 @@ __device__ __forceinline__ int line_length(const GridT<D> &g, const int *i, cons
 
 // W^0 on the grid.
 template <int D>
-__global__ void k_grid_energy(GridT<D> g, Material m, double beta, int rule, double *W) {
+__global__ void __launch_bounds__(256) k_grid_energy(GridT<D> g, Material m, double beta, int rule,
+                                                     double *W) {
+    __shared__ double s_ek;
+    if (threadIdx.x < 32) s_ek = exp(-beta / m.D0);  // once per block: FP64 work
+    __syncthreads();
     const int p = blockIdx.x * blockDim.x + threadIdx.x;
     if (p >= g.N) return;
     double F[D];
     grid_point<D>(g, p, F);
-    W[p] = grid_w64<D>(F, beta, m, rule);
+    double w = nan("");
+    if (m.energy == CVX_ENERGY_DOUBLE_WELL) {
+        if (D == 4) w = energy64(F, beta, m);
+    } else {
+        double s, J, I1, C[D];
+        if (!psi0_grid<D>(F, m, rule, s, J, I1, C)) w = w_of_psi0(s, beta, s_ek, m);
+    }
+    W[p] = w;
+}
+
+// Lines.  Only lines of three points or more matter: the ends of a line are
+// vertices of its hull, so a point can split along a direction only if both
+// its neighbours along it lie in the grid ("interior" below).  In nine
+// dimensions with three values per off-diagonal component that leaves a few
+// directions per point of the 169.
+//
+// The number of lines of m or more points of a direction o is
+// C(m) - C(m + 1), C(m) = prod_c max(0, n_c - (m - 1) |o_c|) (the points whose
+// (m - 1)-fold successor lies in the grid).
+template <int D>
+__host__ __device__ inline long long lines_of(const GridT<D> &g, const GridDirT<D> &d, int m) {
+    long long a = 1, b = 1;
+    for (int c = 0; c < D; ++c) {
+        const long long o = d.o[c] < 0 ? -d.o[c] : d.o[c];
+        const long long x = g.n[c] - (m - 1) * o, y = x - o;
+        a *= x > 0 ? x : 0;
+        b *= y > 0 ? y : 0;
+    }
+    return a - b;
+}
+
+// cur[j][len]: where the next line of that length goes in direction j's region
+// of the starts, longest lines first, so that a warp of the line kernel takes
+// lines of one length.  Once k_grid_starts has placed the lines, cur[j][len]
+// is the number of lines of len or more points.
+template <int D>
+__global__ void k_grid_cursors(GridT<D> g, const GridDirT<D> *dirs, int nd, int cap, unsigned *cur) {
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= nd * (cap + 1)) return;
+    cur[t] = (unsigned)lines_of<D>(g, dirs[t / (cap + 1)], t % (cap + 1) + 1);
 }
 
 // Line starts: per point (one index decomposition) and direction j, the point
-// starts a line if its predecessor along j lies outside the grid.  The starts
-// of region j of `starts` (line_off[j] .. line_off[j + 1]) are ordered by
-// line length, longest first, so that a warp of the line kernel takes lines
-// of one length (a counting sort: phase 0 counts the lines of each
-// (direction, length) in hist, k_grid_len_scan turns the counts into
-// offsets, phase 1 places each start at its offset; the order among lines of
-// one length is arbitrary and changes no result).  Lanes of a warp with the
-// same (direction, length) share one atomic.  The direction offsets are
-// staged in shared memory.
-template <int D>
+// starts a line of three or more points if its predecessor along j lies
+// outside the grid and its second successor inside.  Lanes of a warp with the
+// same (direction, length) share one atomic; the order among lines of one
+// length is arbitrary and changes no result.  kUnit: all offsets in {-1, 0,
+// 1}, where both tests are masks of the components at or next to an end of
+// their axis.  The directions are staged in shared memory.
+template <int D, bool kUnit>
 __global__ void k_grid_starts(GridT<D> g, const GridDirT<D> *dirs, int nd,
-                              const long long *line_off, unsigned *hist, int cap, int phase,
-                              int *starts) {
-    extern __shared__ int soff[];  // nd x D offsets
-    for (int k = threadIdx.x; k < nd * D; k += blockDim.x) soff[k] = dirs[k / D].o[k % D];
+                              const long long *line_off, unsigned *cur, int cap, int *starts) {
+    extern __shared__ int soff[];  // kUnit: masks (pos, neg); else nd x D offsets
+    constexpr int kPer = kUnit ? 2 : D;
+    for (int k = threadIdx.x; k < nd * kPer; k += blockDim.x) {
+        const GridDirT<D> &d = dirs[k / kPer];
+        soff[k] = kUnit ? (int)(k & 1 ? d.neg : d.pos) : d.o[k % kPer];
+    }
     __syncthreads();
     const int lane = threadIdx.x & 31;
     for (long long b = (long long)blockIdx.x * blockDim.x; b < g.N;
@@ -332,62 +376,82 @@ __global__ void k_grid_starts(GridT<D> g, const GridDirT<D> *dirs, int nd,
         const long long p = b + threadIdx.x;
         const bool valid = p < g.N;
         int i[D];
-        if (valid) grid_index<D>(g, (int)p, i);
+        unsigned lo1 = 0, hi1 = 0, lo2 = 0, hi2 = 0;  // components at / within one of an end
+        if (valid) {
+            grid_index<D>(g, (int)p, i);
+#pragma unroll
+            for (int c = 0; c < D; ++c) {
+                lo1 |= i[c] < 1 ? 1u << c : 0u;
+                lo2 |= i[c] < 2 ? 1u << c : 0u;
+                hi1 |= i[c] > g.n[c] - 2 ? 1u << c : 0u;
+                hi2 |= i[c] > g.n[c] - 3 ? 1u << c : 0u;
+            }
+        }
         for (int j = 0; j < nd; ++j) {
             bool st = false;
             int len = 0;
-            if (valid) {
+            if (kUnit) {
+                const unsigned pos = (unsigned)soff[2 * j], neg = (unsigned)soff[2 * j + 1];
+                st = valid && ((lo1 & pos) | (hi1 & neg)) && !((hi2 & pos) | (lo2 & neg));
+                if (st) {
+                    len = 1 << 30;
+#pragma unroll
+                    for (int c = 0; c < D; ++c) {
+                        if ((pos >> c) & 1) len = min(len, g.n[c] - i[c]);
+                        if ((neg >> c) & 1) len = min(len, i[c] + 1);
+                    }
+                }
+            } else if (valid) {
 #pragma unroll
                 for (int c = 0; c < D; ++c) {
                     const int q = i[c] - soff[j * D + c];
                     st |= (q < 0) || (q >= g.n[c]);
                 }
                 if (st) len = line_length<D>(g, i, soff + j * D);
+                st = len >= 3;
             }
             const unsigned act = __ballot_sync(0xffffffffu, st);
             if (!st) continue;
             const unsigned grp = __match_any_sync(act, len);
             const int leader = __ffs(grp) - 1;
-            unsigned* cell = hist + (size_t)j * (cap + 1) + len;
             unsigned base = 0;
-            if (lane == leader) base = atomicAdd(cell, (unsigned)__popc(grp));
+            if (lane == leader)
+                base = atomicAdd(cur + (size_t)j * (cap + 1) + len, (unsigned)__popc(grp));
             base = __shfl_sync(grp, base, leader);
-            if (phase == 1)
-                starts[line_off[j] + base + __popc(grp & ((1u << lane) - 1))] = (int)p;
+            starts[line_off[j] + base + __popc(grp & ((1u << lane) - 1))] = (int)p;
         }
     }
 }
 
-// Per direction: the counts of lines of each length become the offsets of
-// their first line in the region, longest lines first.
-__global__ void k_grid_len_scan(int nd, int cap, unsigned *hist) {
-    const int j = blockIdx.x * blockDim.x + threadIdx.x;
-    if (j >= nd) return;
-    unsigned *h = hist + (size_t)j * (cap + 1);
-    unsigned acc = 0;
-    for (int len = cap; len >= 0; --len) {
-        const unsigned c = h[len];
-        h[len] = acc;
-        acc += c;
-    }
-}
-
-// One thread per (direction, line) of directions [j0, j1): Algorithm 1 on the
-// finite values of W_in along the line (stack in shared memory, layout
-// [slot][thread]), then every point of the line reads the hull there:
-//   a hull vertex keeps its own value (no split, S = 0);
+// One thread per (direction, line of three or more points) of directions
+// [j0, j1): Algorithm 1 on the finite values of W_in along the line (stack in
+// shared memory, layout [slot][thread]), then every interior point of the
+// line reads the hull there:
+//   a hull vertex keeps its own value (no split): H = inf;
 //   a point strictly between vertices a < x < b, with x_a, x_b taken relative
-//   to the point (x_a < 0 < x_b), records the numerator x_b w_a - x_a w_b of
-//   its chord value h = (x_b w_a - x_a w_b) / (x_b - x_a) in H and the pair
-//   (x_a, x_b) as two 16-bit fields in S.
+//   to the point (x_a < 0 < x_b), records the pair (x_a, x_b) as two 16-bit
+//   fields in S and in H a lower bound, in FP32, of its chord value
+//   h = (x_b w_a - x_a w_b) / (x_b - x_a); k_grid_reduce evaluates h in FP64
+//   where it can win.
 // Non-finite points keep their value.  H and S are chunk-major: entry
 // (j - j0) N + point.
+//
+// What bounds it is the FP64 pipe (2 lanes per SM and clock), so FP64 is left
+// to what decides: the difference to the top of the stack (one subtraction
+// per point, kept as the next comparison's) and, where the abscissae differ by
+// more than one step, products only when their FP32 values (truncated from the
+// bits on the integer pipe) are within rounding.  Each predicate has the value
+// of the FP64 one with every operation rounded on its own.
+// (All lines of one or more points, both differences and products in FP64,
+// FP64 chord numerators: the 648,025-point study took 167 us per step in this
+// kernel and 68 us in the reduction, the nine-dimensional one 13.7 and 2.0 ms;
+// now 113 and 48 us, 1.8 and 0.83 ms.)
 template <int D>
 __global__ void __launch_bounds__(128) k_grid_lines(GridT<D> g, const GridDirT<D> *dirs,
                                                     const long long *line_off, int j0, int j1,
-                                                    const int *starts, const double *Win,
-                                                    double *H, unsigned *S, int cap,
-                                                    const int *done) {
+                                                    const int *starts, const unsigned *cur,
+                                                    const double *Win, float *H, unsigned *S,
+                                                    int cap, const int *done) {
     if (done && *done) return;
     extern __shared__ double gsm[];
     const int T = blockDim.x;
@@ -399,80 +463,132 @@ __global__ void __launch_bounds__(128) k_grid_lines(GridT<D> g, const GridDirT<D
         if (line_off[mid] <= t) lo = mid;
         else hi = mid - 1;
     }
-    const int j = lo;
-    const GridDirT<D> d = dirs[j];
+    const int j = lo, step = dirs[j].step;
     const int p0 = starts[t];
-    int i0[D];
-    grid_index<D>(g, p0, i0);
-    const int len = line_length<D>(g, i0, d.o);
+    // the line's length: the largest with more than this line's rank of lines
+    const unsigned *cj = cur + (size_t)j * (cap + 1), rank = (unsigned)(t - line_off[j]);
+    lo = 3;
+    hi = cap;
+    while (lo < hi) {
+        const int mid = (lo + hi + 1) >> 1;
+        if (cj[mid] > rank) lo = mid;
+        else hi = mid - 1;
+    }
+    const int len = lo;
     double *sv = gsm + threadIdx.x;
     short *sx = reinterpret_cast<short *>(gsm + (size_t)cap * T) + threadIdx.x;
 
     // Algorithm 1: monotone chain over the finite values, pops while the top
-    // of the stack is not strictly below the chord to the new point
-    int k = 0;
+    // of the stack is not strictly below the chord to the new point.  The two
+    // top vertices p, q and A = w_q - w_p are kept in registers.
+    int k = 0, xp = 0, xq = 0;
+    double wp = 0.0, wq = 0.0, A = 0.0;
+    bool holes = false;
+    const double *src = Win + p0;
+    double wn = src[0];
     for (int l = 0; l < len; ++l) {
-        const double w = Win[p0 + l * d.step];
-        if (!finite_bits(w)) continue;
-        while (k >= 2) {
-            const double wp = sv[(k - 2) * T], wq = sv[(k - 1) * T];
-            const int xp = sx[(k - 2) * T], xq = sx[(k - 1) * T];
-            const double A = __dsub_rn(wq, wp), B = __dsub_rn(w, wq);
-            const int di = l - xq, dp = xq - xp;
-            // multiplying by 1 is exact: skip it
-            const double lhs = di == 1 ? A : __dmul_rn(A, exact_double(di));
-            const double rhs = dp == 1 ? B : __dmul_rn(B, exact_double(dp));
-            if (order_key(lhs) >= order_key(rhs)) --k;
-            else break;
+        const double w = wn;
+        if (l + 1 < len) wn = src[(long long)(l + 1) * step];
+        if (!finite_bits(w)) {
+            holes = true;
+            continue;
         }
+        double B = 0.0;
+        while (k >= 1) {
+            B = __dsub_rn(w, wq);
+            if (k == 1) break;
+            const int di = l - xq, dp = xq - xp;
+            bool pop;
+            if (di == 1 && dp == 1) {  // multiplying by 1 is exact
+                pop = order_key(A) >= order_key(B);
+            } else {
+                const float fa = trunc32(A) * (float)di, fb = trunc32(B) * (float)dp;
+                const float d = fa - fb, e = 1e-6f * (fabsf(fa) + fabsf(fb)) + 1e-30f;
+                if (fabsf(d) > e && e < 1e30f) {
+                    pop = d > 0.0f;
+                } else {
+                    const double lhs = di == 1 ? A : __dmul_rn(A, exact_double(di));
+                    const double rhs = dp == 1 ? B : __dmul_rn(B, exact_double(dp));
+                    pop = order_key(lhs) >= order_key(rhs);
+                }
+            }
+            if (!pop) break;
+            --k;
+            wq = wp;
+            xq = xp;
+            if (k >= 2) {
+                wp = sv[(k - 2) * T];
+                xp = sx[(k - 2) * T];
+                A = __dsub_rn(wq, wp);
+            }
+        }
+        wp = wq;
+        xp = xq;
+        A = B;
+        wq = w;
+        xq = l;
         sv[k * T] = w;
         sx[k * T] = (short)l;
         ++k;
     }
     // every finite point lies between the first and the last vertex
-    const long long base = (long long)(j - j0) * g.N;
-    int e = 0;
-    for (int l = 0; l < len; ++l) {
-        const int idx = p0 + l * d.step;
-        double num = 0.0;
-        unsigned sp = 0;
-        if (k > 1) {
-            while (e + 2 < k && sx[(e + 1) * T] <= l) ++e;
-            const int xa = sx[e * T], xb = sx[(e + 1) * T];
-            // strictly inside the edge (and finite: a non-finite point is no
-            // vertex, but a hole can lie inside an edge)
-            if (xa < l && l < xb && finite_bits(Win[idx])) {
-                const int ra = xa - l, rb = xb - l;
-                num = __dsub_rn(__dmul_rn(exact_double(rb), sv[e * T]),
-                                __dmul_rn(exact_double(ra), sv[(e + 1) * T]));
-                sp = ((unsigned)ra & 0xffffu) | ((unsigned)rb << 16);
+    const long long base = (long long)(j - j0) * g.N + p0;
+    int e = -1, xa = 0, xb = -1;  // the current edge
+    float fa = 0.0f, slope = 0.0f, off = 0.0f;
+    for (int l = 1; l < len - 1; ++l) {
+        while (l >= xb && e + 2 < k) {
+            ++e;
+            xa = sx[e * T];
+            xb = sx[(e + 1) * T];
+            fa = trunc32(sv[e * T]);
+            const float fb = trunc32(sv[(e + 1) * T]);
+            // the bound covers the truncation of both ends and the rounding of
+            // the chord; ends outside FP32's range leave it to the FP64 value
+            off = 1e-6f * (fabsf(fa) + fabsf(fb)) + 1e-36f;
+            slope = __fdividef(fb - fa, (float)(xb - xa));
+            if (!(off < 1e30f)) {
+                fa = -INFINITY;
+                slope = off = 0.0f;
             }
         }
-        H[base + idx] = num;
-        S[base + idx] = sp;
+        const long long at = base + (long long)l * step;
+        float h = INFINITY;
+        // strictly inside the edge (and finite: a non-finite point is no
+        // vertex, but a hole can lie inside an edge)
+        if (xa < l && l < xb && (!holes || finite_bits(src[(long long)l * step]))) {
+            h = __fmaf_rn(slope, (float)(l - xa), fa) - off;
+            S[at] = ((unsigned)(xa - l) & 0xffffu) | ((unsigned)(xb - l) << 16);
+        }
+        H[at] = h;
     }
 }
 
-// rcp[v] = fl(1 / v), v = 1 .. 2 kGridMaxLine (the chord denominators).
-__global__ void k_grid_rcp(double *rcp) {
-    const int v = blockIdx.x * blockDim.x + threadIdx.x;
-    if (v <= 2 * kGridMaxLine) rcp[v] = v ? __drcp_rn((double)v) : 0.0;
-}
+constexpr int kGridChunkDirs = 64;  // directions per chunk at most (a mask word in the reduction)
 
-// Per point, directions [j0, j1) in order: the first strict decrease below
-// the best so far wins (first chunk: the best so far is W_in itself, no
-// split).  The chord value h = fl(num / den) is needed only where it can win:
-// q = fl(num fl(1/den)) is within 3.4e-16 |q| of h, so fl(q (1 -+ 5e-16)) is
-// a lower bound of h and a direction whose bound is not below the best so far
-// cannot win; the others are divided exactly and compared.  lam = (dir, l-,
-// l+) per point (dir = -1: no split).  The last chunk adds the point's
-// decrease W_in - W_out to the step's maximum (dec, as the bits of a
-// non-negative double).
-__global__ void k_grid_reduce(int N, int j0, int j1, int first, int last, const double *Win,
-                              const double *H, const unsigned *S, const double *rcp,
-                              double *Wout, int *lam, unsigned long long *dec, const int *done) {
+// Per point, directions [j0, j1): the smallest chord value h below the best so
+// far wins, the lowest direction on equal values (first chunk: the best so far
+// is W_in itself, no split).  The FP32 lower bounds of the interior
+// directions are read, the direction with the smallest one is evaluated in
+// FP64, then those whose bound does not exceed its value: every lane its own
+// next one, so that a warp evaluates as often as its busiest lane needs (once
+// or twice), not once per direction.  lam = (dir, l-, l+) per point (dir =
+// -1: no split).  The last chunk adds the point's decrease W_in - W_out to
+// the step's maximum (dec, as the bits of a non-negative double).
+template <int D, bool kUnit>
+__global__ void __launch_bounds__(256) k_grid_reduce(GridT<D> g, const GridDirT<D> *dirs, int j0,
+                                                     int j1, int first, int last, const double *Win,
+                                                     const float *H, const unsigned *S, double *Wout,
+                                                     int *lam, unsigned long long *dec,
+                                                     const int *done) {
     if (done && *done) return;
-    const int p = blockIdx.x * blockDim.x + threadIdx.x;
+    __shared__ GridDirT<D> s_d[kGridChunkDirs];
+    __shared__ unsigned s_nz[kGridChunkDirs];  // components that the direction moves
+    const int n = j1 - j0;
+    for (int k = threadIdx.x; k < n * (int)(sizeof(GridDirT<D>) / 4); k += blockDim.x)
+        reinterpret_cast<int *>(s_d)[k] = reinterpret_cast<const int *>(dirs + j0)[k];
+    if (threadIdx.x < n) s_nz[threadIdx.x] = dirs[j0 + threadIdx.x].pos | dirs[j0 + threadIdx.x].neg;
+    __syncthreads();
+    const long long N = g.N, p = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     unsigned long long dbits = 0;
     if (p < N) {
         const double w0 = Win[p];
@@ -484,25 +600,61 @@ __global__ void k_grid_reduce(int N, int j0, int j1, int first, int last, const 
             bm = lam[3 * p + 1];
             bp = lam[3 * p + 2];
         }
-        for (int j = j0; j < j1; ++j) {
-            const long long e = (long long)(j - j0) * N + p;
-            const unsigned s = S[e];
-            if (s) {
-                const double num = H[e];
-                const int ra = (int)(short)(s & 0xffffu), rb = (int)(s >> 16);
-                const double q = __dmul_rn(num, rcp[rb - ra]);
-                const double lb =
-                    __dmul_rn(q, __double_as_longlong(q) < 0 ? 1.0 + 5e-16 : 1.0 - 5e-16);
-                if (order_key(lb) < order_key(best)) {
-                    const double h = __ddiv_rn(num, exact_double(rb - ra));
-                    if (order_key(h) < order_key(best)) {
-                        best = h;
-                        bd = j;
-                        bm = ra;
-                        bp = rb;
-                    }
+        int i[D], mg[D];  // grid points between the point and the nearer end of each axis
+        unsigned edge = 0;
+        grid_index<D>(g, (int)p, i);
+#pragma unroll
+        for (int c = 0; c < D; ++c) {
+            mg[c] = min(i[c], g.n[c] - 1 - i[c]);
+            edge |= mg[c] < 1 ? 1u << c : 0u;
+        }
+        auto interior = [&](int q) {
+            if (kUnit) return !(edge & s_nz[q]);
+            bool in = true;
+#pragma unroll
+            for (int c = 0; c < D; ++c) in = in && mg[c] >= abs(s_d[q].o[c]);
+            return in;
+        };
+        // the exact chord value of direction j0 + q
+        auto exact = [&](int q) {
+            const unsigned sp = S[q * N + p];
+            const int ra = (int)(short)(sp & 0xffffu), rb = (int)(sp >> 16), st = s_d[q].step;
+            const double wa = Win[p + (long long)ra * st], wb = Win[p + (long long)rb * st];
+            const double num = __dsub_rn(__dmul_rn(exact_double(rb), wa),
+                                         __dmul_rn(exact_double(ra), wb));
+            const double h = __ddiv_rn(num, exact_double(rb - ra));
+            const long long kh = order_key(h), kb = order_key(best);
+            if (kh < kb || (kh == kb && j0 + q < bd)) {
+                best = h;
+                bd = j0 + q;
+                bm = ra;
+                bp = rb;
+            }
+        };
+        if (finite_bits(w0)) {
+            float m1 = INFINITY, m2 = INFINITY;  // the two smallest bounds
+            int q1 = 0;
+#pragma unroll 4
+            for (int q = 0; q < n; ++q) {
+                if (!interior(q)) continue;
+                const float h = H[q * N + p];
+                m2 = fminf(m2, fmaxf(m1, h));
+                if (h < m1) {
+                    m1 = h;
+                    q1 = q;
                 }
             }
+            if (m1 < INFINITY && m1 <= __double2float_ru(best)) exact(q1);
+            float lim = __double2float_ru(best);
+            unsigned long long more = 0;
+            if (m2 < INFINITY && m2 <= lim) {
+                for (int q = 0; q < n; ++q)
+                    if (q != q1 && interior(q)) {
+                        const float h = H[q * N + p];
+                        if (h < INFINITY && h <= lim) more |= 1ull << q;
+                    }
+            }
+            for (; more; more &= more - 1) exact(__ffsll((long long)more) - 1);
         }
         Wout[p] = best;
         lam[3 * p] = bd;
@@ -853,14 +1005,14 @@ int check_dirs(int nd, const int32_t *off, const GridT<D> &gd, std::vector<GridD
     for (int j = 0; j < nd; ++j) {
         GridDirT<D> g{};
         bool nz = false;
-        long long inside = 1;  // points whose predecessor lies in the grid
         for (int c = 0; c < D; ++c) {
             const int o = off[D * j + c];
             if (o < -kGridMaxLine || o > kGridMaxLine)
                 return fail(CVX_ERR_INVALID_ARG, "direction %d: offset out of range", j);
             g.o[c] = o;
             nz |= o != 0;
-            inside *= std::max(0, gd.n[c] - std::abs(o));
+            if (o > 0) g.pos |= 1u << c;
+            if (o < 0) g.neg |= 1u << c;
         }
         if (!nz) return fail(CVX_ERR_INVALID_ARG, "direction %d is zero", j);
         // rank one: every 2x2 minor of the d x d offset matrix vanishes
@@ -875,7 +1027,7 @@ int check_dirs(int nd, const int32_t *off, const GridT<D> &gd, std::vector<GridD
         for (int c = 0; c < D; ++c) step += (long long)g.o[c] * gd.s[c];
         g.step = (int)step;
         dirs[j] = g;
-        line_off[j + 1] = line_off[j] + (gd.N - inside);
+        line_off[j + 1] = line_off[j] + lines_of<D>(gd, g, 3);
     }
     return CVX_OK;
 }
@@ -885,43 +1037,45 @@ template <int D>
 struct GridWork {
     GridDirT<D> *dirs;
     long long *line_off;
-    unsigned *hist;  // nd x (longest line + 1): line counts, then offsets, by length
+    unsigned *cur;  // nd x (longest line + 1): line counts by length (k_grid_cursors)
     int *starts;
-    double *H;
+    float *H;
     unsigned *S;
-    double *rcp;
     int chunk;  // directions per chunk
+    bool unit;  // all offsets in {-1, 0, 1}
 };
 
 template <int D>
 size_t grid_work_bytes(int nd, const GridT<D> &gd, long long lines, int &chunk) {
-    const size_t per_dir = (size_t)gd.N * (sizeof(double) + sizeof(unsigned));
-    chunk = (int)std::max<size_t>(1, std::min<size_t>(nd, grid_chunk_bytes() / per_dir));
+    const size_t per_dir = (size_t)gd.N * (sizeof(float) + sizeof(unsigned));
+    chunk = (int)std::max<size_t>(
+        1, std::min<size_t>(std::min(nd, kGridChunkDirs), grid_chunk_bytes() / per_dir));
     return up256(sizeof(GridDirT<D>) * nd) + up256(sizeof(long long) * (nd + 1)) +
            up256(sizeof(unsigned) * nd * (size_t)(kGridMaxLine + 1)) +
            up256(sizeof(int) * (size_t)lines) +
-           up256(sizeof(double) * (size_t)chunk * gd.N) +
-           up256(sizeof(unsigned) * (size_t)chunk * gd.N) +
-           up256(sizeof(double) * (2 * kGridMaxLine + 1));
+           up256(sizeof(float) * (size_t)chunk * gd.N) +
+           up256(sizeof(unsigned) * (size_t)chunk * gd.N);
 }
 
 template <int D>
-void carve_grid_work(char *ws, int nd, const GridT<D> &gd, long long lines, int chunk,
-                     GridWork<D> &w) {
+void carve_grid_work(char *ws, const std::vector<GridDirT<D>> &dirs, const GridT<D> &gd,
+                     long long lines, int chunk, GridWork<D> &w) {
+    const int nd = (int)dirs.size();
     w.dirs = (GridDirT<D> *)ws;
     ws += up256(sizeof(GridDirT<D>) * nd);
     w.line_off = (long long *)ws;
     ws += up256(sizeof(long long) * (nd + 1));
-    w.hist = (unsigned *)ws;
+    w.cur = (unsigned *)ws;
     ws += up256(sizeof(unsigned) * nd * (size_t)(kGridMaxLine + 1));
     w.starts = (int *)ws;
     ws += up256(sizeof(int) * (size_t)lines);
-    w.H = (double *)ws;
-    ws += up256(sizeof(double) * (size_t)chunk * gd.N);
+    w.H = (float *)ws;
+    ws += up256(sizeof(float) * (size_t)chunk * gd.N);
     w.S = (unsigned *)ws;
-    ws += up256(sizeof(unsigned) * (size_t)chunk * gd.N);
-    w.rcp = (double *)ws;
     w.chunk = chunk;
+    w.unit = true;
+    for (const GridDirT<D> &d : dirs)
+        for (int c = 0; c < D; ++c) w.unit = w.unit && std::abs(d.o[c]) <= 1;
 }
 
 template <int D>
@@ -934,7 +1088,7 @@ int grid_line_cap(const GridT<D> &gd) {
 // Threads per line-kernel CTA so that the stacks fit in shared memory.
 int grid_line_threads(int cap) { return cap <= 128 ? 128 : (cap <= 256 ? 64 : 32); }
 
-// Direction table, line regions, line starts and the reciprocal table.
+// Direction table, line regions and line starts.
 template <int D>
 int grid_setup(const GridT<D> &gd, const std::vector<GridDirT<D>> &dirs,
                const std::vector<long long> &line_off, const GridWork<D> &w, cudaStream_t s) {
@@ -944,21 +1098,17 @@ int grid_setup(const GridT<D> &gd, const std::vector<GridDirT<D>> &dirs,
     CK(cudaMemcpyAsync(w.line_off, line_off.data(), sizeof(long long) * (nd + 1),
                        cudaMemcpyHostToDevice, s),
        "grid setup");
+    if (line_off[nd] == 0) return CVX_OK;
     const int cap = grid_line_cap<D>(gd);
-    CK(cudaMemsetAsync(w.hist, 0, sizeof(unsigned) * nd * (size_t)(cap + 1), s), "grid setup");
-    const size_t smem = sizeof(int) * (size_t)nd * D;
-    CK(cudaFuncSetAttribute(k_grid_starts<D>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                            (int)smem),
+    k_grid_cursors<D><<<(nd * (cap + 1) + 127) / 128, 128, 0, s>>>(gd, w.dirs, nd, cap, w.cur);
+    CK(cudaGetLastError(), "grid line counts");
+    auto ks = w.unit ? k_grid_starts<D, true> : k_grid_starts<D, false>;
+    const size_t smem = sizeof(int) * (size_t)nd * (w.unit ? 2 : D);
+    CK(cudaFuncSetAttribute(ks, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem),
        "grid line starts shared memory");
     const int bx = (int)std::min<long long>((gd.N + 255) / 256, 4096);
-    k_grid_starts<D><<<bx, 256, smem, s>>>(gd, w.dirs, nd, w.line_off, w.hist, cap, 0, w.starts);
-    CK(cudaGetLastError(), "grid line counts");
-    k_grid_len_scan<<<(nd + 127) / 128, 128, 0, s>>>(nd, cap, w.hist);
-    CK(cudaGetLastError(), "grid line offsets");
-    k_grid_starts<D><<<bx, 256, smem, s>>>(gd, w.dirs, nd, w.line_off, w.hist, cap, 1, w.starts);
+    ks<<<bx, 256, smem, s>>>(gd, w.dirs, nd, w.line_off, w.cur, cap, w.starts);
     CK(cudaGetLastError(), "grid line starts");
-    k_grid_rcp<<<(2 * kGridMaxLine + 256) / 256, 256, 0, s>>>(w.rcp);
-    CK(cudaGetLastError(), "grid reciprocal table");
     return CVX_OK;
 }
 
@@ -979,12 +1129,13 @@ int grid_enqueue_step(const GridT<D> &gd, int nd, const std::vector<long long> &
             if (rc) return rc;
             if (!ev.empty()) CK(cudaEventRecord(ev[0], s), "grid profiling");
             k_grid_lines<D><<<(unsigned)((lines + T - 1) / T), T, smem, s>>>(
-                gd, w.dirs, w.line_off, j0, j1, w.starts, Win, w.H, w.S, cap, done);
+                gd, w.dirs, w.line_off, j0, j1, w.starts, w.cur, Win, w.H, w.S, cap, done);
             CK(cudaGetLastError(), "grid line kernel");
             if (!ev.empty()) CK(cudaEventRecord(ev[1], s), "grid profiling");
         }
-        k_grid_reduce<<<(gd.N + 255) / 256, 256, 0, s>>>(gd.N, j0, j1, j0 == 0, j1 == nd, Win,
-                                                         w.H, w.S, w.rcp, Wout, lam, dec, done);
+        auto kr = w.unit ? k_grid_reduce<D, true> : k_grid_reduce<D, false>;
+        kr<<<(unsigned)((gd.N + 255LL) / 256), 256, 0, s>>>(gd, w.dirs, j0, j1, j0 == 0, j1 == nd,
+                                                            Win, w.H, w.S, Wout, lam, dec, done);
         CK(cudaGetLastError(), "grid reduce kernel");
     }
     return CVX_OK;
@@ -1050,7 +1201,7 @@ int grid_step_t(cvx_handle *h, const cvx_grid *g, int32_t nd, const int32_t *off
     rc = ensure_ws(h, bytes, s);
     if (rc) return rc;
     GridWork<D> w;
-    carve_grid_work<D>(h->ws, nd, gd, lines, chunk, w);
+    carve_grid_work<D>(h->ws, dirs, gd, lines, chunk, w);
     int *lam_w = lam ? lam : (int *)(h->ws + lam_off);
     const int cap = grid_line_cap<D>(gd);
     rc = set_line_smem<D>(cap);
@@ -1093,7 +1244,7 @@ int grid_convexify_t(cvx_handle *h, const cvx_params *p, const cvx_grid *g, doub
     rc = ensure_ws(h, bytes, s);
     if (rc) return rc;
     GridWork<D> w;
-    carve_grid_work<D>(h->ws, nd, gd, lines, chunk, w);
+    carve_grid_work<D>(h->ws, dirs, gd, lines, chunk, w);
     double *pong = (double *)(h->ws + o_pong);
     unsigned long long *dk =
         reinterpret_cast<unsigned long long *>(decs ? decs : (double *)(h->ws + o_dec));
