@@ -103,6 +103,21 @@ __device__ __forceinline__ float trunc32(double x) {
     return __int_as_float(b | (hi & 0x80000000));
 }
 
+// num / den for a positive integer den, y = fl(1 / den): the correctly rounded
+// quotient in five operations.  fl(num y) is within two units in the last
+// place, the first correction (residual exact by FMA) makes it faithful, and
+// Markstein's theorem (a faithful quotient corrected with the correctly
+// rounded reciprocal rounds correctly) the second exact.  Outside the exponent
+// range where no intermediate over- or underflows: the division.
+__device__ __forceinline__ double quotient(double num, int den, double y) {
+    const int e = (__double2hiint(num) >> 20) & 0x7ff;
+    const double b = exact_double(den);
+    if (e < 128 || e > 1900) return __ddiv_rn(num, b);
+    double q = __dmul_rn(num, y);
+    q = __fma_rn(__fma_rn(-q, b, num), y, q);
+    return __fma_rn(__fma_rn(-q, b, num), y, q);
+}
+
 template <int D>
 __device__ __forceinline__ void grid_index(const GridT<D> &g, int idx, int *i) {
 #pragma unroll
@@ -131,7 +146,8 @@ __device__ __forceinline__ double w_of_psi0(double s, double beta, double ek, co
 // Invariants of C = F^T F (Sec. 2) for F in R^{dxd}, D = d^2, row-major:
 // I1 = tr C, I2 = the sum of the principal 2x2 minors of C, J = det F; d = 2
 // is plane strain (C33 = 1: I1 gains 1, I2 gains C11 + C22).
-template <int D>
+// kAll false: I1 and J only.
+template <int D, bool kAll>
 __device__ void invariants(const double *F, double &I1, double &I2, double &J, double *C) {
     if (D == 4) {
         C[0] = F[0] * F[0] + F[2] * F[2];
@@ -139,15 +155,16 @@ __device__ void invariants(const double *F, double &I1, double &I2, double &J, d
         C[2] = C[1];
         C[3] = F[1] * F[1] + F[3] * F[3];
         I1 = C[0] + C[3] + 1.0;
-        I2 = (C[0] * C[3] - C[1] * C[1]) + C[0] + C[3];
+        if (kAll) I2 = (C[0] * C[3] - C[1] * C[1]) + C[0] + C[3];
         J = __dsub_rn(__dmul_rn(F[0], F[3]), __dmul_rn(F[1], F[2]));
     } else {
         for (int a = 0; a < 3; ++a)
             for (int b = 0; b < 3; ++b)
                 C[3 * a + b] = F[a] * F[b] + F[3 + a] * F[3 + b] + F[6 + a] * F[6 + b];
         I1 = C[0] + C[4] + C[8];
-        I2 = (C[0] * C[4] - C[1] * C[3]) + (C[0] * C[8] - C[2] * C[6]) +
-             (C[4] * C[8] - C[5] * C[7]);
+        if (kAll)
+            I2 = (C[0] * C[4] - C[1] * C[3]) + (C[0] * C[8] - C[2] * C[6]) +
+                 (C[4] * C[8] - C[5] * C[7]);
         // each operation rounded on its own, in the oracle's order: which
         // points count as det F <= 0 must not depend on FMA contraction
         const double m0 = __dsub_rn(__dmul_rn(F[4], F[8]), __dmul_rn(F[5], F[7]));
@@ -163,12 +180,14 @@ __device__ void invariants(const double *F, double &I1, double &I2, double &J, d
 template <int D>
 __device__ bool psi0_grid(const double *F, const Material &m, int rule, double &s, double &J,
                           double &I1, double *C) {
-    double I2;
-    invariants<D>(F, I1, I2, J, C);
     if (m.energy == CVX_ENERGY_STVK_DAMAGE) {
+        double I2;
+        invariants<D, true>(F, I1, I2, J, C);
         s = m.lam / 8.0 * (I1 - 3.0) * (I1 - 3.0) + m.mu / 4.0 * (I1 * I1 - 2.0 * I1 - 2.0 * I2 + 3.0);
         return rule == 0 && !(J > 0.0);
     }
+    double I2;
+    invariants<D, false>(F, I1, I2, J, C);
     const double aj = fabs(J);
     const double lj = log(aj);
     s = 0.5 * m.mu * (I1 - 3.0) - m.mu * lj + 0.5 * m.lam * lj * lj;
@@ -321,15 +340,21 @@ __global__ void __launch_bounds__(256) k_grid_energy(GridT<D> g, Material m, dou
     W[p] = w;
 }
 
-// Lines.  Only lines of three points or more matter: the ends of a line are
-// vertices of its hull, so a point can split along a direction only if both
-// its neighbours along it lie in the grid ("interior" below).  In nine
-// dimensions with three values per off-diagonal component that leaves a few
-// directions per point of the 169.
+// Lines.  The ends of a line are vertices of its hull, so a point can split
+// along a direction only if both its neighbours along it lie in the grid
+// ("interior" below).  In nine dimensions with three values per off-diagonal
+// component that leaves 15 of the 169 directions per point on average, nearly
+// all of them lines of three points, whose one chord k_grid_reduce takes
+// itself there; the lines listed and walked are those of kMinLine points or
+// more.
 //
 // The number of lines of m or more points of a direction o is
 // C(m) - C(m + 1), C(m) = prod_c max(0, n_c - (m - 1) |o_c|) (the points whose
 // (m - 1)-fold successor lies in the grid).
+// Points of the shortest line that is listed.
+template <int D>
+constexpr int kMinLine = D == 4 ? 3 : 4;
+
 template <int D>
 __host__ __device__ inline long long lines_of(const GridT<D> &g, const GridDirT<D> &d, int m) {
     long long a = 1, b = 1;
@@ -354,8 +379,8 @@ __global__ void k_grid_cursors(GridT<D> g, const GridDirT<D> *dirs, int nd, int 
 }
 
 // Line starts: per point (one index decomposition) and direction j, the point
-// starts a line of three or more points if its predecessor along j lies
-// outside the grid and its second successor inside.  Lanes of a warp with the
+// starts a line of kMinLine or more points if its predecessor along j lies
+// outside the grid and its (kMinLine - 1)-th successor inside.  Lanes of a warp with the
 // same (direction, length) share one atomic; the order among lines of one
 // length is arbitrary and changes no result.  kUnit: all offsets in {-1, 0,
 // 1}, where both tests are masks of the components at or next to an end of
@@ -376,15 +401,15 @@ __global__ void k_grid_starts(GridT<D> g, const GridDirT<D> *dirs, int nd,
         const long long p = b + threadIdx.x;
         const bool valid = p < g.N;
         int i[D];
-        unsigned lo1 = 0, hi1 = 0, lo2 = 0, hi2 = 0;  // components at / within one of an end
+        unsigned lo1 = 0, hi1 = 0, lom = 0, him = 0;  // components at / too near an end
         if (valid) {
             grid_index<D>(g, (int)p, i);
 #pragma unroll
             for (int c = 0; c < D; ++c) {
                 lo1 |= i[c] < 1 ? 1u << c : 0u;
-                lo2 |= i[c] < 2 ? 1u << c : 0u;
+                lom |= i[c] < kMinLine<D> - 1 ? 1u << c : 0u;
                 hi1 |= i[c] > g.n[c] - 2 ? 1u << c : 0u;
-                hi2 |= i[c] > g.n[c] - 3 ? 1u << c : 0u;
+                him |= i[c] > g.n[c] - kMinLine<D> ? 1u << c : 0u;
             }
         }
         for (int j = 0; j < nd; ++j) {
@@ -392,7 +417,7 @@ __global__ void k_grid_starts(GridT<D> g, const GridDirT<D> *dirs, int nd,
             int len = 0;
             if (kUnit) {
                 const unsigned pos = (unsigned)soff[2 * j], neg = (unsigned)soff[2 * j + 1];
-                st = valid && ((lo1 & pos) | (hi1 & neg)) && !((hi2 & pos) | (lo2 & neg));
+                st = valid && ((lo1 & pos) | (hi1 & neg)) && !((him & pos) | (lom & neg));
                 if (st) {
                     len = 1 << 30;
 #pragma unroll
@@ -408,7 +433,7 @@ __global__ void k_grid_starts(GridT<D> g, const GridDirT<D> *dirs, int nd,
                     st |= (q < 0) || (q >= g.n[c]);
                 }
                 if (st) len = line_length<D>(g, i, soff + j * D);
-                st = len >= 3;
+                st = len >= kMinLine<D>;
             }
             const unsigned act = __ballot_sync(0xffffffffu, st);
             if (!st) continue;
@@ -423,7 +448,7 @@ __global__ void k_grid_starts(GridT<D> g, const GridDirT<D> *dirs, int nd,
     }
 }
 
-// One thread per (direction, line of three or more points) of directions
+// One thread per (direction, line of kMinLine or more points) of directions
 // [j0, j1): Algorithm 1 on the finite values of W_in along the line (stack in
 // shared memory, layout [slot][thread]), then every interior point of the
 // line reads the hull there:
@@ -436,16 +461,17 @@ __global__ void k_grid_starts(GridT<D> g, const GridDirT<D> *dirs, int nd,
 // Non-finite points keep their value.  H and S are chunk-major: entry
 // (j - j0) N + point.
 //
-// What bounds it is the FP64 pipe (2 lanes per SM and clock), so FP64 is left
-// to what decides: the difference to the top of the stack (one subtraction
-// per point, kept as the next comparison's) and, where the abscissae differ by
-// more than one step, products only when their FP32 values (truncated from the
-// bits on the integer pipe) are within rounding.  Each predicate has the value
-// of the FP64 one with every operation rounded on its own.
+// The FP64 pipe has 2 lanes per SM and clock, so FP64 is left to what decides:
+// a comparison takes FP32 values (truncated from the bits on the integer
+// pipe), and FP64 where those are within their error.  Each predicate has the
+// value of the FP64 one with every operation rounded on its own.  The stack
+// holds abscissae only; its values are read again from W_in.
 // (All lines of one or more points, both differences and products in FP64,
-// FP64 chord numerators: the 648,025-point study took 167 us per step in this
-// kernel and 68 us in the reduction, the nine-dimensional one 13.7 and 2.0 ms;
-// now 113 and 48 us, 1.8 and 0.83 ms.)
+// FP64 chord numerators of every point and direction read back by the
+// reduction: the 648,025-point study took 167 us per step here and 68 us in
+// the reduction, the nine-dimensional one 13.7 and 2.0 ms; now 103 and 42 us,
+// 0.10 and 0.90 ms.  A loop that pops or pushes once per turn took 121 us, and
+// values kept in the stack 113 us at a third of the resident warps.)
 template <int D>
 __global__ void __launch_bounds__(128) k_grid_lines(GridT<D> g, const GridDirT<D> *dirs,
                                                     const long long *line_off, int j0, int j1,
@@ -453,38 +479,46 @@ __global__ void __launch_bounds__(128) k_grid_lines(GridT<D> g, const GridDirT<D
                                                     const double *Win, float *H, unsigned *S,
                                                     int cap, const int *done) {
     if (done && *done) return;
-    extern __shared__ double gsm[];
-    const int T = blockDim.x;
-    const long long t = line_off[j0] + (long long)blockIdx.x * T + threadIdx.x;
-    if (t >= line_off[j1]) return;
-    int lo = j0, hi = j1 - 1;  // the region holding t
-    while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        if (line_off[mid] <= t) lo = mid;
-        else hi = mid - 1;
+    extern __shared__ short gsm[];
+    const int T = blockDim.x, lane = threadIdx.x & 31;
+    const long long end = line_off[j1];
+    const long long t0 = line_off[j0] + (long long)blockIdx.x * T + (threadIdx.x & ~31), t = t0 + lane;
+    if (t0 >= end) return;  // whole warps only: the search below is warp-wide
+    // the direction of the warp's first line, and that line's length: the
+    // largest with more than its rank of lines
+    int j = j0;
+    for (int b = j0 + 1; b < j1; b += 32)
+        j += __popc(__ballot_sync(0xffffffffu, b + lane < j1 && line_off[b + lane] <= t0));
+    const unsigned rank0 = (unsigned)(t0 - line_off[j]);
+    int len = kMinLine<D> - 1;
+    for (int b = kMinLine<D>; b <= cap; b += 32) {
+        const unsigned m = __ballot_sync(0xffffffffu, b + lane <= cap &&
+                                                          cur[(size_t)j * (cap + 1) + b + lane] > rank0);
+        len += __popc(m);
+        if (m != 0xffffffffu) break;
     }
-    const int j = lo, step = dirs[j].step;
+    if (t >= end) return;
+    while (t >= line_off[j + 1]) {  // later lines of the warp: next directions ...
+        ++j;
+        len = cap;
+    }
+    {  // ... and shorter lines
+        const unsigned *cj = cur + (size_t)j * (cap + 1), rank = (unsigned)(t - line_off[j]);
+        while (cj[len] <= rank) --len;
+    }
+    const int step = dirs[j].step;
     const int p0 = starts[t];
-    // the line's length: the largest with more than this line's rank of lines
-    const unsigned *cj = cur + (size_t)j * (cap + 1), rank = (unsigned)(t - line_off[j]);
-    lo = 3;
-    hi = cap;
-    while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        if (cj[mid] > rank) lo = mid;
-        else hi = mid - 1;
-    }
-    const int len = lo;
-    double *sv = gsm + threadIdx.x;
-    short *sx = reinterpret_cast<short *>(gsm + (size_t)cap * T) + threadIdx.x;
+    const double *src = Win + p0;
+    const long long base = (long long)(j - j0) * g.N + p0;
+    short *sx = gsm + threadIdx.x;
 
     // Algorithm 1: monotone chain over the finite values, pops while the top
     // of the stack is not strictly below the chord to the new point.  The two
-    // top vertices p, q and A = w_q - w_p are kept in registers.
+    // top vertices p, q are kept in registers, their values also in FP32 (P, Q).
     int k = 0, xp = 0, xq = 0;
-    double wp = 0.0, wq = 0.0, A = 0.0;
+    double wp = 0.0, wq = 0.0;
+    float P = 0.0f, Q = 0.0f;
     bool holes = false;
-    const double *src = Win + p0;
     double wn = src[0];
     for (int l = 0; l < len; ++l) {
         const double w = wn;
@@ -493,46 +527,45 @@ __global__ void __launch_bounds__(128) k_grid_lines(GridT<D> g, const GridDirT<D
             holes = true;
             continue;
         }
-        double B = 0.0;
-        while (k >= 1) {
-            B = __dsub_rn(w, wq);
-            if (k == 1) break;
+        const float V = trunc32(w);
+        while (k >= 2) {
+            // (w_q - w_p)(x - x_q) >= (w - w_q)(x_q - x_p)?  The FP32 values
+            // decide where their error (2^-23 of each value) allows
             const int di = l - xq, dp = xq - xp;
+            const float fi = (float)di, fp = (float)dp;
+            const float d = (Q - P) * fi - (V - Q) * fp;
+            const float mag = fabsf(P) + fabsf(Q) + fabsf(V);
             bool pop;
-            if (di == 1 && dp == 1) {  // multiplying by 1 is exact
-                pop = order_key(A) >= order_key(B);
+            if (fabsf(d) > 4e-7f * mag * (fi + fp) && mag < 1e30f && mag > 1e-20f) {
+                pop = d > 0.0f;
             } else {
-                const float fa = trunc32(A) * (float)di, fb = trunc32(B) * (float)dp;
-                const float d = fa - fb, e = 1e-6f * (fabsf(fa) + fabsf(fb)) + 1e-30f;
-                if (fabsf(d) > e && e < 1e30f) {
-                    pop = d > 0.0f;
-                } else {
-                    const double lhs = di == 1 ? A : __dmul_rn(A, exact_double(di));
-                    const double rhs = dp == 1 ? B : __dmul_rn(B, exact_double(dp));
-                    pop = order_key(lhs) >= order_key(rhs);
-                }
+                const double A = __dsub_rn(wq, wp), B = __dsub_rn(w, wq);
+                // multiplying by 1 is exact
+                const double lhs = di == 1 ? A : __dmul_rn(A, exact_double(di));
+                const double rhs = dp == 1 ? B : __dmul_rn(B, exact_double(dp));
+                pop = order_key(lhs) >= order_key(rhs);
             }
             if (!pop) break;
             --k;
             wq = wp;
             xq = xp;
+            Q = P;
             if (k >= 2) {
-                wp = sv[(k - 2) * T];
                 xp = sx[(k - 2) * T];
-                A = __dsub_rn(wq, wp);
+                wp = src[(long long)xp * step];
+                P = trunc32(wp);
             }
         }
         wp = wq;
         xp = xq;
-        A = B;
+        P = Q;
         wq = w;
         xq = l;
-        sv[k * T] = w;
+        Q = V;
         sx[k * T] = (short)l;
         ++k;
     }
     // every finite point lies between the first and the last vertex
-    const long long base = (long long)(j - j0) * g.N + p0;
     int e = -1, xa = 0, xb = -1;  // the current edge
     float fa = 0.0f, slope = 0.0f, off = 0.0f;
     for (int l = 1; l < len - 1; ++l) {
@@ -540,8 +573,8 @@ __global__ void __launch_bounds__(128) k_grid_lines(GridT<D> g, const GridDirT<D
             ++e;
             xa = sx[e * T];
             xb = sx[(e + 1) * T];
-            fa = trunc32(sv[e * T]);
-            const float fb = trunc32(sv[(e + 1) * T]);
+            fa = trunc32(src[(long long)xa * step]);
+            const float fb = trunc32(src[(long long)xb * step]);
             // the bound covers the truncation of both ends and the rounding of
             // the chord; ends outside FP32's range leave it to the FP64 value
             off = 1e-6f * (fabsf(fa) + fabsf(fb)) + 1e-36f;
@@ -563,7 +596,23 @@ __global__ void __launch_bounds__(128) k_grid_lines(GridT<D> g, const GridDirT<D
     }
 }
 
+constexpr int kRcp = 64;  // chord denominators with a tabulated reciprocal
 constexpr int kGridChunkDirs = 64;  // directions per chunk at most (a mask word in the reduction)
+
+// For offsets in {-1, 0, 1}: the directions of a chunk along which a point is
+// interior depend only on which components lie at an end of their axis; per
+// chunk and pattern of components, their mask (nine dimensions: most points
+// are interior along few directions, and testing each cost more than the
+// rest).
+template <int D>
+__global__ void k_grid_patterns(const GridDirT<D> *dirs, int nd, int chunk, unsigned long long *pat) {
+    const int t = blockIdx.x * blockDim.x + threadIdx.x, j0 = (t >> D) * chunk;
+    if (j0 >= nd) return;
+    unsigned long long m = 0;
+    for (int q = 0; q < chunk && j0 + q < nd; ++q)
+        if (!((t & ((1 << D) - 1)) & (dirs[j0 + q].pos | dirs[j0 + q].neg))) m |= 1ull << q;
+    pat[t] = m;
+}
 
 // Per point, directions [j0, j1): the smallest chord value h below the best so
 // far wins, the lowest direction on equal values (first chunk: the best so far
@@ -577,12 +626,16 @@ constexpr int kGridChunkDirs = 64;  // directions per chunk at most (a mask word
 template <int D, bool kUnit>
 __global__ void __launch_bounds__(256) k_grid_reduce(GridT<D> g, const GridDirT<D> *dirs, int j0,
                                                      int j1, int first, int last, const double *Win,
-                                                     const float *H, const unsigned *S, double *Wout,
+                                                     const float *H, const unsigned *S,
+                                                     const unsigned long long *pat, double *Wout,
                                                      int *lam, unsigned long long *dec,
                                                      const int *done) {
     if (done && *done) return;
+    constexpr bool kPat = kUnit && D == 9;
     __shared__ GridDirT<D> s_d[kGridChunkDirs];
     __shared__ unsigned s_nz[kGridChunkDirs];  // components that the direction moves
+    __shared__ double s_y[kRcp];               // fl(1 / den)
+    if (threadIdx.x < kRcp) s_y[threadIdx.x] = __drcp_rn((double)max((int)threadIdx.x, 1));
     const int n = j1 - j0;
     for (int k = threadIdx.x; k < n * (int)(sizeof(GridDirT<D>) / 4); k += blockDim.x)
         reinterpret_cast<int *>(s_d)[k] = reinterpret_cast<const int *>(dirs + j0)[k];
@@ -601,12 +654,14 @@ __global__ void __launch_bounds__(256) k_grid_reduce(GridT<D> g, const GridDirT<
             bp = lam[3 * p + 2];
         }
         int i[D], mg[D];  // grid points between the point and the nearer end of each axis
-        unsigned edge = 0;
+        unsigned edge = 0, lo2 = 0, hi2 = 0;  // components at an end, within one of an end
         grid_index<D>(g, (int)p, i);
 #pragma unroll
         for (int c = 0; c < D; ++c) {
             mg[c] = min(i[c], g.n[c] - 1 - i[c]);
             edge |= mg[c] < 1 ? 1u << c : 0u;
+            lo2 |= i[c] < 2 ? 1u << c : 0u;
+            hi2 |= i[c] > g.n[c] - 3 ? 1u << c : 0u;
         }
         auto interior = [&](int q) {
             if (kUnit) return !(edge & s_nz[q]);
@@ -615,14 +670,49 @@ __global__ void __launch_bounds__(256) k_grid_reduce(GridT<D> g, const GridDirT<
             for (int c = 0; c < D; ++c) in = in && mg[c] >= abs(s_d[q].o[c]);
             return in;
         };
+        // an interior point's line has three points: neither second neighbour
+        // lies in the grid
+        auto three = [&](int q) {
+            if (kMinLine<D> == 3) return false;  // listed
+            const GridDirT<D> &d = s_d[q];
+            if (kUnit) return ((hi2 & d.pos) | (lo2 & d.neg)) && ((lo2 & d.pos) | (hi2 & d.neg));
+            bool fwd = true, back = true;
+#pragma unroll
+            for (int c = 0; c < D; ++c) {
+                const int a = i[c] + 2 * d.o[c], b = i[c] - 2 * d.o[c];
+                fwd = fwd && a >= 0 && a < g.n[c];
+                back = back && b >= 0 && b < g.n[c];
+            }
+            return !fwd && !back;
+        };
+        // FP32 lower bound of the chord value of interior direction j0 + q, inf
+        // if the point is a vertex of the line's hull
+        const float f0 = trunc32(w0);
+        auto lower = [&](int q) {
+            if (!three(q)) return H[q * N + p];
+            // Algorithm 1 on three points: the centre is popped unless it lies
+            // strictly below the chord of its neighbours
+            const int st = s_d[q].step;
+            const double wa = Win[p - st], wb = Win[p + st];
+            if (!finite_bits(wa) || !finite_bits(wb)) return INFINITY;
+            const float fa = trunc32(wa), fb = trunc32(wb), a = fabsf(fa) + fabsf(fb);
+            const float d = (f0 - fa) - (fb - f0), mag = a + fabsf(f0);
+            bool in;
+            if (fabsf(d) > 1e-6f * mag && mag < 1e30f && mag > 1e-20f) in = d > 0.0f;
+            else in = order_key(__dsub_rn(w0, wa)) >= order_key(__dsub_rn(wb, w0));
+            if (!in) return INFINITY;
+            return a < 1e30f ? 0.5f * (fa + fb) - (1e-6f * a + 1e-36f) : -INFINITY;
+        };
         // the exact chord value of direction j0 + q
         auto exact = [&](int q) {
-            const unsigned sp = S[q * N + p];
+            const unsigned sp = three(q) ? 0x0001ffffu : S[q * N + p];  // (-1, 1)
             const int ra = (int)(short)(sp & 0xffffu), rb = (int)(sp >> 16), st = s_d[q].step;
             const double wa = Win[p + (long long)ra * st], wb = Win[p + (long long)rb * st];
             const double num = __dsub_rn(__dmul_rn(exact_double(rb), wa),
                                          __dmul_rn(exact_double(ra), wb));
-            const double h = __ddiv_rn(num, exact_double(rb - ra));
+            const int den = rb - ra;
+            const double h = den < kRcp ? quotient(num, den, s_y[den])
+                                        : __ddiv_rn(num, exact_double(den));
             const long long kh = order_key(h), kb = order_key(best);
             if (kh < kb || (kh == kb && j0 + q < bd)) {
                 best = h;
@@ -634,25 +724,37 @@ __global__ void __launch_bounds__(256) k_grid_reduce(GridT<D> g, const GridDirT<
         if (finite_bits(w0)) {
             float m1 = INFINITY, m2 = INFINITY;  // the two smallest bounds
             int q1 = 0;
-#pragma unroll 4
-            for (int q = 0; q < n; ++q) {
-                if (!interior(q)) continue;
-                const float h = H[q * N + p];
+            auto see = [&](int q) {
+                const float h = lower(q);
                 m2 = fminf(m2, fmaxf(m1, h));
                 if (h < m1) {
                     m1 = h;
                     q1 = q;
                 }
+            };
+            unsigned long long in = 0;
+            if (kPat) {
+                in = pat[edge];
+                for (unsigned long long m = in; m; m &= m - 1) see(__ffsll((long long)m) - 1);
+            } else {
+#pragma unroll 4
+                for (int q = 0; q < n; ++q)
+                    if (interior(q)) see(q);
             }
             if (m1 < INFINITY && m1 <= __double2float_ru(best)) exact(q1);
             float lim = __double2float_ru(best);
             unsigned long long more = 0;
             if (m2 < INFINITY && m2 <= lim) {
-                for (int q = 0; q < n; ++q)
-                    if (q != q1 && interior(q)) {
-                        const float h = H[q * N + p];
-                        if (h < INFINITY && h <= lim) more |= 1ull << q;
-                    }
+                auto again = [&](int q) {
+                    const float h = lower(q);
+                    if (q != q1 && h < INFINITY && h <= lim) more |= 1ull << q;
+                };
+                if (kPat) {
+                    for (unsigned long long m = in; m; m &= m - 1) again(__ffsll((long long)m) - 1);
+                } else {
+                    for (int q = 0; q < n; ++q)
+                        if (interior(q)) again(q);
+                }
             }
             for (; more; more &= more - 1) exact(__ffsll((long long)more) - 1);
         }
@@ -1027,7 +1129,7 @@ int check_dirs(int nd, const int32_t *off, const GridT<D> &gd, std::vector<GridD
         for (int c = 0; c < D; ++c) step += (long long)g.o[c] * gd.s[c];
         g.step = (int)step;
         dirs[j] = g;
-        line_off[j + 1] = line_off[j] + lines_of<D>(gd, g, 3);
+        line_off[j + 1] = line_off[j] + lines_of<D>(gd, g, kMinLine<D>);
     }
     return CVX_OK;
 }
@@ -1041,9 +1143,15 @@ struct GridWork {
     int *starts;
     float *H;
     unsigned *S;
+    unsigned long long *pat;  // k_grid_patterns
     int chunk;  // directions per chunk
     bool unit;  // all offsets in {-1, 0, 1}
 };
+
+template <int D>
+size_t grid_patterns(int nd, int chunk) {
+    return (size_t)((nd + chunk - 1) / chunk) << D;
+}
 
 template <int D>
 size_t grid_work_bytes(int nd, const GridT<D> &gd, long long lines, int &chunk) {
@@ -1052,7 +1160,7 @@ size_t grid_work_bytes(int nd, const GridT<D> &gd, long long lines, int &chunk) 
         1, std::min<size_t>(std::min(nd, kGridChunkDirs), grid_chunk_bytes() / per_dir));
     return up256(sizeof(GridDirT<D>) * nd) + up256(sizeof(long long) * (nd + 1)) +
            up256(sizeof(unsigned) * nd * (size_t)(kGridMaxLine + 1)) +
-           up256(sizeof(int) * (size_t)lines) +
+           up256(sizeof(int) * (size_t)lines) + up256(sizeof(unsigned long long) * grid_patterns<D>(nd, chunk)) +
            up256(sizeof(float) * (size_t)chunk * gd.N) +
            up256(sizeof(unsigned) * (size_t)chunk * gd.N);
 }
@@ -1069,6 +1177,8 @@ void carve_grid_work(char *ws, const std::vector<GridDirT<D>> &dirs, const GridT
     ws += up256(sizeof(unsigned) * nd * (size_t)(kGridMaxLine + 1));
     w.starts = (int *)ws;
     ws += up256(sizeof(int) * (size_t)lines);
+    w.pat = (unsigned long long *)ws;
+    ws += up256(sizeof(unsigned long long) * grid_patterns<D>(nd, chunk));
     w.H = (float *)ws;
     ws += up256(sizeof(float) * (size_t)chunk * gd.N);
     w.S = (unsigned *)ws;
@@ -1098,6 +1208,11 @@ int grid_setup(const GridT<D> &gd, const std::vector<GridDirT<D>> &dirs,
     CK(cudaMemcpyAsync(w.line_off, line_off.data(), sizeof(long long) * (nd + 1),
                        cudaMemcpyHostToDevice, s),
        "grid setup");
+    if (w.unit && D == 9) {
+        const size_t np = grid_patterns<D>(nd, w.chunk);
+        k_grid_patterns<D><<<(unsigned)((np + 127) / 128), 128, 0, s>>>(w.dirs, nd, w.chunk, w.pat);
+        CK(cudaGetLastError(), "grid patterns");
+    }
     if (line_off[nd] == 0) return CVX_OK;
     const int cap = grid_line_cap<D>(gd);
     k_grid_cursors<D><<<(nd * (cap + 1) + 127) / 128, 128, 0, s>>>(gd, w.dirs, nd, cap, w.cur);
@@ -1119,7 +1234,7 @@ int grid_enqueue_step(const GridT<D> &gd, int nd, const std::vector<long long> &
                       unsigned long long *dec, const int *done, cudaStream_t s,
                       cvx_handle *h) {
     const int T = grid_line_threads(cap);
-    const size_t smem = (size_t)cap * T * (sizeof(double) + sizeof(short));
+    const size_t smem = (size_t)cap * T * sizeof(short);
     for (int j0 = 0; j0 < nd; j0 += w.chunk) {
         const int j1 = std::min(nd, j0 + w.chunk);
         const long long lines = line_off[j1] - line_off[j0];
@@ -1135,7 +1250,9 @@ int grid_enqueue_step(const GridT<D> &gd, int nd, const std::vector<long long> &
         }
         auto kr = w.unit ? k_grid_reduce<D, true> : k_grid_reduce<D, false>;
         kr<<<(unsigned)((gd.N + 255LL) / 256), 256, 0, s>>>(gd, w.dirs, j0, j1, j0 == 0, j1 == nd,
-                                                            Win, w.H, w.S, Wout, lam, dec, done);
+                                                            Win, w.H, w.S,
+                                                            w.pat + ((size_t)(j0 / w.chunk) << D),
+                                                            Wout, lam, dec, done);
         CK(cudaGetLastError(), "grid reduce kernel");
     }
     return CVX_OK;
@@ -1144,7 +1261,7 @@ int grid_enqueue_step(const GridT<D> &gd, int nd, const std::vector<long long> &
 template <int D>
 int set_line_smem(int cap) {
     const int T = grid_line_threads(cap);
-    const size_t smem = (size_t)cap * T * (sizeof(double) + sizeof(short));
+    const size_t smem = (size_t)cap * T * sizeof(short);
     CK(cudaFuncSetAttribute(k_grid_lines<D>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                             (int)smem),
        "grid line kernel shared memory");
