@@ -103,6 +103,16 @@ __device__ __forceinline__ float trunc32(double x) {
     return __int_as_float(b | (hi & 0x80000000));
 }
 
+// fl(1 / v), v = 1 .. 2 kGridMaxLine (the chord denominators; the compiler's
+// constant division is correctly rounded).
+struct RcpTable {
+    double y[2 * kGridMaxLine + 1];
+    constexpr RcpTable() : y() {
+        for (int v = 1; v <= 2 * kGridMaxLine; ++v) y[v] = 1.0 / v;
+    }
+};
+__device__ const RcpTable kRcp = RcpTable();
+
 // num / den for a positive integer den, y = fl(1 / den): the correctly rounded
 // quotient in five operations.  fl(num y) is within two units in the last
 // place, the first correction (residual exact by FMA) makes it faithful, and
@@ -596,7 +606,6 @@ __global__ void __launch_bounds__(128) k_grid_lines(GridT<D> g, const GridDirT<D
     }
 }
 
-constexpr int kRcp = 64;  // chord denominators with a tabulated reciprocal
 constexpr int kGridChunkDirs = 64;  // directions per chunk at most (a mask word in the reduction)
 
 // For offsets in {-1, 0, 1}: the directions of a chunk along which a point is
@@ -634,8 +643,6 @@ __global__ void __launch_bounds__(256) k_grid_reduce(GridT<D> g, const GridDirT<
     constexpr bool kPat = kUnit && D == 9;
     __shared__ GridDirT<D> s_d[kGridChunkDirs];
     __shared__ unsigned s_nz[kGridChunkDirs];  // components that the direction moves
-    __shared__ double s_y[kRcp];               // fl(1 / den)
-    if (threadIdx.x < kRcp) s_y[threadIdx.x] = __drcp_rn((double)max((int)threadIdx.x, 1));
     const int n = j1 - j0;
     for (int k = threadIdx.x; k < n * (int)(sizeof(GridDirT<D>) / 4); k += blockDim.x)
         reinterpret_cast<int *>(s_d)[k] = reinterpret_cast<const int *>(dirs + j0)[k];
@@ -705,14 +712,20 @@ __global__ void __launch_bounds__(256) k_grid_reduce(GridT<D> g, const GridDirT<
         };
         // the exact chord value of direction j0 + q
         auto exact = [&](int q) {
-            const unsigned sp = three(q) ? 0x0001ffffu : S[q * N + p];  // (-1, 1)
-            const int ra = (int)(short)(sp & 0xffffu), rb = (int)(sp >> 16), st = s_d[q].step;
-            const double wa = Win[p + (long long)ra * st], wb = Win[p + (long long)rb * st];
-            const double num = __dsub_rn(__dmul_rn(exact_double(rb), wa),
-                                         __dmul_rn(exact_double(ra), wb));
-            const int den = rb - ra;
-            const double h = den < kRcp ? quotient(num, den, s_y[den])
-                                        : __ddiv_rn(num, exact_double(den));
+            int ra = -1, rb = 1;
+            const int st = s_d[q].step;
+            double h;
+            if (three(q)) {
+                h = __dmul_rn(0.5, __dadd_rn(Win[p + st], Win[p - st]));
+            } else {
+                const unsigned sp = S[q * N + p];
+                ra = (int)(short)(sp & 0xffffu);
+                rb = (int)(sp >> 16);
+                const double wa = Win[p + (long long)ra * st], wb = Win[p + (long long)rb * st];
+                const double num = __dsub_rn(__dmul_rn(exact_double(rb), wa),
+                                             __dmul_rn(exact_double(ra), wb));
+                h = quotient(num, rb - ra, kRcp.y[rb - ra]);
+            }
             const long long kh = order_key(h), kb = order_key(best);
             if (kh < kb || (kh == kb && j0 + q < bd)) {
                 best = h;
