@@ -47,4 +47,21 @@ bool make_tmap_bf16(CUtensorMap *map, const void *ptr, long long rows, long long
 cudaError_t launch_gemm(const CUtensorMap &tA, const CUtensorMap &tB, int M, int N, int K,
                         int k_split, int BN, const GemmEpi &ep, cudaStream_t s);
 
+// Inference of the whole network in one kernel (cvx_mlp_fused.cu).
+struct MlpForward {
+    int M;             // rows
+    const int *M_dev;  // optional device-side row count; rows valid = *M_dev - m_off
+    int m_off;
+    const float *X;            // M x 6 raw features, standardised with scale, or
+    const __nv_bfloat16 *X16;  // M x 16 standardised rows (X unused)
+    const float *scale;        // mean (6), 1 / deviation (6)
+    // weights as k-blocks of 8 elements x all output rows (256, or 16 for the
+    // last layer) x 16 bytes
+    const __nv_bfloat16 *W[5];
+    const float *bias[5];
+    float *out;  // M x 7
+    int *err;    // set to 1 if a wait timed out
+};
+cudaError_t launch_mlp_forward(const MlpForward &f, cudaStream_t s);
+
 }  // namespace cvx

@@ -284,7 +284,7 @@ int surrogate_propose(cvx_handle *h, const cvx_params *p, int64_t n, const doubl
             const int m = (int)std::min<long long>(chunk, max_nodes - off);
             k_feat<<<(m + 255) / 256, 256, 0, s>>>(pp, l, (int)off, m, S.scale, S.X);
             CK(cudaGetLastError(), "surrogate_propose/features");
-            rc = sur_forward(h, m, false, s, pp.cnt + l, (int)off);
+            rc = sur_infer(h, m, nullptr, S.out, s, pp.cnt + l, (int)off);
             if (rc) return rc;
             k_decode<<<(m + 255) / 256, 256, 0, s>>>(pp, l, (int)off, m, S.out);
             CK(cudaGetLastError(), "surrogate_propose/decode");

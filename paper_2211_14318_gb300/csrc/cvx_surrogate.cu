@@ -34,9 +34,10 @@ static_assert(kBOff[4] + 7 == kSurParams, "parameter layout");
 using bf16 = __nv_bfloat16;
 
 // ------------------------------------------------------------------ kernels
-// P (rows_pad x cols_pad) = W (out x in) zero-padded; T (cols_pad x rows_pad) = P^T.
+// P (rows_pad x cols_pad) = W (out x in) zero-padded; T (cols_pad x rows_pad) =
+// P^T; B = P in k-blocks of 8 columns: (cols_pad / 8) x rows_pad x 8.
 __global__ void k_pack(const float *W, int out, int in, int rows_pad, int cols_pad, bf16 *P,
-                       bf16 *T) {
+                       bf16 *T, bf16 *B) {
     const int idx = blockIdx.x * blockDim.x + threadIdx.x;
     if (idx >= rows_pad * cols_pad) return;
     const int r = idx / cols_pad, c = idx % cols_pad;
@@ -44,6 +45,7 @@ __global__ void k_pack(const float *W, int out, int in, int rows_pad, int cols_p
     const bf16 b = __float2bfloat16_rn(v);
     if (P) P[(long long)r * cols_pad + c] = b;
     if (T) T[(long long)c * rows_pad + r] = b;
+    B[((long long)(c >> 3) * rows_pad + r) * 8 + (c & 7)] = b;
 }
 
 // Standardised inputs of rows idx[m] (or m) -> X (n x 16, bf16, zero-padded)
@@ -146,6 +148,7 @@ void destroy_surrogate(cvx_handle *h) {
     for (int l = 0; l < 5; ++l) {
         cudaFree(S->Wp[l]);
         cudaFree(S->Wt[l]);
+        cudaFree(S->Wb[l]);
     }
     for (int l = 0; l < 4; ++l) {
         cudaFree(S->A[l]);
@@ -179,6 +182,7 @@ int sur_params(cvx_handle *h) {
     }
     CK(alloc(&S.Wp[4], 16 * 256), "surrogate");
     CK(alloc(&S.Wt[4], 256 * 16), "surrogate");
+    for (int l = 0; l < 5; ++l) CK(alloc(&S.Wb[l], l == 0 ? 256 * 16 : (l < 4 ? 256 * 256 : 16 * 256)), "surrogate");
     return CVX_OK;
 }
 
@@ -230,7 +234,7 @@ cudaError_t sur_pack(Surrogate &S, cudaStream_t s) {
     for (int l = 0; l < 5; ++l) {
         const int total = rp[l] * cp[l];
         k_pack<<<(total + 255) / 256, 256, 0, s>>>(S.w + kWOff[l], kOut[l], kIn[l], rp[l], cp[l],
-                                                   S.Wp[l], l ? S.Wt[l] : nullptr);
+                                                   S.Wp[l], l ? S.Wt[l] : nullptr, S.Wb[l]);
     }
     return cudaGetLastError();
 }
@@ -251,41 +255,59 @@ GemmEpi epi(int mode, int Mv, int *err) {
 
 }  // namespace
 
-// Forward pass of n <= cap standardised rows in S.X (and S.XT).  train: keep
-// Z, A^T for the backward pass (otherwise the activations alternate between
-// two buffers).  M_dev (optional): device-side row count, of which rows
-// m_off .. m_off + n - 1 are these.
-int sur_forward(cvx_handle *h, int n, bool train, cudaStream_t s, const int *M_dev, int m_off) {
+// Inference of n rows in one kernel: raw features X, or (X null) the
+// standardised rows in S.X.  M_dev (optional): device-side row count, of which
+// rows m_off .. m_off + n - 1 are these.
+int sur_infer(cvx_handle *h, int n, const float *X, float *out, cudaStream_t s, const int *M_dev,
+              int m_off) {
+    Surrogate &S = *h->sur;
+    MlpForward f = {};
+    f.M = n;
+    f.M_dev = M_dev;
+    f.m_off = m_off;
+    f.X = X;
+    f.X16 = X ? nullptr : S.X;
+    f.scale = S.scale;
+    for (int l = 0; l < 5; ++l) {
+        f.W[l] = S.Wb[l];
+        f.bias[l] = S.w + kBOff[l];
+    }
+    f.out = out;
+    f.err = S.err;
+    CK(launch_mlp_forward(f, s), "surrogate forward");
+    return CVX_OK;
+}
+
+namespace {
+
+// Forward pass of n <= cap standardised rows in S.X (and S.XT), layer by layer,
+// keeping Z, A and A^T for the backward pass.
+int sur_forward(cvx_handle *h, int n, cudaStream_t s) {
     Surrogate &S = *h->sur;
     CUtensorMap tX, tW, tA;
     TMAP(tX, S.X, n, 16, 16, 128);
     TMAP(tW, S.Wp[0], 256, 16, 16, 256);
     GemmEpi e = epi(EPI_HIDDEN, n, S.err);
-    e.M_dev = M_dev;
-    e.m_off = m_off;
     e.bias = S.w + kBOff[0];
-    e.Z = train ? S.Z[0] : nullptr;
+    e.Z = S.Z[0];
     e.ldz = 256;
     e.A = S.A[0];
     e.lda = 256;
-    e.AT = train ? S.AT[0] : nullptr;
+    e.AT = S.AT[0];
     e.ldat = S.cap;
     CK(launch_gemm(tX, tW, n, 256, 16, 16, 256, e, s), "surrogate forward");
     for (int l = 1; l < 4; ++l) {
-        bf16 *in = train ? S.A[l - 1] : S.A[(l - 1) & 1];
-        TMAP(tA, in, n, 256, 256, 128);
+        TMAP(tA, S.A[l - 1], n, 256, 256, 128);
         TMAP(tW, S.Wp[l], 256, 256, 256, 256);
         e.bias = S.w + kBOff[l];
-        e.Z = train ? S.Z[l] : nullptr;
-        e.A = train ? S.A[l] : S.A[l & 1];
-        e.AT = train ? S.AT[l] : nullptr;
+        e.Z = S.Z[l];
+        e.A = S.A[l];
+        e.AT = S.AT[l];
         CK(launch_gemm(tA, tW, n, 256, 256, 256, 256, e, s), "surrogate forward");
     }
-    TMAP(tA, train ? S.A[3] : S.A[1], n, 256, 256, 128);
+    TMAP(tA, S.A[3], n, 256, 256, 128);
     TMAP(tW, S.Wp[4], 16, 256, 256, 16);
     GemmEpi o = epi(EPI_OUT, n, S.err);
-    o.M_dev = M_dev;
-    o.m_off = m_off;
     o.C = S.out;
     o.ldc = 7;
     o.n_store = 7;
@@ -293,8 +315,6 @@ int sur_forward(cvx_handle *h, int n, bool train, cudaStream_t s, const int *M_d
     CK(launch_gemm(tA, tW, n, 16, 256, 256, 16, o, s), "surrogate forward");
     return CVX_OK;
 }
-
-namespace {
 
 // Loss and gradient (added to S.g) of the batch in S.X / S.Yb after
 // sur_forward(train = true).
@@ -460,18 +480,11 @@ int surrogate_forward(cvx_handle *h, int64_t n, const float *X, float *out, cvx_
     DeviceGuard g(h->device);
     cudaStream_t s = (cudaStream_t)sv;
     Surrogate &S = *h->sur;
-    const int chunk = 1 << 16;
-    int rc = sur_batch(h, (int)std::min<int64_t>(n, chunk));
-    if (rc) return rc;
+    const int64_t chunk = (int64_t)1 << 30;  // rows per launch
     for (int64_t o = 0; o < n; o += chunk) {
-        const int m = (int)std::min<int64_t>(chunk, n - o);
-        k_input<<<(m + 255) / 256, 256, 0, s>>>(m, nullptr, X + 6 * o, S.scale, S.X, nullptr, 0,
-                                                nullptr, nullptr);
-        CK(cudaGetLastError(), "surrogate_forward");
-        rc = sur_forward(h, m, false, s, nullptr, 0);
+        const int rc = sur_infer(h, (int)std::min<int64_t>(chunk, n - o), X + 6 * o, out + 7 * o, s,
+                                 nullptr, 0);
         if (rc) return rc;
-        CK(cudaMemcpyAsync(out + 7 * o, S.out, sizeof(float) * 7 * m, cudaMemcpyDeviceToDevice, s),
-           "surrogate_forward");
     }
     return check_err(S, s);
 }
@@ -492,7 +505,7 @@ int surrogate_loss_grad(cvx_handle *h, int64_t n, const float *X, const float *Y
     CK(cudaGetLastError(), "surrogate_loss_grad");
     CK(cudaMemsetAsync(S.g, 0, sizeof(float) * kSurParams, s), "surrogate_loss_grad");
     CK(cudaMemsetAsync(S.loss, 0, sizeof(float), s), "surrogate_loss_grad");
-    rc = sur_forward(h, (int)n, true, s, nullptr, 0);
+    rc = sur_forward(h, (int)n, s);
     if (rc) return rc;
     rc = sur_backward(h, (int)n, s);
     if (rc) return rc;
@@ -556,7 +569,7 @@ int surrogate_train(cvx_handle *h, int64_t n, const float *X, const float *Y,
             k_input<<<(m + 255) / 256, 256, 0, s>>>(m, S.idx + o, X, S.scale, S.X, S.XT, S.cap, Y, S.Yb);
             CK(cudaGetLastError(), "surrogate_train");
             CK(cudaMemsetAsync(S.g, 0, sizeof(float) * kSurParams, s), "surrogate_train");
-            rc = sur_forward(h, m, true, s, nullptr, 0);
+            rc = sur_forward(h, m, s);
             if (rc) return rc;
             rc = sur_backward(h, m, s);
             if (rc) return rc;

@@ -5,6 +5,8 @@
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
+#include "cvx_mlp.h"
+
 struct cvx_handle;
 
 namespace cvx {
@@ -20,6 +22,7 @@ struct Surrogate {
     float *scale = nullptr;
     float *w = nullptr, *g = nullptr, *m = nullptr, *v = nullptr;
     __nv_bfloat16 *Wp[5] = {}, *Wt[5] = {};
+    __nv_bfloat16 *Wb[5] = {};  // packed weights as k-blocks (MlpForward::W)
     long long adam_t = 0;
     int cap = 0;
     __nv_bfloat16 *X = nullptr, *XT = nullptr, *A[4] = {}, *AT[4] = {}, *dZo = nullptr,
@@ -34,6 +37,7 @@ void destroy_surrogate(cvx_handle *h);
 int sur_params(cvx_handle *h);
 // Batch buffers for at least n rows.
 int sur_batch(cvx_handle *h, int n);
-int sur_forward(cvx_handle *h, int n, bool train, cudaStream_t s, const int *M_dev, int m_off);
+int sur_infer(cvx_handle *h, int n, const float *X, float *out, cudaStream_t s, const int *M_dev,
+              int m_off);
 
 }  // namespace cvx
