@@ -1,19 +1,17 @@
-// cvx_gemm.cu -- the BF16 tensor-core GEMM of the surrogate network
-// (tcgen05, FP32 accumulation in TMEM, operands staged by TMA) with the
-// epilogues of the network's forward and backward passes fused in.
+// cvx_gemm.cu -- the BF16 tensor-core GEMM behind cvx_gemm_bf16 (tcgen05, FP32
+// accumulation in TMEM, operands staged by TMA).
 //
-//   D[m][n] = sum_k A[m][k] B[n][k]       (A: M x K, B: N x K, both bf16,
+//   C[m][n] = sum_k A[m][k] B[n][k]       (A: M x K, B: N x K, both bf16,
 //                                          row-major with K contiguous)
 //
-// One CTA of 256 threads computes a 128 x BN tile over a K range (split-K for
-// the weight gradients).  Thread 0 issues the TMA loads (one box per k-block
-// of 8 elements, two stages of 64) and the MMAs (K = 16 each); then warps w
-// and w + 4 read the TMEM lanes of rows 32 (w % 4) .. +31 (one accumulator
-// row per thread), each half of the columns, and apply the epilogue.
+// One CTA of 256 threads computes a 128 x BN tile.  Thread 0 issues the TMA
+// loads (one box per k-block of 8 elements, two stages of 64) and the MMAs
+// (K = 16 each); then warps w and w + 4 read the TMEM lanes of rows
+// 32 (w % 4) .. +31 (one accumulator row per thread), each half of the
+// columns.  The network itself runs in cvx_mlp_fused.cu and cvx_mlp_train.cu.
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
-#include <math.h>
 
 #include <algorithm>
 #include <mutex>
@@ -28,107 +26,18 @@ namespace {
 constexpr int kBM = 128, kBK = 64, kStages = 2;
 constexpr uint64_t kWaitNs = 1000000000ull;  // 1 s per wait, then give up
 
-// Normal CDF Phi(z) and density phi(z) with erf from Abramowitz & Stegun,
-// Handbook of Mathematical Functions, formula 7.1.26:
-//   erf(x) = 1 - (a1 t + a2 t^2 + a3 t^3 + a4 t^4 + a5 t^5) exp(-x^2),
-//   t = 1 / (1 + p x), x >= 0, |error| <= 1.5e-7
-// (one exponential shared by Phi and phi).
-__device__ __forceinline__ void normal_cdf_pdf(float z, float &Phi, float &phi) {
-    const float x = fabsf(z) * 0.70710678118654752f;
-    const float t = __fdividef(1.0f, fmaf(0.3275911f, x, 1.0f));
-    const float poly =
-        t * fmaf(t, fmaf(t, fmaf(t, fmaf(t, 1.061405429f, -1.453152027f), 1.421413741f),
-                         -0.284496736f),
-                 0.254829592f);
-    const float ex = __expf(-x * x);
-    const float erfx = 1.0f - poly * ex;
-    Phi = 0.5f * (1.0f + (z < 0.0f ? -erfx : erfx));
-    phi = 0.39894228040143268f * ex;
-}
-__device__ __forceinline__ float gelu(float z) {
-    float Phi, phi;
-    normal_cdf_pdf(z, Phi, phi);
-    return z * Phi;
-}
-__device__ __forceinline__ float gelu_grad(float z) {
-    float Phi, phi;
-    normal_cdf_pdf(z, Phi, phi);
-    return Phi + z * phi;
-}
-
-__device__ __forceinline__ void store_bf16x16(__nv_bfloat16 *dst, const float (&v)[16]) {
-    uint32_t w[8];
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-        __nv_bfloat162 h = __floats2bfloat162_rn(v[2 * i], v[2 * i + 1]);
-        w[i] = *reinterpret_cast<uint32_t *>(&h);
-    }
-    uint4 *d = reinterpret_cast<uint4 *>(dst);
-    d[0] = make_uint4(w[0], w[1], w[2], w[3]);
-    d[1] = make_uint4(w[4], w[5], w[6], w[7]);
-}
-
-// The epilogue of 16 accumulator columns n .. n + 15 of row m (one thread).
-__device__ __forceinline__ void gemm_epilogue(const GemmEpi &ep, int m, int n, const float (&v)[16],
-                                              int Mv, int N, int lane) {
-    switch (ep.mode) {
-    case EPI_F32:
-        if (m < Mv)
-            for (int i = 0; i < 16; ++i)
-                if (n + i < N) ep.C[(long long)m * ep.ldc + n + i] = v[i];
-        break;
-    case EPI_HIDDEN: {
-        if (m >= Mv) break;
-        float a[16];
-        for (int i = 0; i < 16; ++i) {
-            const float z = v[i] + ep.bias[n + i];
-            if (ep.Z) ep.Z[(long long)m * ep.ldz + n + i] = z;
-            a[i] = gelu(z);
-        }
-        store_bf16x16(ep.A + (long long)m * ep.lda + n, a);
-        if (ep.AT)
-            for (int i = 0; i < 16; ++i)
-                ep.AT[(long long)(n + i) * ep.ldat + m] = __float2bfloat16_rn(a[i]);
-        break;
-    }
-    case EPI_OUT:
-        if (m < Mv)
-            for (int i = 0; i < 16; ++i)
-                if (n + i < ep.n_store)
-                    ep.C[(long long)m * ep.ldc + n + i] = v[i] + ep.bias[n + i];
-        break;
-    case EPI_DA: {
-        float dz[16];
-        const bool in = m < Mv;
+// 16 accumulator columns n .. n + 15 of row m (one thread).
+__device__ __forceinline__ void store_row(const GemmEpi &ep, int m, int n, const float (&v)[16],
+                                          int N) {
+    if (m < ep.M_valid)
         for (int i = 0; i < 16; ++i)
-            dz[i] = in ? v[i] * gelu_grad(ep.Z[(long long)m * ep.ldz + n + i]) : 0.0f;
-        if (in) {
-            store_bf16x16(ep.A + (long long)m * ep.lda + n, dz);
-            if (ep.AT)
-                for (int i = 0; i < 16; ++i)
-                    ep.AT[(long long)(n + i) * ep.ldat + m] = __float2bfloat16_rn(dz[i]);
-        }
-        if (ep.dbias) {
-            for (int i = 0; i < 16; ++i) {
-                float s = dz[i];
-                for (int o = 16; o; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-                if (lane == 0) atomicAdd(ep.dbias + n + i, s);
-            }
-        }
-        break;
-    }
-    case EPI_DW:
-        if (m < ep.m_store)
-            for (int i = 0; i < 16; ++i)
-                if (n + i < ep.n_store) atomicAdd(ep.C + (long long)m * ep.ldc + n + i, v[i]);
-        break;
-    }
+            if (n + i < N) ep.C[(long long)m * ep.ldc + n + i] = v[i];
 }
 
 template <int BN>
 __global__ void __launch_bounds__(256, 1)
     k_gemm(const __grid_constant__ CUtensorMap tA, const __grid_constant__ CUtensorMap tB, int M,
-           int N, int K, int k_split, GemmEpi ep) {
+           int N, int K, GemmEpi ep) {
     constexpr int A_BYTES = kBM * kBK * 2;
     constexpr int B_BYTES = BN * kBK * 2;
     constexpr uint32_t TCOLS = BN < 32 ? 32 : BN;
@@ -142,11 +51,6 @@ __global__ void __launch_bounds__(256, 1)
     __shared__ int s_fail;
 
     const int m0 = blockIdx.x * kBM, n0 = blockIdx.y * BN;
-    const int kc0 = blockIdx.z * k_split;
-    const int kc1 = min(K, kc0 + k_split);
-    const int Mv = ep.M_dev ? min(*ep.M_dev - ep.m_off, ep.M_valid) : ep.M_valid;
-    if (ep.mode != EPI_DW && m0 >= Mv) return;  // the whole tile is padding
-    if (kc0 >= kc1) return;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
     if (threadIdx.x == 0) {
@@ -164,13 +68,13 @@ __global__ void __launch_bounds__(256, 1)
     tc_fence_after();
     const uint32_t tmem = s_tmem;
 
-    const int nchunks = (kc1 - kc0 + kBK - 1) / kBK;
+    const int nchunks = (K + kBK - 1) / kBK;
     if (threadIdx.x == 0) {
         const uint32_t idesc = idesc_bf16(kBM, BN);
         auto issue = [&](int c) {
             const int s = c % kStages;
-            const int k0 = kc0 + c * kBK;
-            const int kbn = min(kBK, kc1 - k0) / 8;
+            const int k0 = c * kBK;
+            const int kbn = min(kBK, K - k0) / 8;
             mbar_expect_tx(&bar_full[s], (unsigned)(kbn * (kBM + BN) * 16));
             for (int kb = 0; kb < kbn; ++kb) {
                 tma_load_2d(sA + s * A_BYTES + kb * kBM * 16, &tA, &bar_full[s], k0 + 8 * kb, m0);
@@ -190,7 +94,7 @@ __global__ void __launch_bounds__(256, 1)
             ok = mbar_wait(&bar_full[s], (c / kStages) & 1, kWaitNs);
             if (!ok) break;
             tc_fence_after();
-            const int kbn = min(kBK, kc1 - (kc0 + c * kBK)) / 8;
+            const int kbn = min(kBK, K - c * kBK) / 8;
             const uint32_t a0 = smem_u32(sA + s * A_BYTES), b0 = smem_u32(sB + s * B_BYTES);
             for (int j = 0; j < kbn / 2; ++j) {
                 const uint64_t ad = smem_desc(a0 + 2 * j * kBM * 16, kBM * 16, 128);
@@ -221,7 +125,7 @@ __global__ void __launch_bounds__(256, 1)
     for (int c0 = cbeg; c0 < cend; c0 += 16) {
         float v[16];
         tmem_ld16(trow + c0, v);
-        if (ok) gemm_epilogue(ep, m, n0 + c0, v, Mv, N, lane);
+        if (ok) store_row(ep, m, n0 + c0, v, N);
     }
     tc_fence_before();
     __syncthreads();
@@ -231,9 +135,8 @@ __global__ void __launch_bounds__(256, 1)
     }
 }
 
-// Persistent, warp-specialised form for K <= 256 (all forward layers and
-// the input-gradient products): the B operand (the weights, BN x K) stays in
-// shared memory for the whole kernel; A tiles (128 x 64) stream through a
+// Persistent, warp-specialised form for K <= 256 and one column of tiles: the
+// B operand (BN x K) stays in shared memory for the whole kernel; A tiles (128 x 64) stream through a
 // four-stage ring; two TMEM accumulators let the epilogue of one tile run
 // while the MMAs of the next are in flight.  Warp 0 (lane 0) issues the TMA
 // loads, warp 1 (lane 0) the MMAs, warps 4..11 run the epilogue (two per
@@ -261,9 +164,7 @@ __global__ void __launch_bounds__(kWsThreads, 1)
     __shared__ __align__(8) uint64_t full[kWsStages], empty[kWsStages], bfull, accf[2], acce[2];
     __shared__ uint32_t s_tmem;
 
-    const int Mv = ep.M_dev ? min(*ep.M_dev - ep.m_off, ep.M_valid) : ep.M_valid;
-    const int ntiles = Mv > 0 ? (Mv + kBM - 1) / kBM : 0;
-    if ((int)blockIdx.x >= ntiles) return;
+    const int ntiles = (M + kBM - 1) / kBM;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int nkc = (K + kBK - 1) / kBK;
 
@@ -351,7 +252,7 @@ __global__ void __launch_bounds__(kWsThreads, 1)
             for (int c0 = cbeg; c0 < cend; c0 += 16) {
                 float r[16];
                 tmem_ld16(trow + c0, r);
-                gemm_epilogue(ep, m, c0, r, Mv, N, lane);
+                store_row(ep, m, c0, r, N);
             }
             tc_fence_before();
             __syncwarp();
@@ -411,9 +312,9 @@ bool make_tmap_bf16(CUtensorMap *map, const void *ptr, long long rows, long long
 }
 
 cudaError_t launch_gemm(const CUtensorMap &tA, const CUtensorMap &tB, int M, int N, int K,
-                        int k_split, int BN, const GemmEpi &ep, cudaStream_t s) {
-    if (K % 16 || k_split % 16 || k_split < 16) return cudaErrorInvalidValue;
-    if (ep.mode != EPI_DW && K <= 256 && k_split >= K && N <= BN) {
+                        int BN, const GemmEpi &ep, cudaStream_t s) {
+    if (K % 16) return cudaErrorInvalidValue;
+    if (K <= 256 && N <= BN) {
         // one tile column, the whole K: the persistent warp-specialised form
         int dev = 0, sms = 0;
         cudaGetDevice(&dev);
@@ -437,17 +338,17 @@ cudaError_t launch_gemm(const CUtensorMap &tA, const CUtensorMap &tB, int M, int
         }
         return cudaGetLastError();
     }
-    const dim3 grid((M + kBM - 1) / kBM, (N + BN - 1) / BN, (K + k_split - 1) / k_split);
+    const dim3 grid((M + kBM - 1) / kBM, (N + BN - 1) / BN);
     if (BN == 256) {
         const size_t sm = gemm_smem<256>();
         cudaError_t e = cudaFuncSetAttribute(k_gemm<256>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
         if (e != cudaSuccess) return e;
-        k_gemm<256><<<grid, 256, sm, s>>>(tA, tB, M, N, K, k_split, ep);
+        k_gemm<256><<<grid, 256, sm, s>>>(tA, tB, M, N, K, ep);
     } else if (BN == 16) {
         const size_t sm = gemm_smem<16>();
         cudaError_t e = cudaFuncSetAttribute(k_gemm<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
         if (e != cudaSuccess) return e;
-        k_gemm<16><<<grid, 256, sm, s>>>(tA, tB, M, N, K, k_split, ep);
+        k_gemm<16><<<grid, 256, sm, s>>>(tA, tB, M, N, K, ep);
     } else {
         return cudaErrorInvalidValue;
     }

@@ -9,30 +9,11 @@
 
 namespace cvx {
 
-enum GemmEpiMode {
-    EPI_F32 = 0,     // C = D (FP32)
-    EPI_HIDDEN = 1,  // z = D + bias -> Z (FP32, optional), A = gelu(z) (bf16), AT = A^T (optional)
-    EPI_OUT = 2,     // C[:, :n_store] = D + bias (FP32)
-    EPI_DA = 3,      // dz = D * gelu'(Z) -> A (bf16), AT = dz^T, dbias += column sums
-    EPI_DW = 4       // C[:m_store, :n_store] += D (FP32 atomics; split-K partial sums)
-};
-
+// The result of launch_gemm: C (M_valid x N, FP32).
 struct GemmEpi {
-    int mode;
-    int M_valid;       // rows holding data (EPI_F32/HIDDEN/OUT/DA)
-    const int *M_dev;  // optional device-side row count; rows valid = *M_dev - m_off
-    int m_off;
+    int M_valid;
     float *C;
     int ldc;
-    int m_store, n_store;
-    const float *bias;
-    float *Z;
-    int ldz;
-    __nv_bfloat16 *A;
-    int lda;
-    __nv_bfloat16 *AT;
-    int ldat;
-    float *dbias;
     int *err;  // set to 1 if a wait timed out
 };
 
@@ -42,10 +23,10 @@ struct GemmEpi {
 bool make_tmap_bf16(CUtensorMap *map, const void *ptr, long long rows, long long cols,
                     long long ld, int box_rows);
 
-// D = A B^T over M x N (tiles of 128 x BN, BN = 16 or 256), K in slices of
-// k_split (multiples of 16).  tA: box rows 128; tB: box rows BN.
+// C = A B^T over M x N (tiles of 128 x BN, BN = 16 or 256), K a multiple of
+// 16.  tA: box rows 128; tB: box rows BN.
 cudaError_t launch_gemm(const CUtensorMap &tA, const CUtensorMap &tB, int M, int N, int K,
-                        int k_split, int BN, const GemmEpi &ep, cudaStream_t s);
+                        int BN, const GemmEpi &ep, cudaStream_t s);
 
 // Inference of the whole network in one kernel (cvx_mlp_fused.cu).
 struct MlpForward {
@@ -63,5 +44,28 @@ struct MlpForward {
     int *err;    // set to 1 if a wait timed out
 };
 cudaError_t launch_mlp_forward(const MlpForward &f, cudaStream_t s);
+
+// Mean loss and its gradient over n rows (cvx_mlp_train.cu), added to loss,
+// dbias and dW.
+struct MlpTrain {
+    int n;
+    long long ld;     // rows of the buffers below, a multiple of 128
+    const int *idx;   // optional: row m is sample idx[m]
+    const float *X;   // x 6 raw features, standardised with scale
+    const float *Y;   // x 7 labels
+    const float *scale;
+    const __nv_bfloat16 *W[5];   // as MlpForward::W
+    const __nv_bfloat16 *Wt[5];  // transposed weights of layers 1-4 in the same layout
+    const float *bias[5];
+    // per hidden layer: Z (FP32, [column / 4][row][4]); A and dZ (BF16) with
+    // element (row, column) at ((row / 8) width + column) 8 + row % 8, as the
+    // input XT (width 16) and the output gradient dZoT (width 16)
+    float *Z[4];
+    __nv_bfloat16 *AT[4], *dZT[4], *XT, *dZoT;
+    float *dW[5], *dbias[5];  // gradients, weights row-major (out, in)
+    float *loss;
+    int *err;  // set to 1 if a wait timed out
+};
+cudaError_t launch_mlp_grad(const MlpTrain &f, cudaStream_t s);
 
 }  // namespace cvx

@@ -28,83 +28,17 @@
 
 #include <algorithm>
 
-#include "cvx_device.cuh"
-#include "cvx_mlp.h"
-#include "cvx_tc.cuh"
+#include "cvx_mlp_tile.cuh"
 
 namespace cvx {
 
 namespace {
 
-constexpr int kRows = 128, kWidth = 256, kOutPad = 16, kInPad = 16;
-constexpr int kRing = 4, kStageK = 32;                       // stages, k per stage
-constexpr int kStageBytes = kWidth * kStageK * 2;            // 16 KB
-constexpr int kABytes = kRows * kWidth * 2;                  // 64 KB
-constexpr int kW0Bytes = kWidth * kInPad * 2, kW4Bytes = kOutPad * kWidth * 2;
-constexpr int kBiasFloats = 4 * kWidth + kOutPad;
 constexpr size_t kSmem = 2 * kABytes + kRing * kStageBytes + kW0Bytes + kW4Bytes +
                          kBiasFloats * sizeof(float) + 1024;
 constexpr int kThreads = 640;
-constexpr uint64_t kWaitNs = 1000000000ull;  // 1 s per wait, then give up
-
-__device__ __forceinline__ float rcp_approx(float x) {
-    float y;
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-    return y;
-}
-// GELU z Phi(z) of two activations, erf from Abramowitz & Stegun, Handbook of
-// Mathematical Functions, formula 7.1.26 (|error| <= 1.5e-7), as in
-// cvx_gemm.cu, two values per instruction; packed to BF16.
-__device__ __forceinline__ uint32_t gelu2_bf16(f32x2 z) {
-    auto c2 = [](float c) { return pk2(c, c); };
-    float z0, z1, x0, x1;
-    upk2(z, z0, z1);
-    const f32x2 x = mul2(pk2(fabsf(z0), fabsf(z1)), c2(0.70710678118654752f));
-    float d0, d1;
-    upk2(fma2(c2(0.3275911f), x, c2(1.0f)), d0, d1);
-    const f32x2 t = pk2(rcp_approx(d0), rcp_approx(d1));
-    // minus the polynomial: all coefficients negated
-    f32x2 p = fma2(t, c2(-1.061405429f), c2(1.453152027f));
-    p = fma2(t, p, c2(-1.421413741f));
-    p = fma2(t, p, c2(0.284496736f));
-    p = mul2(t, fma2(t, p, c2(-0.254829592f)));
-    upk2(mul2(mul2(x, x), c2(-1.4426950408889634f)), x0, x1);
-    const f32x2 e = fma2(p, pk2(ex2_approx(x0), ex2_approx(x1)), c2(1.0f));  // erf(x)
-    float e0, e1;
-    upk2(e, e0, e1);
-    const f32x2 s = pk2(copysignf(e0, z0), copysignf(e1, z1));
-    float a0, a1;
-    upk2(mul2(z, fma2(c2(0.5f), s, c2(0.5f))), a0, a1);
-    const __nv_bfloat162 h = __floats2bfloat162_rn(a0, a1);
-    return *reinterpret_cast<const uint32_t *>(&h);
-}
 
 }  // namespace
-
-// Contiguous bytes, global to shared memory (both 16-byte aligned, a multiple
-// of 16 bytes).
-__device__ __forceinline__ void bulk_load(void *dst, const void *src, unsigned bytes, uint64_t *bar) {
-    asm volatile(
-        "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-            smem_u32(dst)),
-        "l"(src), "r"(bytes), "r"(smem_u32(bar))
-        : "memory");
-}
-
-// 32 consecutive FP32 columns of this thread's TMEM lane.
-__device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32]) {
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
-        "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
-        "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
-          "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]),
-          "=r"(r[14]), "=r"(r[15]), "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]),
-          "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]), "=r"(r[25]),
-          "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
-        : "r"(taddr));
-    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-}
 
 __global__ void __launch_bounds__(kThreads, 1)
     k_mlp_forward(const MlpForward f) {

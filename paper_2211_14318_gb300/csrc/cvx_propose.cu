@@ -258,7 +258,7 @@ int surrogate_propose(cvx_handle *h, const cvx_params *p, int64_t n, const doubl
     pp.counters = h->d_counters;
     const long long maxq = pp.K > 0 ? (n << (pp.K - 1)) : 0;
     const int chunk = (int)std::min<long long>(kChunk, std::max<long long>(maxq, 1));
-    rc = sur_batch(h, chunk);
+    rc = sur_rows(h, chunk);
     if (rc) return rc;
     Surrogate &S = *h->sur;
     // pageable source: returns once staged

@@ -1,6 +1,6 @@
 // cvx_surrogate.cu -- the surrogate proposal network: parameters, BF16
-// packing, the forward and backward passes as sequences of tensor-core GEMMs
-// (cvx_gemm.cu) with fused epilogues, the loss, Adam, training, save/load.
+// packing, Adam, training, save/load.  Inference is one kernel
+// (cvx_mlp_fused.cu), the loss and its gradient are two (cvx_mlp_train.cu).
 //
 // Network: x = standardised (F11, F12, F21, F22, beta_k, ln det F) ->
 // 4 x [256, GELU] -> 7 outputs (two direction angles, the logit of the volume
@@ -34,94 +34,35 @@ static_assert(kBOff[4] + 7 == kSurParams, "parameter layout");
 using bf16 = __nv_bfloat16;
 
 // ------------------------------------------------------------------ kernels
-// P (rows_pad x cols_pad) = W (out x in) zero-padded; T (cols_pad x rows_pad) =
-// P^T; B = P in k-blocks of 8 columns: (cols_pad / 8) x rows_pad x 8.
-__global__ void k_pack(const float *W, int out, int in, int rows_pad, int cols_pad, bf16 *P,
-                       bf16 *T, bf16 *B) {
-    const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= rows_pad * cols_pad) return;
-    const int r = idx / cols_pad, c = idx % cols_pad;
-    const float v = (r < out && c < in) ? W[(long long)r * in + c] : 0.0f;
-    const bf16 b = __float2bfloat16_rn(v);
-    if (P) P[(long long)r * cols_pad + c] = b;
-    if (T) T[(long long)c * rows_pad + r] = b;
-    B[((long long)(c >> 3) * rows_pad + r) * 8 + (c & 7)] = b;
-}
+struct Packed {
+    bf16 *W[5], *Wt[5];
+};
 
-// Standardised inputs of rows idx[m] (or m) -> X (n x 16, bf16, zero-padded)
-// and its transpose XT (16 x ldt); optional labels gathered the same way.
-__global__ void k_input(int n, const int *idx, const float *Xraw, const float *scale, bf16 *X,
-                        bf16 *XT, int ldt, const float *Yraw, float *Y) {
-    const int m = blockIdx.x * blockDim.x + threadIdx.x;
-    if (m >= n) return;
-    const long long src = idx ? idx[m] : m;
-    for (int k = 0; k < 16; ++k) {
-        const float v = k < 6 ? (Xraw[src * 6 + k] - scale[k]) * scale[6 + k] : 0.0f;
-        const bf16 b = __float2bfloat16_rn(v);
-        X[(long long)m * 16 + k] = b;
-        if (XT) XT[(long long)k * ldt + m] = b;
-    }
-    if (Y)
-        for (int k = 0; k < 7; ++k) Y[(long long)m * 7 + k] = Yraw[src * 7 + k];
-}
-
-// Loss of the batch (mean over its n samples) and dL/d(out), rounded to bf16
-// as the operand of the last layer's back-propagation (dZ, n x 16 and its
-// transpose); the output bias gradient from the unrounded values.
-__global__ void k_loss(int n, const float *out, const float *Y, bf16 *dZ, bf16 *dZT, int ldt,
-                       float *g_b4, float *loss) {
-    __shared__ float s_l[8], s_b[8][7];
-    const int m = blockIdx.x * blockDim.x + threadIdx.x;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const float inv_n = 1.0f / (float)n;
-    float L = 0.0f, g[7] = {0, 0, 0, 0, 0, 0, 0};
-    if (m < n) {
-        const float *o = out + (long long)m * 7;
-        const float *y = Y + (long long)m * 7;
-        if (!isnan(y[0])) {
-            for (int i = 0; i < 2; ++i) {
-                const float d = 2.0f * (o[i] - y[i]);
-                L += 1.0f - cosf(d);
-                g[i] = 2.0f * sinf(d);
-            }
-        }
-        if (!isnan(y[2])) {
-            const float s = 1.0f / (1.0f + expf(-o[2]));
-            L += (s - y[2]) * (s - y[2]);
-            g[2] = 2.0f * (s - y[2]) * s * (1.0f - s);
-        }
-        for (int j = 3; j < 7; ++j) {
-            const float d = o[j] - y[j];
-            L += d * d;
-            g[j] = 2.0f * d;
-        }
-        for (int j = 0; j < 16; ++j) {
-            const bf16 b = __float2bfloat16_rn(j < 7 ? g[j] * inv_n : 0.0f);
-            dZ[(long long)m * 16 + j] = b;
-            dZT[(long long)j * ldt + m] = b;
-        }
-    }
-    for (int o = 16; o; o >>= 1) L += __shfl_xor_sync(0xffffffffu, L, o);
-    for (int j = 0; j < 7; ++j)
-        for (int o = 16; o; o >>= 1) g[j] += __shfl_xor_sync(0xffffffffu, g[j], o);
-    if (lane == 0) {
-        s_l[warp] = L;
-        for (int j = 0; j < 7; ++j) s_b[warp][j] = g[j];
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        float a = 0.0f, b[7] = {0, 0, 0, 0, 0, 0, 0};
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) {
-            a += s_l[w];
-            for (int j = 0; j < 7; ++j) b[j] += s_b[w][j];
-        }
-        atomicAdd(loss, a * inv_n);
-        for (int j = 0; j < 7; ++j) atomicAdd(g_b4 + j, b[j] * inv_n);
+// Parameter i, if it is a weight, to its places in the packed operands: W[r][c]
+// of layer l as k-blocks of 8 columns x all rows (256; 16 for the last layer)
+// and W^T likewise (layers 1-4).  The padding stays zero.
+__device__ __forceinline__ void pack_weight(long long i, float w, const Packed &p) {
+#pragma unroll
+    for (int l = 0; l < 5; ++l) {
+        const int in = l ? 256 : 6, out = l < 4 ? 256 : 7;
+        constexpr long long kOff[5] = {0, 1792, 67584, 133376, 199168};  // kWOff
+        const long long k = i - kOff[l];
+        if (k < 0 || k >= (long long)in * out) continue;
+        const int r = (int)(k / in), c = (int)(k % in);
+        const bf16 b = __float2bfloat16_rn(w);
+        p.W[l][((c >> 3) * (l < 4 ? 256 : 16) + r) * 8 + (c & 7)] = b;
+        if (l) p.Wt[l][((r >> 3) * 256 + c) * 8 + (r & 7)] = b;
     }
 }
 
+__global__ void k_pack(long long n, const float *w, Packed p) {
+    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < n) pack_weight(i, w[i], p);
+}
+
+// One Adam step, and the packed weights of the result.
 __global__ void k_adam(long long n, float *w, const float *g, float *m, float *v, float lr,
-                       float b1, float b2, float eps, float c1, float c2) {
+                       float b1, float b2, float eps, float c1, float c2, Packed p) {
     const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     const float gi = g[i];
@@ -129,7 +70,9 @@ __global__ void k_adam(long long n, float *w, const float *g, float *m, float *v
     const float vi = b2 * v[i] + (1.0f - b2) * gi * gi;
     m[i] = mi;
     v[i] = vi;
-    w[i] -= lr * (mi / c1) / (sqrtf(vi / c2) + eps);
+    const float wi = w[i] - lr * (mi / c1) / (sqrtf(vi / c2) + eps);
+    w[i] = wi;
+    pack_weight(i, wi, p);
 }
 
 template <typename T>
@@ -142,22 +85,17 @@ cudaError_t alloc(T **p, size_t count) {
 void destroy_surrogate(cvx_handle *h) {
     Surrogate *S = h->sur;
     if (!S) return;
-    void *ptrs[] = {S->scale, S->w, S->g, S->m, S->v, S->X, S->XT, S->dZo, S->dZoT, S->out, S->Yb,
-                    S->loss, S->err, S->idx};
+    void *ptrs[] = {S->scale, S->w, S->g, S->m, S->v, S->X, S->out, S->XT, S->dZoT, S->loss, S->err,
+                    S->idx};
     for (void *p : ptrs) cudaFree(p);
     for (int l = 0; l < 5; ++l) {
-        cudaFree(S->Wp[l]);
-        cudaFree(S->Wt[l]);
         cudaFree(S->Wb[l]);
+        cudaFree(S->Wt[l]);
     }
     for (int l = 0; l < 4; ++l) {
-        cudaFree(S->A[l]);
         cudaFree(S->AT[l]);
-        cudaFree(S->Z[l]);
-    }
-    for (int l = 0; l < 2; ++l) {
-        cudaFree(S->dZ[l]);
         cudaFree(S->dZT[l]);
+        cudaFree(S->Z[l]);
     }
     delete S;
     h->sur = nullptr;
@@ -175,83 +113,75 @@ int sur_params(cvx_handle *h) {
     CK(alloc(&S.loss, 1), "surrogate");
     CK(alloc(&S.err, 1), "surrogate");
     CK(cudaMemset(S.err, 0, sizeof(int)), "surrogate");
-    CK(alloc(&S.Wp[0], 256 * 16), "surrogate");
-    for (int l = 1; l < 4; ++l) {
-        CK(alloc(&S.Wp[l], 256 * 256), "surrogate");
-        CK(alloc(&S.Wt[l], 256 * 256), "surrogate");
+    for (int l = 0; l < 5; ++l) {
+        const size_t n = l == 0 || l == 4 ? 256 * 16 : 256 * 256;
+        CK(alloc(&S.Wb[l], n), "surrogate");
+        CK(cudaMemset(S.Wb[l], 0, sizeof(bf16) * n), "surrogate");
+        CK(alloc(&S.Wt[l], n), "surrogate");
+        CK(cudaMemset(S.Wt[l], 0, sizeof(bf16) * n), "surrogate");
     }
-    CK(alloc(&S.Wp[4], 16 * 256), "surrogate");
-    CK(alloc(&S.Wt[4], 256 * 16), "surrogate");
-    for (int l = 0; l < 5; ++l) CK(alloc(&S.Wb[l], l == 0 ? 256 * 16 : (l < 4 ? 256 * 256 : 16 * 256)), "surrogate");
     return CVX_OK;
 }
 
-int sur_batch(cvx_handle *h, int n) {
+int sur_rows(cvx_handle *h, int n) {
     Surrogate &S = *h->sur;
-    if (n <= S.cap) return CVX_OK;
-    const int cap = ((n + 127) / 128) * 128;
+    if (n <= S.rows_cap) return CVX_OK;
+    const size_t cap = (size_t)((n + 127) / 128) * 128;
     cudaDeviceSynchronize();
-    bf16 **b16[] = {&S.X, &S.XT, &S.dZo, &S.dZoT};
-    for (auto p : b16) {
-        cudaFree(*p);
-        *p = nullptr;
-    }
-    for (int l = 0; l < 4; ++l) {
-        cudaFree(S.A[l]);
-        cudaFree(S.AT[l]);
-        cudaFree(S.Z[l]);
-    }
-    for (int l = 0; l < 2; ++l) {
-        cudaFree(S.dZ[l]);
-        cudaFree(S.dZT[l]);
-    }
+    cudaFree(S.X);
     cudaFree(S.out);
-    cudaFree(S.Yb);
-    S.cap = 0;
-    CK(alloc(&S.X, (size_t)cap * 16), "surrogate batch");
-    CK(alloc(&S.XT, (size_t)cap * 16), "surrogate batch");
-    CK(alloc(&S.dZo, (size_t)cap * 16), "surrogate batch");
-    CK(alloc(&S.dZoT, (size_t)cap * 16), "surrogate batch");
-    for (int l = 0; l < 4; ++l) {
-        CK(alloc(&S.A[l], (size_t)cap * 256), "surrogate batch");
-        CK(alloc(&S.AT[l], (size_t)cap * 256), "surrogate batch");
-        CK(alloc(&S.Z[l], (size_t)cap * 256), "surrogate batch");
-    }
-    for (int l = 0; l < 2; ++l) {
-        CK(alloc(&S.dZ[l], (size_t)cap * 256), "surrogate batch");
-        CK(alloc(&S.dZT[l], (size_t)cap * 256), "surrogate batch");
-    }
-    CK(alloc(&S.out, (size_t)cap * 7), "surrogate batch");
-    CK(alloc(&S.Yb, (size_t)cap * 7), "surrogate batch");
-    S.cap = cap;
+    S.X = nullptr;
+    S.out = nullptr;
+    S.rows_cap = 0;
+    CK(alloc(&S.X, cap * 16), "surrogate rows");
+    CK(alloc(&S.out, cap * 7), "surrogate rows");
+    S.rows_cap = (int)cap;
     return CVX_OK;
 }
 
 namespace {
 
-cudaError_t sur_pack(Surrogate &S, cudaStream_t s) {
-    const int rp[5] = {256, 256, 256, 256, 16}, cp[5] = {16, 256, 256, 256, 256};
-    for (int l = 0; l < 5; ++l) {
-        const int total = rp[l] * cp[l];
-        k_pack<<<(total + 255) / 256, 256, 0, s>>>(S.w + kWOff[l], kOut[l], kIn[l], rp[l], cp[l],
-                                                   S.Wp[l], l ? S.Wt[l] : nullptr, S.Wb[l]);
+// Training buffers for at least n rows.
+int sur_batch(cvx_handle *h, int n) {
+    Surrogate &S = *h->sur;
+    if (n <= S.cap) return CVX_OK;
+    const size_t cap = (size_t)((n + 127) / 128) * 128;
+    cudaDeviceSynchronize();
+    cudaFree(S.XT);
+    cudaFree(S.dZoT);
+    S.XT = S.dZoT = nullptr;
+    for (int l = 0; l < 4; ++l) {
+        cudaFree(S.AT[l]);
+        cudaFree(S.dZT[l]);
+        cudaFree(S.Z[l]);
+        S.AT[l] = S.dZT[l] = nullptr;
+        S.Z[l] = nullptr;
     }
+    S.cap = 0;
+    CK(alloc(&S.XT, cap * 16), "surrogate batch");
+    CK(alloc(&S.dZoT, cap * 16), "surrogate batch");
+    for (int l = 0; l < 4; ++l) {
+        CK(alloc(&S.AT[l], cap * 256), "surrogate batch");
+        CK(alloc(&S.dZT[l], cap * 256), "surrogate batch");
+        CK(alloc(&S.Z[l], cap * 256), "surrogate batch");
+    }
+    S.cap = (int)cap;
+    return CVX_OK;
+}
+
+Packed packed(const Surrogate &S) {
+    Packed p;
+    for (int l = 0; l < 5; ++l) {
+        p.W[l] = S.Wb[l];
+        p.Wt[l] = S.Wt[l];
+    }
+    return p;
+}
+
+cudaError_t sur_pack(Surrogate &S, cudaStream_t s) {
+    k_pack<<<(kSurParams + 255) / 256, 256, 0, s>>>(kSurParams, S.w, packed(S));
     return cudaGetLastError();
 }
-
-GemmEpi epi(int mode, int Mv, int *err) {
-    GemmEpi e = {};
-    e.mode = mode;
-    e.M_valid = Mv;
-    e.err = err;
-    return e;
-}
-
-#define TMAP(map, ptr, rows, cols, ld, box)                                           \
-    do {                                                                              \
-        if (!make_tmap_bf16(&(map), (ptr), (rows), (cols), (ld), (box)))              \
-            return fail(CVX_ERR_CUDA, "tensor map for %s failed", #ptr);              \
-    } while (0)
 
 }  // namespace
 
@@ -280,100 +210,35 @@ int sur_infer(cvx_handle *h, int n, const float *X, float *out, cudaStream_t s, 
 
 namespace {
 
-// Forward pass of n <= cap standardised rows in S.X (and S.XT), layer by layer,
-// keeping Z, A and A^T for the backward pass.
-int sur_forward(cvx_handle *h, int n, cudaStream_t s) {
+// Loss and gradient (added to loss and g, 16-byte aligned) of n <= cap samples,
+// row m being sample idx[m] (or m).
+int sur_grad(cvx_handle *h, int n, const int *idx, const float *X, const float *Y, float *loss,
+             float *g, cudaStream_t s) {
     Surrogate &S = *h->sur;
-    CUtensorMap tX, tW, tA;
-    TMAP(tX, S.X, n, 16, 16, 128);
-    TMAP(tW, S.Wp[0], 256, 16, 16, 256);
-    GemmEpi e = epi(EPI_HIDDEN, n, S.err);
-    e.bias = S.w + kBOff[0];
-    e.Z = S.Z[0];
-    e.ldz = 256;
-    e.A = S.A[0];
-    e.lda = 256;
-    e.AT = S.AT[0];
-    e.ldat = S.cap;
-    CK(launch_gemm(tX, tW, n, 256, 16, 16, 256, e, s), "surrogate forward");
-    for (int l = 1; l < 4; ++l) {
-        TMAP(tA, S.A[l - 1], n, 256, 256, 128);
-        TMAP(tW, S.Wp[l], 256, 256, 256, 256);
-        e.bias = S.w + kBOff[l];
-        e.Z = S.Z[l];
-        e.A = S.A[l];
-        e.AT = S.AT[l];
-        CK(launch_gemm(tA, tW, n, 256, 256, 256, 256, e, s), "surrogate forward");
+    MlpTrain f = {};
+    f.n = n;
+    f.ld = S.cap;
+    f.idx = idx;
+    f.X = X;
+    f.Y = Y;
+    f.scale = S.scale;
+    for (int l = 0; l < 5; ++l) {
+        f.W[l] = S.Wb[l];
+        f.Wt[l] = S.Wt[l];
+        f.bias[l] = S.w + kBOff[l];
+        f.dW[l] = g + kWOff[l];
+        f.dbias[l] = g + kBOff[l];
     }
-    TMAP(tA, S.A[3], n, 256, 256, 128);
-    TMAP(tW, S.Wp[4], 16, 256, 256, 16);
-    GemmEpi o = epi(EPI_OUT, n, S.err);
-    o.C = S.out;
-    o.ldc = 7;
-    o.n_store = 7;
-    o.bias = S.w + kBOff[4];
-    CK(launch_gemm(tA, tW, n, 16, 256, 256, 16, o, s), "surrogate forward");
-    return CVX_OK;
-}
-
-// Loss and gradient (added to S.g) of the batch in S.X / S.Yb after
-// sur_forward(train = true).
-int sur_backward(cvx_handle *h, int n, cudaStream_t s) {
-    Surrogate &S = *h->sur;
-    const int ld = S.cap;
-    k_loss<<<(n + 255) / 256, 256, 0, s>>>(n, S.out, S.Yb, S.dZo, S.dZoT, ld, S.g + kBOff[4],
-                                           S.loss);
-    CK(cudaGetLastError(), "surrogate loss");
-    const int K = ((n + 15) / 16) * 16;
-    const int ks = 1024;
-    CUtensorMap ta, tb;
-    // last layer: dW4 = dZo^T A4, dZ4 = (dZo W4) * gelu'(Z4)
-    TMAP(ta, S.dZoT, 16, n, ld, 128);
-    TMAP(tb, S.AT[3], 256, n, ld, 256);
-    GemmEpi w = epi(EPI_DW, 16, S.err);
-    w.C = S.g + kWOff[4];
-    w.ldc = 256;
-    w.m_store = 7;
-    w.n_store = 256;
-    CK(launch_gemm(ta, tb, 16, 256, K, ks, 256, w, s), "surrogate backward");
-    TMAP(ta, S.dZo, n, 16, 16, 128);
-    TMAP(tb, S.Wt[4], 256, 16, 16, 256);
-    GemmEpi d = epi(EPI_DA, n, S.err);
-    d.Z = S.Z[3];
-    d.ldz = 256;
-    d.A = S.dZ[0];
-    d.lda = 256;
-    d.AT = S.dZT[0];
-    d.ldat = ld;
-    d.dbias = S.g + kBOff[3];
-    CK(launch_gemm(ta, tb, n, 256, 16, 16, 256, d, s), "surrogate backward");
-    int cur = 0;
-    for (int l = 3; l >= 1; --l) {
-        // dW_l = dZ_{l+1}^T A_l (A_l = output of hidden layer l)
-        TMAP(ta, S.dZT[cur], 256, n, ld, 128);
-        TMAP(tb, S.AT[l - 1], 256, n, ld, 256);
-        w.C = S.g + kWOff[l];
-        w.m_store = 256;
-        w.M_valid = 256;
-        CK(launch_gemm(ta, tb, 256, 256, K, ks, 256, w, s), "surrogate backward");
-        // dZ_l = (dZ_{l+1} W_l) * gelu'(Z_l)
-        TMAP(ta, S.dZ[cur], n, 256, 256, 128);
-        TMAP(tb, S.Wt[l], 256, 256, 256, 256);
-        d.Z = S.Z[l - 1];
-        d.A = S.dZ[cur ^ 1];
-        d.AT = S.dZT[cur ^ 1];
-        d.dbias = S.g + kBOff[l - 1];
-        CK(launch_gemm(ta, tb, n, 256, 256, 256, 256, d, s), "surrogate backward");
-        cur ^= 1;
+    for (int l = 0; l < 4; ++l) {
+        f.Z[l] = S.Z[l];
+        f.AT[l] = S.AT[l];
+        f.dZT[l] = S.dZT[l];
     }
-    // dW0 = dZ_1^T X
-    TMAP(ta, S.dZT[cur], 256, n, ld, 128);
-    TMAP(tb, S.XT, 16, n, ld, 16);
-    w.C = S.g + kWOff[0];
-    w.ldc = 6;
-    w.m_store = 256;
-    w.n_store = 6;
-    CK(launch_gemm(ta, tb, 256, 16, K, ks, 16, w, s), "surrogate backward");
+    f.XT = S.XT;
+    f.dZoT = S.dZoT;
+    f.loss = loss;
+    f.err = S.err;
+    CK(launch_mlp_grad(f, s), "surrogate gradient");
     return CVX_OK;
 }
 
@@ -434,14 +299,16 @@ int cvx_gemm_bf16(cvx_handle *h, int M, int N, int K, const uint16_t *A, const u
     DeviceGuard g(h->device);
     CUtensorMap ta, tb;
     const int BN = N <= 16 ? 16 : 256;
-    TMAP(ta, A, M, K, K, 128);
-    TMAP(tb, B, N, K, K, BN);
+    if (!make_tmap_bf16(&ta, A, M, K, K, 128) || !make_tmap_bf16(&tb, B, N, K, K, BN))
+        return fail(CVX_ERR_CUDA, "cvx_gemm_bf16: tensor map failed");
     int rc = sur_params(h);
     if (rc) return rc;
-    GemmEpi e = epi(EPI_F32, M, h->sur->err);
+    GemmEpi e = {};
+    e.M_valid = M;
+    e.err = h->sur->err;
     e.C = C;
     e.ldc = N;
-    CK(launch_gemm(ta, tb, M, N, K, ((K + 63) / 64) * 64, BN, e, (cudaStream_t)sv), "cvx_gemm_bf16");
+    CK(launch_gemm(ta, tb, M, N, K, BN, e, (cudaStream_t)sv), "cvx_gemm_bf16");
     return check_err(*h->sur, (cudaStream_t)sv);
 }
 
@@ -500,17 +367,15 @@ int surrogate_loss_grad(cvx_handle *h, int64_t n, const float *X, const float *Y
     Surrogate &S = *h->sur;
     int rc = sur_batch(h, (int)n);
     if (rc) return rc;
-    k_input<<<((int)n + 255) / 256, 256, 0, s>>>((int)n, nullptr, X, S.scale, S.X, S.XT, S.cap, Y,
-                                                 S.Yb);
-    CK(cudaGetLastError(), "surrogate_loss_grad");
-    CK(cudaMemsetAsync(S.g, 0, sizeof(float) * kSurParams, s), "surrogate_loss_grad");
-    CK(cudaMemsetAsync(S.loss, 0, sizeof(float), s), "surrogate_loss_grad");
-    rc = sur_forward(h, (int)n, s);
+    // straight into the caller's gradient where its alignment allows the paired
+    // additions
+    float *g_out = ((uintptr_t)grad & 15) == 0 ? grad : S.g;
+    CK(cudaMemsetAsync(g_out, 0, sizeof(float) * kSurParams, s), "surrogate_loss_grad");
+    CK(cudaMemsetAsync(loss, 0, sizeof(float), s), "surrogate_loss_grad");
+    rc = sur_grad(h, (int)n, nullptr, X, Y, loss, g_out, s);
     if (rc) return rc;
-    rc = sur_backward(h, (int)n, s);
-    if (rc) return rc;
-    CK(cudaMemcpyAsync(grad, S.g, sizeof(float) * kSurParams, cudaMemcpyDeviceToDevice, s), "surrogate_loss_grad");
-    CK(cudaMemcpyAsync(loss, S.loss, sizeof(float), cudaMemcpyDeviceToDevice, s), "surrogate_loss_grad");
+    if (g_out != grad)
+        CK(cudaMemcpyAsync(grad, S.g, sizeof(float) * kSurParams, cudaMemcpyDeviceToDevice, s), "surrogate_loss_grad");
     return check_err(S, s);
 }
 
@@ -566,17 +431,13 @@ int surrogate_train(cvx_handle *h, int64_t n, const float *X, const float *Y,
         int batches = 0;
         for (int64_t o = 0; o + B <= n || (o == 0 && n < B); o += B) {
             const int m = (int)std::min<int64_t>(B, n - o);
-            k_input<<<(m + 255) / 256, 256, 0, s>>>(m, S.idx + o, X, S.scale, S.X, S.XT, S.cap, Y, S.Yb);
-            CK(cudaGetLastError(), "surrogate_train");
             CK(cudaMemsetAsync(S.g, 0, sizeof(float) * kSurParams, s), "surrogate_train");
-            rc = sur_forward(h, m, s);
-            if (rc) return rc;
-            rc = sur_backward(h, m, s);
+            rc = sur_grad(h, m, S.idx + o, X, Y, S.loss, S.g, s);
             if (rc) return rc;
             ++S.adam_t;
             const float c1 = 1.0f - powf(b1, (float)S.adam_t), c2 = 1.0f - powf(b2, (float)S.adam_t);
-            k_adam<<<(kSurParams + 255) / 256, 256, 0, s>>>(kSurParams, S.w, S.g, S.m, S.v, cfg->lr, b1, b2, eps, c1, c2);
-            CK(sur_pack(S, s), "surrogate_train");
+            k_adam<<<(kSurParams + 255) / 256, 256, 0, s>>>(kSurParams, S.w, S.g, S.m, S.v, cfg->lr, b1, b2, eps, c1, c2, packed(S));
+            CK(cudaGetLastError(), "surrogate_train");
             ++batches;
             if (n < B) break;
         }

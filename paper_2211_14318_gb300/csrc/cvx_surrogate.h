@@ -21,13 +21,14 @@ struct Surrogate {
     float scale_h[12];  // mean (6), 1/std (6)
     float *scale = nullptr;
     float *w = nullptr, *g = nullptr, *m = nullptr, *v = nullptr;
-    __nv_bfloat16 *Wp[5] = {}, *Wt[5] = {};
-    __nv_bfloat16 *Wb[5] = {};  // packed weights as k-blocks (MlpForward::W)
+    __nv_bfloat16 *Wb[5] = {}, *Wt[5] = {};  // packed weights (MlpForward::W, MlpTrain::Wt)
     long long adam_t = 0;
-    int cap = 0;
-    __nv_bfloat16 *X = nullptr, *XT = nullptr, *A[4] = {}, *AT[4] = {}, *dZo = nullptr,
-                  *dZoT = nullptr, *dZ[2] = {}, *dZT[2] = {};
-    float *Z[4] = {}, *out = nullptr, *Yb = nullptr, *loss = nullptr;
+    int rows_cap = 0;  // rows of X and out (surrogate_propose)
+    __nv_bfloat16 *X = nullptr;
+    float *out = nullptr;
+    int cap = 0;  // rows of the training buffers (MlpTrain)
+    __nv_bfloat16 *XT = nullptr, *dZoT = nullptr, *AT[4] = {}, *dZT[4] = {};
+    float *Z[4] = {}, *loss = nullptr;
     int *err = nullptr;
     int *idx = nullptr;
     long long idx_cap = 0;
@@ -35,8 +36,8 @@ struct Surrogate {
 
 void destroy_surrogate(cvx_handle *h);
 int sur_params(cvx_handle *h);
-// Batch buffers for at least n rows.
-int sur_batch(cvx_handle *h, int n);
+// Input and output rows of surrogate_propose's nodes, at least n.
+int sur_rows(cvx_handle *h, int n);
 int sur_infer(cvx_handle *h, int n, const float *X, float *out, cudaStream_t s, const int *M_dev,
               int m_off);
 

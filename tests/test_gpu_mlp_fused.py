@@ -29,3 +29,49 @@ def test_forward_row_counts(cv, orc, n):  # noqa: F811
     r = ref[:first.shape[0]]
     assert np.max(np.abs(first - r) / (1 + np.abs(r))) < 2e-3
     assert np.array_equal(out, out[:2048][at])
+
+
+@pytest.mark.parametrize("n", [1, 30, 127, 129, 1024, 152 * 128 + 1, 2 * 152 * 128 + 77])
+@pytest.mark.parametrize("aligned", [True, False])
+def test_gradient_row_counts(cv, orc, n, aligned):  # noqa: F811
+    """Loss and gradient over part of a tile, several slices of the weight
+    gradients and a last turn of one tile; into a gradient buffer at any
+    float address.  Bars of test_gpu_surrogate."""
+    import ctypes
+
+    import torch
+
+    from paper_2211_14318_gb300 import api
+
+    X, mean, std = _net_inputs(orc, 2048, 33)
+    flat = _set(cv, 10)
+    cv.surrogate_set_weights(flat, mean, std)
+    rng = np.random.default_rng(n)
+    at = np.arange(n) % 2048
+    Y = np.column_stack([rng.uniform(0, np.pi, (n, 2)), rng.uniform(0.05, 0.95, n),
+                         rng.normal(0, 0.3, (n, 4))]).astype(np.float32)
+    Y[::5, :3] = np.nan
+    Xd, Yd = torch.from_numpy(X.astype(np.float32)[at]).cuda(), torch.from_numpy(Y).cuda()
+    if aligned:
+        loss, grad = cv.surrogate_loss_grad(Xd, Yd)
+    else:
+        loss = torch.empty(1, device="cuda")
+        grad = torch.empty(api.SURROGATE_PARAMS + 1, device="cuda")[1:]
+        rc = api.lib().surrogate_loss_grad(cv._h, ctypes.c_int64(n), Xd.data_ptr(), Yd.data_ptr(),
+                                           loss.data_ptr(), grad.data_ptr(),
+                                           torch.cuda.current_stream().cuda_stream)
+        assert rc == 0
+    g = grad.cpu().numpy().astype(np.float64)
+    istd = (1.0 / std.astype(np.float32)).astype(np.float32).astype(np.float64)
+    out, cache = mlp.forward(flat, X.astype(np.float32).astype(np.float64)[at], mean, 1.0 / istd, bf=True)
+    L, dout = mlp.loss_and_grad(out, Y.astype(np.float64))
+    ref = mlp.backward(flat, cache, dout, bf=True)
+    assert abs(loss.item() - L) < 1e-3 * (1 + abs(L))
+    o = 0
+    for shp in mlp.SHAPES:
+        k = int(np.prod(shp))
+        a, b = g[o:o + k], ref[o:o + k]
+        rel = np.linalg.norm(a - b) / (np.linalg.norm(b) + 1e-30)
+        cos = a @ b / (np.linalg.norm(a) * np.linalg.norm(b) + 1e-30)
+        assert rel < 2e-2 and cos > 0.9995, (shp, rel, cos)
+        o += k
