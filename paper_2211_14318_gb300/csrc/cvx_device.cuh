@@ -410,6 +410,12 @@ __device__ __forceinline__ NHPair nh_pair_node(const NodeLine &nl) {
     c.A1 = c.A2 = c.CJ = c.J0 = c.A0;
     return c;
 }
+// d + K2' min(d, 0) with min(d, 0) = d - max(d, 0), exact, one paired addition
+// instead of two minima (d = +inf, J = 0, gives NaN instead of +inf: no sample
+// either way).
+__device__ __forceinline__ f32x2 nh_branch2(const NHPair &c, f32x2 D, float m0, float m1) {
+    return fma2(c.K2, add2(D, pk2(-m0, -m1)), D);
+}
 __device__ __forceinline__ f32x2 sample_nh2(const NHPair &c, f32x2 T) {
     const f32x2 P = fma2(T, fma2(T, c.A2, c.A1), c.A0);
     float j0, j1;
@@ -418,9 +424,9 @@ __device__ __forceinline__ f32x2 sample_nh2(const NHPair &c, f32x2 T) {
     const f32x2 D = fma2(LG, fma2(LG, c.B2, c.B1), P);
     float d0, d1;
     upk2(D, d0, d1);
-    const f32x2 E = pk2(ex2_approx(-fmaxf(d0, 0.0f)), ex2_approx(-fmaxf(d1, 0.0f)));
-    const f32x2 W = fma2(c.K2, pk2(fminf(d0, 0.0f), fminf(d1, 0.0f)), D);
-    return fma2(c.NK1, E, W);
+    const float m0 = fmaxf(d0, 0.0f), m1 = fmaxf(d1, 0.0f);
+    const f32x2 E = pk2(ex2_approx(-m0), ex2_approx(-m1));
+    return fma2(c.NK1, E, nh_branch2(c, D, m0, m1));
 }
 
 // energy64 of the damage energy with the node's e_k = exp(-beta_k / D_0)

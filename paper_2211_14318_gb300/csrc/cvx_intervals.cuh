@@ -90,10 +90,10 @@ __device__ __forceinline__ void iv_eval(const NHPair &c, f32x2 H, f32x2 NS, f32x
     const f32x2 LG = pk2(lg2_approx(j0), lg2_approx(j1));
     const f32x2 D = fma2(LG, fma2(LG, c.B2, c.B1), P);
     upk2(D, d0, d1);
-    E0 = ex2_approx(-fmaxf(d0, 0.0f));
-    E1 = ex2_approx(-fmaxf(d1, 0.0f));
-    const f32x2 W = fma2(c.K2, pk2(fminf(d0, 0.0f), fminf(d1, 0.0f)), D);
-    upk2(fma2(NS, X, fma2(c.NK1, pk2(E0, E1), W)), g0, g1);
+    const float m0 = fmaxf(d0, 0.0f), m1 = fmaxf(d1, 0.0f);
+    E0 = ex2_approx(-m0);
+    E1 = ex2_approx(-m1);
+    upk2(fma2(NS, X, fma2(c.NK1, pk2(E0, E1), nh_branch2(c, D, m0, m1))), g0, g1);
 }
 
 // Intervals (a mask) of the region from sample xb (value ga, Ea) to fl with
@@ -144,6 +144,58 @@ __device__ __forceinline__ unsigned iv_sweep(const IvLine &l, const IvGeom &G, f
         }
     }
     return mask & (NI >= 32 ? 0xffffffffu : (1u << NI) - 1u);
+}
+
+// Second derivative of v on [t0, t1]: +1 and a positive lower bound `low` of
+// v'' if it is positive there, -1 if it is negative, 0 if undecided.  With E =
+// 2^{-max(d, 0)}, v'' = d'' + K2' E (d'' - ln 2 d'^2 [d > 0]).  d'' lies
+// between its values for the smallest and the largest J; where it is positive
+// |d'| is largest at an end, and d lies at most max(d'') (t1 - t0)^2 / 8
+// below its end values.  The margins (1e-4 of the terms' magnitudes, 1e-5 of
+// those of d') are far above the FP32 rounding.
+__device__ __forceinline__ int line_shape(const IvLine &l, float t0, float t1, float &low) {
+    float A0, A1, B1, B2, u;
+    upk2(l.c.A0, A0, u);
+    upk2(l.c.A1, A1, u);
+    upk2(l.c.B1, B1, u);
+    upk2(l.c.B2, B2, u);
+    const float Ja = __fmaf_rn(t0, l.cJ, l.J0), Jb = __fmaf_rn(t1, l.cJ, l.J0);
+    const float Jn = fminf(Ja, Jb), Jx = fmaxf(Ja, Jb);
+    if (!(Jn > 0.0f)) return 0;
+    const float lga = lg2_approx(Ja), lgb = lg2_approx(Jb);
+    const float lgn = fminf(lga, lgb), lgx = fmaxf(lga, lgb);
+    const float cn2 = (l.cJ / Jn) * (l.cJ / Jn), cx2 = (l.cJ / Jx) * (l.cJ / Jx);
+    const float fn = __fmaf_rn(-l.c1, lgn, l.c0), fx = __fmaf_rn(-l.c1, lgx, l.c0);
+    const float Dx = __fmaf_rn(cn2, fmaxf(fn, 0.0f), 2.0f * l.A2);
+    const float Dn = __fmaf_rn(fx >= 0.0f ? cx2 : cn2, fx, 2.0f * l.A2);
+    const float Dm = __fmaf_rn(cn2, fmaxf(fabsf(fn), fabsf(fx)), 2.0f * l.A2);
+    if (!(Dm < 1e30f)) return 0;
+    const float da = __fmaf_rn(lga, __fmaf_rn(lga, B2, B1), __fmaf_rn(t0, __fmaf_rn(t0, l.A2, A1), A0));
+    const float db = __fmaf_rn(lgb, __fmaf_rn(lgb, B2, B1), __fmaf_rn(t1, __fmaf_rn(t1, l.A2, A1), A0));
+    const float ka = l.cJ / Ja * (1.0f / kLn2), kb = l.cJ / Jb * (1.0f / kLn2);
+    const float ra = __fmaf_rn(2.0f * B2, lga, B1), rb = __fmaf_rn(2.0f * B2, lgb, B1);
+    const float pa = __fmaf_rn(ka, ra, __fmaf_rn(2.0f * l.A2, t0, A1));
+    const float pb = __fmaf_rn(kb, rb, __fmaf_rn(2.0f * l.A2, t1, A1));
+    const float mg = 1e-5f * (fabsf(A1) + 2.0f * l.A2 * fmaxf(fabsf(t0), fabsf(t1)) +
+                              fmaxf(fabsf(ka), fabsf(kb)) *
+                                  (fabsf(B1) + 2.0f * B2 * fmaxf(fabsf(lga), fabsf(lgb))));
+    const float eta = Dx * (t1 - t0) * (t1 - t0) * 0.125f;
+    const float dn = fminf(da, db) - eta;
+    const float Ex = dn > 0.0f ? 1.00001f * ex2_approx(-dn) : 1.0f;
+    const float Ke = l.K2 * fminf(Ex, 1.0f);
+    const float px = fmaxf(fabsf(pa), fabsf(pb)) + mg;
+    const float qx = kLn2 * px * px;
+    // v'' is linear in E: its lower bound at E = 0 or the largest E
+    low = Dn + Ke * fminf(0.0f, Dn - qx) - 1e-4f * (Dm + Ke * (Dm + qx));
+    if (Dn > 0.0f && low > 0.0f) return 1;
+    // concave: d > 0 throughout, |d'| from below
+    const float dmag = 1e-5f * (fabsf(A0) + fabsf(A1) * fmaxf(fabsf(t0), fabsf(t1)) + 1.0f);
+    if (!(dn > dmag) || !(Dn > 0.0f) || !(pa * pb > 0.0f)) return 0;
+    const float pn = fminf(fabsf(pa), fabsf(pb)) - mg;
+    if (!(pn > 0.0f)) return 0;
+    const float En = l.K2 * ex2_approx(-fmaxf(da, db)) * 0.9999f;
+    const float qn = kLn2 * pn * pn;
+    return Dx + En * (Dx - qn) < -1e-4f * (Dm + Ke * (Dm + qx)) ? -1 : 0;
 }
 
 }  // namespace cvx

@@ -263,6 +263,27 @@ __device__ bool flat_certificate(const LaneNode &N, const DirLine &dl, float4 d3
                               k1e * kLn2f * kLn2f * dpa * dpa * 0.5f);
     const float c1 = 16.0f * kU32 * (S1 + fabsf(s0));
     const float c2 = 16.0f * kU32 * (1.0f + N.d0abs) * S2;
+    // All near samples at once where v'' has a positive lower bound `low` on the
+    // near region: their remainder is at least low t^2 / 2, so if low h^2 / 2 >=
+    // 2 (c1 + c2) it exceeds twice the threshold at every |x| >= 1, and its FP32
+    // value (the threshold bounds its error) the threshold itself; d keeps its
+    // sign if the tangent's reach says so (d >= its tangent at 0, d convex) or,
+    // for d0 <= 0, the largest d'' does.  The loop below would accept each.
+    // (64 samples per line otherwise: 13.5 of 73 ms for 16,384 mesh points.)
+    {
+        float low;
+        const IvLine l = iv_line(N.nl, dl.A1, dl.A2, dl.cJ);
+        if (line_shape(l, (float)xl * h, (float)xr * h, low) > 0 &&
+            0.5f * low * h * h >= 2.0f * (c1 + c2)) {
+            const float tm = xm * h, reach = 1.001f * fabsf(dprime) * tm;
+            const float J = N.nl.J0 - fabsf(dl.cJ) * tm, r = dl.cJ / J;
+            const float dd = __fmaf_rn(r * r, fmaxf(__fmaf_rn(-l.c1, lg2_approx(J), l.c0), 0.0f), 2.0f * A2);
+            const float slack = 1e-5f * (N.d0abs + 1.0f);
+            if (d0 > 0.0f ? d0 - reach > slack
+                          : J > 0.0f && d0 + reach + 0.5f * dd * tm * tm < -slack)
+                return true;
+        }
+    }
     bool ok = true;
     for (int x = xl; x <= xr && ok; ++x) {
         if (x == 0) continue;
