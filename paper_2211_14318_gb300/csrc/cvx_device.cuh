@@ -440,6 +440,30 @@ __device__ inline double energy64_ek(const double F[4], double beta_k, double ek
     return (1.0 - m.Dinf) * (s - beta_k) + m.Dinf * m.D0 * (ek - exp(-s / m.D0));
 }
 
+// energy64 and stress64 at one F sharing the invariants and the exponentials
+// (ek = exp(-beta_k / D_0); the same operations on the same values).
+__device__ inline void energy_stress64(const double F[4], double beta_k, double ek,
+                                       const Material &m, double &W, double P[4]) {
+    if (m.energy == CVX_ENERGY_DOUBLE_WELL) {
+        W = energy64(F, beta_k, m);
+        stress64(F, beta_k, m, P);
+        return;
+    }
+    double lj, J;
+    const double s = psi0_nh64(F, m, &lj, &J);
+    if (!(J > 0.0)) {
+        W = P[0] = P[1] = P[2] = P[3] = nan("");
+        return;
+    }
+    const double es = s > beta_k ? exp(-s / m.D0) : ek;
+    if (s <= beta_k) W = (1.0 - m.Dinf * (1.0 - ek)) * (s - beta_k);
+    else W = (1.0 - m.Dinf) * (s - beta_k) + m.Dinf * m.D0 * (ek - es);
+    const double g = 1.0 - m.Dinf * (1.0 - es);
+    const double iJ = 1.0 / J;
+    const double FiT[4] = {F[3] * iJ, -F[2] * iJ, -F[1] * iJ, F[0] * iJ};  // F^{-T}
+    for (int k = 0; k < 4; ++k) P[k] = g * (m.mu * (F[k] - FiT[k]) + m.lam * lj * FiT[k]);
+}
+
 // FP64 sample of W along the line: G = F + t R with t = (m - m0) h and R, G
 // rounded exactly as the split points are (no contraction).
 __device__ __forceinline__ double sample_w64(const double F[4], const double R[4], int m, int m0,
