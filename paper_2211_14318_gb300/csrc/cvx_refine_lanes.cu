@@ -17,7 +17,12 @@
 //  - elsewhere every sample whose FP32 value is inconclusive is taken.
 // Samples on or below the chord move the pair to the lowest one of its side
 // (the supporting-slope iteration; ties to the outermost sample, as in
-// Algorithm 1); a side whose neighbours fail is searched in full first.
+// Algorithm 1).  The scan's pair is that of FP32 samples, on nearly affine
+// lines up to 64 samples off: an end in a convex run first goes to where v has
+// the chord's slope (a Newton step in FP32, twice at most), and a neighbour
+// found on or below the chord is moved to (three times at most) before its
+// side is searched in full.  None of these decides anything: the pair is done
+// when the intervals and samples above say so for its own chord.
 //
 // The samples to be taken in FP64 queue in shared memory over the warp's 32
 // candidates and are taken 32 at a time, one per lane.  What bounds the
@@ -36,6 +41,10 @@ namespace cvx {
 namespace {
 
 constexpr int kRefWarps = 4;
+// Newton steps and neighbour moves per candidate.  Without them a candidate of
+// a load step's proposal windows took 29 FP64 samples beside its chords' ends,
+// with them 2 (k_refine_lanes 15.9 -> 5.2 ms of a step).
+constexpr int kRefJumps = 2, kRefWalks = 3;
 constexpr int kRefRounds = 24;  // chords per candidate before the whole line is taken in FP64
 
 // A lane's candidate as the queue's other lanes need it.
@@ -137,6 +146,25 @@ __device__ __noinline__ void ref_full(const RefLane &r, int L, int lane, int &a,
     }
 }
 
+// Samples from t to where v has slope ls per sample, by one Newton step in FP32
+// (v' and v'' from the line's constants, so their error is relative to them and
+// not to v).  Only a guess: the samples decide.
+__device__ __forceinline__ float tangent_step(const IvLine &l, float t, float h, float ls) {
+    float A0, A1, B1, B2, u;
+    upk2(l.c.A0, A0, u);
+    upk2(l.c.A1, A1, u);
+    upk2(l.c.B1, B1, u);
+    upk2(l.c.B2, B2, u);
+    const float J = __fmaf_rn(t, l.cJ, l.J0), lg = lg2_approx(J), r = __fdividef(l.cJ, J);
+    const float d = __fmaf_rn(lg, __fmaf_rn(lg, B2, B1), __fmaf_rn(t, __fmaf_rn(t, l.A2, A1), A0));
+    const float d1 = __fmaf_rn(r * (1.0f / kLn2), __fmaf_rn(2.0f * B2, lg, B1), __fmaf_rn(2.0f * l.A2, t, A1));
+    const float d2 = __fmaf_rn(r * r, __fmaf_rn(-l.c1, lg, l.c0), 2.0f * l.A2);
+    const float E = l.K2 * ex2_approx(-fmaxf(d, 0.0f));
+    const float v1 = h * __fmaf_rn(E, d1, d1);
+    const float v2 = h * h * (d > 0.0f ? __fmaf_rn(E, d2 - kLn2 * d1 * d1, d2) : __fmaf_rn(E, d2, d2));
+    return __fdividef(ls - v1, v2);
+}
+
 }  // namespace
 
 // One warp takes 32 candidates at a time: phase 0 each node's first candidate,
@@ -146,8 +174,8 @@ __device__ __noinline__ void ref_full(const RefLane &r, int L, int lane, int &a,
 // with 32 or 64 FP64 samples in two windows and the certificate over every
 // FP32 sample: 1,706,177 candidates at L = 201: 22.3 -> 1.25 ms (one spot
 // sample each); 1,809,226 candidates of a load
-// step's proposal windows at L = 2049, nearly affine lines: 47.5 -> 15.9 ms
-// (29 spot samples each); 110 candidates: 474 -> 48 us over four launches.
+// step's proposal windows at L = 2049, nearly affine lines: 47.5 -> 5.2 ms (2
+// each); 110 candidates: 474 -> 48 us over four launches.
 __global__ void __launch_bounds__(32 * kRefWarps) k_refine_lanes(const Pipe P, int level, int phase) {
     __shared__ RefLane s_rl[kRefWarps][32];
     __shared__ int s_q[kRefWarps][96];
@@ -233,6 +261,7 @@ __global__ void __launch_bounds__(32 * kRefWarps) k_refine_lanes(const Pipe P, i
         bool slow = act && !(hab >= 0 && a < m0 && b > m0 && b < L);
         bool done = !act || slow;
         bool newA = true, newB = true, fullL = false, fullR = false;
+        int jumps = 0, walks = 0;  // tangent steps and neighbour moves taken
         double wa = 0.0, wb = 0.0;
         __syncwarp();
 
@@ -254,6 +283,7 @@ __global__ void __launch_bounds__(32 * kRefWarps) k_refine_lanes(const Pipe P, i
             // ---- intervals that can hold a sample on or below it
             unsigned todo[2] = {0u, 0u};
             int spot[4] = {-1, -1, -1, -1};
+            bool moved = false;
             if (!done) {
                 const float base = iv_base(kapf, Cf, ls, m0);
                 float lev = __fmaf_rn(-ls, (float)(a - m0), la);  // the chord in v - s x
@@ -284,6 +314,23 @@ __global__ void __launch_bounds__(32 * kRefWarps) k_refine_lanes(const Pipe P, i
                             const int k0 = side ? m0 + 1 : 0, k1 = side ? L - 1 : m0 - 1;
                             spot[2 * side] = k > k0 ? k - 1 : -1;
                             spot[2 * side + 1] = k < k1 ? k + 1 : -1;
+                            if (jumps < kRefJumps && k > k0 && k < k1) {
+                                // to where the chord's slope is the tangent's, if
+                                // that is another sample of the run
+                                const float st = tangent_step(l, (float)(k - m0) * G.h, G.h, ls);
+                                const int kt = max(max(k0, x0 + m0), min(min(k1, x1 + m0),
+                                                   k + (int)rintf(fmaxf(fminf(st, 4096.0f), -4096.0f))));
+                                if (kt != k) {
+                                    moved = true;
+                                    if (side) {
+                                        b = kt;
+                                        newB = true;
+                                    } else {
+                                        a = kt;
+                                        newA = true;
+                                    }
+                                }
+                            }
                         } else if (!(sh < 0 && edge)) {
                             full = true;
                         }
@@ -293,6 +340,12 @@ __global__ void __launch_bounds__(32 * kRefWarps) k_refine_lanes(const Pipe P, i
                     if (side) fullR = full;
                     else fullL = full;
                 }
+            }
+            if (moved) {  // nothing to check against this chord
+                ++jumps;
+                fullL = fullR = false;
+                todo[0] = todo[1] = 0u;
+                for (int i = 0; i < 4; ++i) spot[i] = -1;
             }
             // ---- the neighbours of the pair's ends
             int nq = 0;
@@ -346,22 +399,27 @@ __global__ void __launch_bounds__(32 * kRefWarps) k_refine_lanes(const Pipe P, i
             ref_spots(rl, q, nq, true, lane, n_spot);
             __syncwarp();
             // ---- certified, or on to the next chord
-            if (!done) {
+            if (!done && !moved) {
                 const bool lowL = my.key[0] < kKeyInf, lowR = my.key[1] < kKeyInf;
                 if (!lowL && !lowR) done = true;
+                // a side searched in full moves to its lowest sample; where only
+                // neighbours were taken, to the lower neighbour a few times, then
+                // the side is searched in full
+                const bool step = walks < kRefWalks;
+                if (lowL || lowR) ++walks;
                 if (lowL) {
-                    if (fullL) {
+                    if (fullL || step) {
                         a = my.k[0];
                         newA = true;
                     }
-                    fullL = !fullL;
+                    fullL = !(fullL || step);
                 }
                 if (lowR) {
-                    if (fullR) {
+                    if (fullR || step) {
                         b = my.k[1];
                         newB = true;
                     }
-                    fullR = !fullR;
+                    fullR = !(fullR || step);
                 }
                 // the chord changed: start from the neighbours again
                 if (newA || newB) {
