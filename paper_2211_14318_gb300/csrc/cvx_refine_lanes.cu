@@ -169,7 +169,10 @@ __device__ __forceinline__ float tangent_step(const IvLine &l, float t, float h,
 
 // One warp takes 32 candidates at a time: phase 0 each node's first candidate,
 // phase 1 the others whose lower bound does not exceed the node's first value
-// (see k_refine).  With fewer candidates than lanes the warps take fewer each.
+// (see k_refine).  With fewer candidates than lanes the warps take fewer each,
+// but eight at least: a chord's two FP64 samples cost a warp the same for 1 and
+// 32 lanes (an FE step of 20,011 points: 10.80 ms with one, 10.60 with 8,
+// 10.58 with 16, 10.64 with 32).
 // Measured per call, all launches together, against one warp per candidate
 // with 32 or 64 FP64 samples in two windows and the certificate over every
 // FP32 sample: 1,706,177 candidates at L = 201: 22.3 -> 1.25 ms (one spot
@@ -188,7 +191,7 @@ __global__ void __launch_bounds__(32 * kRefWarps) k_refine_lanes(const Pipe P, i
     const unsigned below = (1u << lane) - 1u;
     const int nwarps = gridDim.x * kRefWarps, gw = blockIdx.x * kRefWarps + warp;
     const int nwork = P.cnt[(P.K + 1) + level];
-    const int bs = min(32, max(1, (nwork + nwarps - 1) / nwarps));
+    const int bs = min(32, max(8, (nwork + nwarps - 1) / nwarps));
     const int32_t *qp = P.qp[level], *qh = P.qh[level];
     unsigned n_ref = 0, n_full = 0, n_spot = 0;
     long long blk = gw;
