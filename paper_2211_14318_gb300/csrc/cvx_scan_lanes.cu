@@ -61,6 +61,8 @@ struct LaneState {
 // Node constants of a warp's item.
 struct LaneNode : ScanConsts {
     NodeLine nl;
+    IvGeom G;
+    float kap;
 };
 
 struct SideMin {
@@ -115,6 +117,42 @@ __device__ __forceinline__ SideMin line_pass(const NHPair &c, f32x2 H, float ns,
     return r;
 }
 
+__device__ __forceinline__ float key2f(int k) { return __int_as_float(f2key(__int_as_float(k))); }
+
+// Line constants of one direction (A1, A2, cJ) in register pairs.
+__device__ __forceinline__ NHPair line_pair(const NodeLine &nl, const float4 &d) {
+    NHPair c = nh_pair_node(nl);
+    c.J0 = pk2(nl.J0, nl.J0);
+    c.A1 = pk2(d.x, d.x);
+    c.A2 = pk2(d.y, d.y);
+    c.CJ = pk2(d.z, d.z);
+    return c;
+}
+
+// A warp's queue of intervals to be sampled (owner lane << 6 | side << 5 |
+// interval), the lanes' lines (A1, A2, cJ, ns) and each side's minimum so far.
+template <bool kShare>
+struct LaneTasks {
+    float4 line[32];
+    unsigned long long key[2][kShare ? 32 : 1];  // side_key
+    unsigned short q[kShare ? 64 : 1];
+};
+
+// Lanes that must have an interval left for each to sample its own (16 to 32:
+// within 2 % of each other).
+constexpr int kOwnMin = 24;
+// Lines of up to this many samples (the longest of a launch) are sampled by
+// their own lanes only: a short line's intervals (6 pairs of samples at most)
+// cost less than their queue.  1,048,576 points, L = 201: 57.3 ms without the
+// queue, 61.0 with it; an FE step at L = 333: 10.7 and 9.9 ms.
+constexpr int kOwnMaxL = 256;
+constexpr unsigned long long kSideNone = ~0ull;
+
+// Smaller value first, then the lower pair; -0 and +0 are equal.
+__device__ __forceinline__ unsigned long long side_key(float e, int k) {
+    return (unsigned long long)((unsigned)f2key(e + 0.0f) ^ 0x80000000u) << 32 | (unsigned)k;
+}
+
 // ---- the lane's own pass over a line: the same minima (bit for bit, lowest
 // pair on equal values) without sampling the whole line.  The ends of the
 // intervals (cvx_intervals.cuh) are sampled first; an interval whose bound
@@ -135,74 +173,187 @@ __device__ __forceinline__ SideMin line_pass(const NHPair &c, f32x2 H, float ns,
 // line's minimisers).  Not inlined: three call sites share one copy, which
 // keeps the kernel in the instruction cache (inlined copies left the warps
 // waiting for instructions 6.4 cycles per issue).
-__device__ __noinline__ SideMin lane_pass(const LaneNode &N, const IvGeom &G, float A1, float A2,
-                                          float cJ, float ns, float base, int kl, int xlL, int kr,
-                                          int xsL, int xsR) {
-    const int m0 = G.m0, PP = G.PP, np = m0 >> 1;
-    const f32x2 H = pk2(G.h, G.h), NS = pk2(ns, ns);
-    const IvLine l = iv_line(N.nl, A1, A2, cJ);
-    float gs0, gs1, eu0, eu1;
-    iv_eval(l.c, H, NS, pk2((float)xsL, (float)xsR), gs0, gs1, eu0, eu1);
+//
+// The lane's line is in T.line.  kShare: called by the whole warp (act: the
+// lane has a line), and the intervals are spread over its lanes.  Lines differ
+// in how many they have to sample (3.2 on average and 5.6 in the line of a
+// warp that has most, at L = 2049), so that a third of the lanes idled: once
+// fewer than kOwnMin lanes have an interval left, the rest go through a queue
+// in shared memory to whichever lane is free.  load path 66.6 -> 56.1 ms, mesh
+// 66.1 -> 59.5 ms (the inputs above), a load step's windows 35 -> 31.5 ms.
+template <bool kShare>
+__device__ __noinline__ SideMin lane_pass(const LaneNode &N, LaneTasks<kShare> &T, bool act, int kl,
+                                          int xlL, int kr, int xsL, int xsR) {
+    const int m0 = N.G.m0, PP = N.G.PP, np = m0 >> 1, lane = threadIdx.x & 31;
+    const f32x2 H = pk2(N.G.h, N.G.h);
     unsigned mL = 0, mR = 0;
     float lastL = INFINITY, lastR = INFINITY;
-#pragma unroll 1
-    for (int side = 0; side < 2; ++side) {
-        const int xb = side ? 2 * kr + 1 : -m0;
-        const int xl = side ? m0 : xlL;
-        const int npr = side ? np - kr : kl;
-        if (xl < xb) continue;
-        float ga, g1, Ea, E1;
-        iv_eval(l.c, H, NS, pk2((float)xb, (float)xl), ga, g1, Ea, E1);
-        float e = fmin3(side ? gs1 : gs0, ga, g1);
-        if (side) lastR = g1;
-        else lastL = g1;
-        const unsigned mask =
-            iv_sweep<true>(l, G, H, NS, base, xb, (float)xl, iv_count(G, npr), ga, Ea, e);
-        if (side) mR = mask;
-        else mL = mask;
-    }
     SideMin r;
     r.eL = r.eR = INFINITY;
     r.kL = r.kR = -1;
-    const f32x2 TWO = pk2(2.0f, 2.0f);
+    if (act) {
+        const float4 d = T.line[lane];
+        const f32x2 NS = pk2(d.w, d.w);
+        const IvGeom G = N.G;
+        const float base = iv_base(N.kap, N.C, d.w, m0);
+        const IvLine l = iv_line(N.nl, d.x, d.y, d.z);
+        float gs0, gs1, eu0, eu1;
+        iv_eval(l.c, H, NS, pk2((float)xsL, (float)xsR), gs0, gs1, eu0, eu1);
 #pragma unroll 1
-    while (mL | mR) {
-        const bool left = mL != 0;
-        const unsigned m = left ? mL : mR;
-        const int ka = (__ffs(m) - 1) * PP;
-        const int kb = min(left ? kl : np - kr, ka + PP);
-        float e = left ? r.eL : r.eR;
-        int kk = -1;
-        const float x = (float)((left ? -m0 : 2 * kr + 1) + 2 * ka);
-        f32x2 X = pk2(x, x + 1.0f);
-#pragma unroll 2
-        for (int k = ka; k < kb; ++k) {
-            float b0, b1;
-            upk2(fma2(NS, X, sample_nh2(l.c, mul2(X, H))), b0, b1);
-            const float en = fmin3(e, b0, b1);
-            if (en < e) kk = k;
-            e = en;
-            X = add2(X, TWO);
+        for (int side = 0; side < 2; ++side) {
+            const int xb = side ? 2 * kr + 1 : -m0;
+            const int xl = side ? m0 : xlL;
+            const int npr = side ? np - kr : kl;
+            if (xl < xb) continue;
+            float ga, g1, Ea, E1;
+            iv_eval(l.c, H, NS, pk2((float)xb, (float)xl), ga, g1, Ea, E1);
+            float e = fmin3(side ? gs1 : gs0, ga, g1);
+            if (side) lastR = g1;
+            else lastL = g1;
+            const unsigned mask =
+                iv_sweep<true>(l, G, H, NS, base, xb, (float)xl, iv_count(G, npr), ga, Ea, e);
+            if (side) mR = mask;
+            else mL = mask;
         }
-        if (left) {
-            mL = m & (m - 1);
-            r.eL = e;
-            r.kL = kk >= 0 ? kk : r.kL;
+        if (kShare) {
+            T.key[0][lane] = T.key[1][lane] = kSideNone;
         } else {
-            mR = m & (m - 1);
-            r.eR = e;
-            r.kR = kk >= 0 ? kk + kr : r.kR;
+            const f32x2 TWO = pk2(2.0f, 2.0f);
+#pragma unroll 1
+            while (mL | mR) {
+                const bool left = mL != 0;
+                const unsigned m = left ? mL : mR;
+                const int ka = (__ffs(m) - 1) * PP;
+                const int kb = min(left ? kl : np - kr, ka + PP);
+                float e = left ? r.eL : r.eR;
+                int kk = -1;
+                const float x = (float)((left ? -m0 : 2 * kr + 1) + 2 * ka);
+                f32x2 X = pk2(x, x + 1.0f);
+#pragma unroll 2
+                for (int k = ka; k < kb; ++k) {
+                    float b0, b1;
+                    upk2(fma2(NS, X, sample_nh2(l.c, mul2(X, H))), b0, b1);
+                    const float en = fmin3(e, b0, b1);
+                    if (en < e) kk = k;
+                    e = en;
+                    X = add2(X, TWO);
+                }
+                if (left) {
+                    mL = m & (m - 1);
+                    r.eL = e;
+                    r.kL = kk >= 0 ? kk : r.kL;
+                } else {
+                    mR = m & (m - 1);
+                    r.eR = e;
+                    r.kR = kk >= 0 ? kk : r.kR;
+                }
+            }
         }
     }
-    // the last sample of a side with an odd number of them is a pair of its own
-    // (elsewhere it lies in the last pair)
-    if (lastL < r.eL) {
-        r.eL = lastL;
-        r.kL = np;
+    if (kShare) {
+        NHPair c = line_pair(N.nl, T.line[lane]);
+        const f32x2 TWO = pk2(2.0f, 2.0f);
+        // samples the interval ent (LaneTasks::q) of its line
+        auto sample = [&](int ent, float ns, float e, int &kk) {
+            const f32x2 NS = pk2(ns, ns);
+            const bool right = (ent & 32) != 0;
+            const int ka = (ent & 31) * PP;
+            const int kb = min(right ? np - kr : kl, ka + PP);
+            const float x = (float)((right ? 2 * kr + 1 : -m0) + 2 * ka);
+            f32x2 X = pk2(x, x + 1.0f);
+#pragma unroll 2
+            for (int k = ka; k < kb; ++k) {
+                float b0, b1;
+                upk2(fma2(NS, X, sample_nh2(c, mul2(X, H))), b0, b1);
+                const float en = fmin3(e, b0, b1);
+                if (en < e) kk = k;
+                e = en;
+                X = add2(X, TWO);
+            }
+            return e;
+        };
+        // takes the lane's next interval off its masks (-1: none left)
+        auto next = [&]() {
+            const bool left = mL != 0;
+            const unsigned m = left ? mL : mR;
+            if (left) mL = m & (m - 1);
+            else mR = m & (m - 1);
+            return m ? lane << 6 | (left ? 0 : 32) | (__ffs(m) - 1) : -1;
+        };
+        auto own = [&](int ent, float ns) {
+            int kk = -1;
+            const float e = sample(ent, ns, ent & 32 ? r.eR : r.eL, kk);
+            if (ent & 32) {
+                r.eR = e;
+                r.kR = kk >= 0 ? kk : r.kR;
+            } else {
+                r.eL = e;
+                r.kL = kk >= 0 ? kk : r.kL;
+            }
+        };
+        const unsigned below = (1u << lane) - 1u;
+        const float ns = T.line[lane].w;
+        // most lanes have an interval left: each takes its own
+        unsigned bal;
+#pragma unroll 1
+        for (;;) {
+            bal = __ballot_sync(kFull, (mL | mR) != 0);
+            if (__popc(bal) < kOwnMin) break;
+            const int ent = next();
+            if (ent >= 0) own(ent, ns);
+            __syncwarp();
+        }
+        // the rest by whichever lane is free, one of each lane in turn until
+        // 32 are queued
+        int nq = 0;
+#pragma unroll 1
+        for (;;) {
+            while (bal && nq < 32) {
+                const int ent = next();
+                if (ent >= 0) T.q[nq + __popc(bal & below)] = (unsigned short)ent;
+                nq += __popc(bal);
+                bal = __ballot_sync(kFull, (mL | mR) != 0);
+            }
+            if (nq == 0) break;
+            __syncwarp();
+            const int n = min(nq, 32);
+            nq -= n;
+            if (lane < n) {
+                const int ent = T.q[nq + lane];
+                const float4 d = T.line[ent >> 6];
+                c.A1 = pk2(d.x, d.x);
+                c.A2 = pk2(d.y, d.y);
+                c.CJ = pk2(d.z, d.z);
+                int kk = -1;
+                const float e = sample(ent, d.w, INFINITY, kk);
+                if (kk >= 0) atomicMin(&T.key[(ent >> 5) & 1][ent >> 6], side_key(e, kk));
+            }
+            __syncwarp();
+        }
     }
-    if (lastR < r.eR) {
-        r.eR = lastR;
-        r.kR = np;
+    if (act) {
+        if (kShare) {  // the queue's minima; on equal values the lower pair
+            const unsigned long long kL = T.key[0][lane], kR = T.key[1][lane];
+            if (kL < side_key(r.eL, r.kL)) {
+                r.eL = key2f((int)((unsigned)(kL >> 32) ^ 0x80000000u));
+                r.kL = (int)(kL & 0xffffffffu);
+            }
+            if (kR < side_key(r.eR, r.kR)) {
+                r.eR = key2f((int)((unsigned)(kR >> 32) ^ 0x80000000u));
+                r.kR = (int)(kR & 0xffffffffu);
+            }
+        }
+        if (r.kR >= 0) r.kR += kr;
+        // the last sample of a side with an odd number of them is a pair of its
+        // own (elsewhere it lies in the last pair)
+        if (lastL < r.eL) {
+            r.eL = lastL;
+            r.kL = np;
+        }
+        if (lastR < r.eR) {
+            r.eR = lastR;
+            r.kR = np;
+        }
     }
     return r;
 }
@@ -390,17 +541,6 @@ __device__ __forceinline__ int enc_ab(int a, int b) {
     return a < 0 ? (kConv | kNoPair) : (a | (b << 12));
 }
 
-__device__ __forceinline__ float key2f(int k) { return __int_as_float(f2key(__int_as_float(k))); }
-
-// Line constants of one direction in register pairs.
-__device__ __forceinline__ NHPair line_pair(const NHPair &node, const DirLine &dl) {
-    NHPair c = node;
-    c.A1 = pk2(dl.A1, dl.A1);
-    c.A2 = pk2(dl.A2, dl.A2);
-    c.CJ = pk2(dl.cJ, dl.cJ);
-    return c;
-}
-
 // Global direction index of entry j of a node's proposal window (row-major
 // over (da, db) in [-w, w]^2 around the centre cell, indices wrapping).
 __device__ __forceinline__ int lane_window_dir(const ProbDesc &pd, int2 c, int j) {
@@ -418,11 +558,13 @@ __device__ __forceinline__ int lane_window_dir(const ProbDesc &pd, int2 c, int j
 #define CVX_LANE_MIN_BLOCKS 4  // CTAs of 256 threads per SM the registers target
 #endif
 
+template <bool kShare>
 __global__ void __launch_bounds__(32 * kLaneWarps, CVX_LANE_MIN_BLOCKS)
     k_scan_lanes(const Pipe P, int level) {
     __shared__ LaneState s_st[kLaneWarps][kLaneItemMax];
     __shared__ unsigned short s_live[kLaneWarps][kLaneItemMax];
     __shared__ LaneNode s_nd[kLaneWarps];
+    __shared__ LaneTasks<kShare> s_tk[kLaneWarps];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const bool win = P.pass == PASS_WINDOW;
     const int n_nodes = P.cnt[level];
@@ -431,6 +573,7 @@ __global__ void __launch_bounds__(32 * kLaneWarps, CVX_LANE_MIN_BLOCKS)
     LaneState *st = s_st[warp];
     unsigned short *live = s_live[warp];
     LaneNode &N = s_nd[warp];
+    LaneTasks<kShare> &T = s_tk[warp];
     unsigned long long n_valid = 0;
     unsigned n_lines = 0, n_drop = 0, n_flat = 0, n_extra = 0, n_cert = 0;
 
@@ -466,9 +609,11 @@ __global__ void __launch_bounds__(32 * kLaneWarps, CVX_LANE_MIN_BLOCKS)
             return win ? lane_window_dir(pd, cen, d0 + blk + j) : d0 + blk + j;
         };
         const f32x2 H = pk2(ln.h32, ln.h32);
-        const IvGeom G = iv_geom(ln.h32, m0);
-        NHPair node = nh_pair_node(N.nl);
-        node.J0 = pk2(N.nl.J0, N.nl.J0);
+        if (lane == 0) {
+            N.G = iv_geom(ln.h32, m0);
+            N.kap = kap;
+        }
+        __syncwarp();
         // the item's best directions so far: lane i < kItemTop holds entry i
         float tq = INFINITY;
         int td = INT_MAX, tab = -1;
@@ -492,28 +637,34 @@ __global__ void __launch_bounds__(32 * kLaneWarps, CVX_LANE_MIN_BLOCKS)
             const int kf = max(0, np - Xn / 2), kn = min(np, Xn / 2);
             for (int q = 0; q < Pn; ++q) {
                 const int j = lane * Pn + q;
-                if (j >= nb) break;
-                const int gd = gdir(blk, j);
-                const DirLine dl = make_dir_line<CVX_ENERGY_NH_DAMAGE>(N.nl, P.dir32[doff + gd]);
-                const NHPair c = line_pair(node, dl);
-                const bool tangent = !warm;
-                const float s0 = warm ? s_prev : sa * __fmaf_rn(cb, dl.cJ, dl.A1);
-                const SideMin sm = lane_pass(N, G, dl.A1, dl.A2, dl.cJ, -s0, iv_base(kap, C, s0, m0),
-                                           np, -1, 0, xsL, xsR);
-                const Bounds b = pass_bounds(c, H, s0, m0, sm);
+                const bool act = j < nb;
+                const int gd = gdir(blk, act ? j : 0);
+                {
+                    const DirLine dl = make_dir_line<CVX_ENERGY_NH_DAMAGE>(N.nl, P.dir32[doff + gd]);
+                    const float s0 = warm ? s_prev : sa * __fmaf_rn(cb, dl.cJ, dl.A1);
+                    T.line[lane] = make_float4(dl.A1, dl.A2, dl.cJ, -s0);
+                }
+                if (!kShare && !act) break;
+                const SideMin sm = lane_pass<kShare>(N, T, act, np, -1, 0, xsL, xsR);
+                if (!act) continue;
+                const float4 d = T.line[lane];
+                const Bounds b = pass_bounds(line_pair(N.nl, d), H, -d.w, m0, sm);
                 LaneState t;
                 t.q_lo = b.q_lo;
                 t.q_hi = b.q_hi;
                 t.s = b.s;
                 t.ab = enc_ab(b.a, b.b);
                 if (b.q_hi - b.q_lo <= 0.25f * eps32_at(b.q_lo, kap, C)) t.ab |= kConv;
-                if (tangent) t.ab |= kTan;
+                if (!warm) t.ab |= kTan;
                 st[j] = t;
                 umin = fminf(umin, b.q_hi);
                 warm = b.a >= 0 && b.q_hi < w0 - epsc;
                 xsL = b.a >= 0 ? b.a - m0 : -1;
                 xsR = b.a >= 0 ? b.b - m0 : 1;
                 s_prev = b.s;
+                DirLine dl;
+                dl.cJ = d.z;
+                dl.J0 = N.nl.J0;
                 n_valid += valid_samples(dl, ln, CVX_ENERGY_NH_DAMAGE);
             }
             n_lines += nb;
@@ -549,17 +700,22 @@ __global__ void __launch_bounds__(32 * kLaneWarps, CVX_LANE_MIN_BLOCKS)
                 float um = INFINITY;
                 if (n_live >= kLaneCoop) {
                     // lane by lane
-                    for (int i = lane; i < n_live; i += 32) {
-                        const int j = live[i];
-                        const DirLine dl =
-                            make_dir_line<CVX_ENERGY_NH_DAMAGE>(N.nl, P.dir32[doff + gdir(blk, j)]);
-                        const NHPair c = line_pair(node, dl);
+                    for (int i = lane; i - lane < n_live; i += 32) {
+                        const bool act = i < n_live;
+                        const int j = live[act ? i : 0];
+                        {
+                            const DirLine dl = make_dir_line<CVX_ENERGY_NH_DAMAGE>(
+                                N.nl, P.dir32[doff + gdir(blk, j)]);
+                            T.line[lane] = make_float4(dl.A1, dl.A2, dl.cJ, -st[j].s);
+                        }
+                        const int ab0 = st[j].ab;
+                        if (!kShare && !act) break;
+                        const SideMin sm = lane_pass<kShare>(N, T, act, np, -1, 0, (ab0 & 0xfff) - m0,
+                                                     ((ab0 >> 12) & 0xfff) - m0);
+                        if (!act) continue;
+                        const float4 d = T.line[lane];
                         LaneState t = st[j];
-                        const int a0 = t.ab & 0xfff, b0 = (t.ab >> 12) & 0xfff;
-                        const SideMin sm = lane_pass(N, G, dl.A1, dl.A2, dl.cJ, -t.s,
-                                                   iv_base(kap, C, t.s, m0), np, -1, 0, a0 - m0,
-                                                   b0 - m0);
-                        const Bounds b = pass_bounds(c, H, t.s, m0, sm);
+                        const Bounds b = pass_bounds(line_pair(N.nl, d), H, t.s, m0, sm);
                         const int ab = enc_ab(b.a, b.b);
                         const bool same = ab == (t.ab & ~kTan);
                         t.q_lo = fmaxf(t.q_lo, b.q_lo);
@@ -576,7 +732,8 @@ __global__ void __launch_bounds__(32 * kLaneWarps, CVX_LANE_MIN_BLOCKS)
                         const int j = live[i];
                         const DirLine dl =
                             make_dir_line<CVX_ENERGY_NH_DAMAGE>(N.nl, P.dir32[doff + gdir(blk, j)]);
-                        const NHPair c = line_pair(node, dl);
+                        const NHPair c =
+                            line_pair(N.nl, make_float4(dl.A1, dl.A2, dl.cJ, 0.0f));
                         LaneState t = st[j];
                         SideMin sm = line_pass(c, H, -t.s, m0, lane, 32);
                         warp_side(sm.eL, sm.kL);
@@ -629,16 +786,19 @@ __global__ void __launch_bounds__(32 * kLaneWarps, CVX_LANE_MIN_BLOCKS)
                     n_try += __popc(bal);
                 }
                 __syncwarp();
-                for (int i = lane; i < n_try; i += 32) {
-                    const int j = live[i];
+                for (int i = lane; i - lane < n_try; i += 32) {
+                    const bool act = i < n_try;
+                    const int j = live[act ? i : 0];
                     const float4 d32 = P.dir32[doff + gdir(blk, j)];
                     const DirLine dl = make_dir_line<CVX_ENERGY_NH_DAMAGE>(N.nl, d32);
                     const float s0 = sa * __fmaf_rn(cb, dl.cJ, dl.A1);
+                    T.line[lane] = make_float4(dl.A1, dl.A2, dl.cJ, -s0);
                     // the smallest v - s0 x over the far samples (left pairs k < kf,
                     // right pairs k >= kn, and the last sample if m0 is odd)
                     const int xlL = 2 * kf - 1 - m0;
-                    const SideMin sf = lane_pass(N, G, dl.A1, dl.A2, dl.cJ, -s0, iv_base(kap, C, s0, m0),
-                                               kf, xlL, kn, xlL, min(2 * kn + 1, m0));
+                    if (!kShare && !act) break;
+                    const SideMin sf = lane_pass<kShare>(N, T, act, kf, xlL, kn, xlL, min(2 * kn + 1, m0));
+                    if (!act) continue;
                     const float ef = fminf(sf.eL, sf.eR);
                     if (flat_certificate(N, dl, d32, ln.h32, m0, 2 * kf - m0, 2 * kn, s0, ef, kap))
                         st[j].ab |= kCert;
@@ -748,11 +908,13 @@ __global__ void __launch_bounds__(32 * kLaneWarps, CVX_LANE_MIN_BLOCKS)
 }
 
 int lane_scan_blocks_per_sm() {
-    int nb = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_scan_lanes, 32 * kLaneWarps, 0) !=
-        cudaSuccess)
+    int a = 0, b = 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&a, k_scan_lanes<false>, 32 * kLaneWarps, 0) !=
+            cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_scan_lanes<true>, 32 * kLaneWarps, 0) !=
+            cudaSuccess)
         return 0;
-    return nb;
+    return a < b ? a : b;
 }
 
 bool lane_scan_enabled(int energy) {
@@ -768,7 +930,10 @@ cudaError_t launch_scan_lanes(const Pipe &p, int level, int sms, cudaStream_t s)
     static int bpsm = 0;
     if (!bpsm) bpsm = lane_scan_blocks_per_sm();
     if (bpsm < 1) return cudaErrorInvalidConfiguration;
-    k_scan_lanes<<<sms * bpsm, 32 * kLaneWarps, 0, s>>>(p, level);
+    if (p.stride32 > kOwnMaxL)
+        k_scan_lanes<true><<<sms * bpsm, 32 * kLaneWarps, 0, s>>>(p, level);
+    else
+        k_scan_lanes<false><<<sms * bpsm, 32 * kLaneWarps, 0, s>>>(p, level);
     return cudaGetLastError();
 }
 
