@@ -42,7 +42,12 @@ sys.path.insert(0, ROOT)
 METRIC = "quadrature points convexified/s (W^R+P) at 1e-6 rel. error, surrogate vs full-scan"
 MAT = dict(mu=1.0, lambda_L=5.0, D_inf=0.99, D0=0.5)
 NX, STRETCH, ANGLES, LINE, DEPTH, T_HALF = 128, 1.3, 64, 1025, 3, 0.5
-FLOP_PER_SAMPLE = 30  # algorithmic FP32 work per valid line sample (energy 22 + hull 8)
+# algorithmic FP32 work per valid line sample (energy 22 + hull 8).  The line scan
+# does not take every sample: a part of a line whose bound lies above the minimum
+# looked for is left out, so that "achieved" is the rate of a scan that takes them
+# all (it can exceed the peak); the same holds for the grid's line kernel, which
+# takes no FP64 step where an FP32 bound decides
+FLOP_PER_SAMPLE = 30
 FP32_LANES_PER_SM = 128
 
 
@@ -225,8 +230,8 @@ def fp32_peak_tflops(torch, dev):
 
 # the translation unit of k_scan_lanes (the kernel and its launch) and the
 # headers it includes
-SCAN_SOURCES = ("cvx_scan_lanes.cu", "cvx_line.cuh", "cvx_bridge.cuh", "cvx_device.cuh",
-                "cvx_internal.h")
+SCAN_SOURCES = ("cvx_scan_lanes.cu", "cvx_intervals.cuh", "cvx_line.cuh", "cvx_bridge.cuh",
+                "cvx_device.cuh", "cvx_internal.h")
 
 
 GRID_SOURCES = ("cvx_grid.cu", "cvx_device.cuh", "cvx_internal.h", "cvx_handle.h")
@@ -447,13 +452,13 @@ def run_ours(a):
                          "frac": (achieved / peak) if achieved else None,
                          "traffic": traffic,
                          "peak_source": f"{sms} SMs x {FP32_LANES_PER_SM} FP32 lanes x 2 x {mhz:.0f} MHz ({peak_src})",
-                         "flop_per_valid_sample": FLOP_PER_SAMPLE,
+                         "flop_per_valid_sample": FLOP_PER_SAMPLE, "flop_counted": "every valid sample",
                          "kernel_share_of_step": scan_ms / dev_ms if dev_ms else None,
                          "launches": scan_launches},
             "cpu_baseline": cpu,
             "e2e": {"value": e2e_value, "unit": "points/s",
                     "h2d_bytes_per_step": 2 * n * 4 * 8, "d2h_bytes_per_step": n * 8 + n * 4 * 8},
-            "gpu_launches": a.steps * (3 + 4 * DEPTH),  # history, init, 4 per level, leaf
+            "gpu_launches": a.steps * (3 + 6 * DEPTH),  # history, init, 6 per level, leaf
             "clocks": ck,
             "stats": st,
         }
@@ -532,13 +537,14 @@ def train_proposal(cv, api, inputs, path, dev):
 
 def propose_launches(n, K, R, mirror=False):
     """Kernels of this library one surrogate_propose call and its history
-    update launch: k_init; per level and 65,536-node chunk the features, five
-    tensor-core GEMMs and the decoding; per level R + 1 window passes, R + 1
-    mirror-window passes (with the mirror window) and the fallback pass (line
-    scan, select, refine, commit each); k_leaf, k_fell_back; k_history."""
+    update launch: k_init; per level and 65,536-node chunk the features, the
+    network and the decoding; per level R + 1 window passes, R + 1
+    mirror-window passes (with the mirror window) and the fallback pass (node
+    constants, line scan, select, two of refine, commit each); k_leaf,
+    k_fell_back; k_history."""
     chunks = sum(-(-(n << l) // 65536) for l in range(K))
     passes = (R + 1) * (2 if mirror else 1) + 1
-    return 1 + 7 * chunks + 4 * passes * K + 3
+    return 1 + 3 * chunks + 6 * passes * K + 3
 
 
 def timed_full_scan(cv, p, F, beta, steps, torch):
@@ -575,7 +581,7 @@ def roofline_obj(st, scan_ms, launches, step_ms, peak, sms, mhz, peak_src, traff
             "unit": "TFLOP/s", "frac": (achieved / peak) if achieved else None,
             "traffic": traffic,
             "peak_source": f"{sms} SMs x {FP32_LANES_PER_SM} FP32 lanes x 2 x {mhz:.0f} MHz ({peak_src})",
-            "flop_per_valid_sample": FLOP_PER_SAMPLE,
+            "flop_per_valid_sample": FLOP_PER_SAMPLE, "flop_counted": "every valid sample",
             "kernel_share_of_step": scan_ms / step_ms if step_ms else None,
             "launches": launches}
 
@@ -950,7 +956,7 @@ def global_grid_line(a, cv, api, inputs, torch, dev, sms, mhz, peak_src, runs=10
                         "flop_per_point_direction": GRID_FLOP_PER_POINT_DIR,
                         "kernel_ms_per_launch": lines_ms / max(1, launches),
                         "kernel_share": lines_ms / t, "launches": launches},
-           "gpu_launches_per_run": 1 + 1 + c["kmax"] * 3 + 1}
+           "gpu_launches_per_run": 1 + 2 + c["kmax"] * 3 + 1}
     # Algorithms 2 and 3 at 1,048,576 points of the grid's box
     lo = np.array(g.lo)
     hi = lo + (np.array(g.n) - 1) * np.array(g.delta)
@@ -1377,7 +1383,7 @@ def run_train(a):
                                "material points (16x16 angles, L=201, depth 2, lambda in [1,2])",
                    "form": "train", "train_samples": int(n_train), "batch": 8192,
                    "epochs": a.train_epochs, "held_out": int(Xh.shape[0])},
-        "roofline": {"bound": "tensor", "kernel": "k_gemm (forward, inference)",
+        "roofline": {"bound": "tensor", "kernel": "k_mlp_forward (inference)",
                      "achieved": ach_inf, "peak": peak, "unit": "TFLOP/s",
                      "frac": ach_inf / peak if peak else None,
                      "training_tflops": train_flop * train_rate / 1e12,

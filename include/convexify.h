@@ -398,7 +398,7 @@ int cvx_grid_energy(cvx_handle *h, const cvx_params *p, const cvx_grid *g, doubl
 /* One iteration of Eq. (4.3): W_out from W_in (DEVICE, N each, no aliasing);
  * lam (DEVICE, N x 3 int32, nullable) = the laminate records; dec (DEVICE
  * scalar, nullable) = the largest decrease W_in - W_out over the points where
- * both are finite.  Workspace: the handle's (12 bytes per point and
+ * both are finite.  Workspace: the handle's (8 bytes per point and
  * direction, in chunks of at most 1 GB, plus the line starts). */
 int cvx_grid_step(cvx_handle *h, const cvx_grid *g, int32_t nd, const int32_t *off,
                   const double *W_in, double *W_out, int32_t *lam, double *dec, cvx_stream s);
