@@ -6,8 +6,9 @@
 // A warp takes a work item (a node and up to 256 of its directions) and each
 // lane takes its own line, two samples per paired FP32 instruction, without
 // storing it, and without taking the samples that a bound of v'' shows to lie
-// above the minimum looked for (lane_pass).  For the hull at t = 0 of the left set {x < 0} and the right set
-// {x > 0} of the samples (x = m - m0) the pass at a slope s yields
+// above the minimum looked for (lane_pass).  For the hull at t = 0 of the left
+// set {x < 0} and the right set {x > 0} of the samples (x = m - m0) the pass at
+// a slope s yields
 //   e_L = min over the left of (v - s x),  e_R = min over the right,
 // and their minimisers a < 0 < b.  For any s, min(e_L, e_R) is a lower bound
 // of the hull value at 0 (an affine minorant read at 0), and the chord of
@@ -21,8 +22,8 @@
 // only lines that are still candidates take further passes: many of them
 // lane by lane, a few of them with the whole warp on one line.  No decision
 // is taken here: the item's best directions by lower bound go to k_select,
-// and the node is decided on FP64 samples by k_refine / k_commit, exactly as
-// after the warp-per-line scan.
+// and the node is decided on FP64 samples by k_refine_lanes / k_commit, with
+// the results of the warp-per-line scan's k_refine.
 #include <cuda_runtime.h>
 #include <limits.h>
 #include <stdlib.h>
@@ -159,12 +160,13 @@ __device__ __forceinline__ unsigned long long side_key(float e, int k) {
 // exceeds the smallest sample seen so far cannot hold the side's minimum and
 // is never sampled, the others (the interval of the minimum and its
 // neighbours as a rule) are sampled in full.
-// What bounds it: instruction issue (79 % of the slots at L = 201).  Taking
+// What bounds it: instruction issue (77 % of the slots at L = 201, 70 % at
+// L = 2049).  Taking
 // every sample instead: 3,001 load-path points, 128^2 directions, L = 2049,
 // depth 3: 326.9 ms of line scan, 70.9 ms with the intervals; 16,384 mesh
 // points, 64^2, L = 1025: 227.9 -> 70 ms; 1,048,576 points, 16^2, L = 201:
-// 86.9 -> 51 ms.  2.5 to 4.0 intervals are sampled per line, both sides
-// together.
+// 86.9 -> 42 ms.  2.6 to 6.9 intervals are sampled per line, both sides
+// together (two at least).
 //
 // The pass at slope s = -ns over the left samples -m0 .. xlL (the pairs
 // k < kl, and x = -1 if that is a pair of its own) and the right pairs
