@@ -165,7 +165,7 @@ __device__ __forceinline__ unsigned long long side_key(float e, int k) {
 // every sample instead: 3,001 load-path points, 128^2 directions, L = 2049,
 // depth 3: 326.9 ms of line scan, 70.9 ms with the intervals; 16,384 mesh
 // points, 64^2, L = 1025: 227.9 -> 70 ms; 1,048,576 points, 16^2, L = 201:
-// 86.9 -> 42 ms.  2.6 to 6.9 intervals are sampled per line, both sides
+// 86.9 -> 50 ms.  2.6 to 6.9 intervals are sampled per line, both sides
 // together (two at least).
 //
 // The pass at slope s = -ns over the left samples -m0 .. xlL (the pairs
