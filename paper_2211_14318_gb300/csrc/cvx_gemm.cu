@@ -111,8 +111,8 @@ __global__ void __launch_bounds__(256, 1)
         }
     }
     __syncwarp();
-    bool ok = mbar_wait(&bar_done, 0, kWaitNs);
-    if (!ok && ep.err) atomicExch(ep.err, 1);
+    const bool ok = mbar_wait_warp(&bar_done, 0, kWaitNs);
+    if (!ok && lane == 0 && ep.err) atomicExch(ep.err, 1);
     tc_fence_after();
 
     const int quarter = warp & 3;
@@ -242,8 +242,8 @@ __global__ void __launch_bounds__(kWsThreads, 1)
         int v = 0;
         for (int t = blockIdx.x; t < ntiles; t += gridDim.x, ++v) {
             const int acc = v & 1, vu = v >> 1;
-            if (!mbar_wait(&accf[acc], vu & 1, kWaitNs)) {
-                if (ep.err) atomicExch(ep.err, 1);
+            if (!mbar_wait_warp(&accf[acc], vu & 1, kWaitNs)) {
+                if (lane == 0 && ep.err) atomicExch(ep.err, 1);
                 break;
             }
             tc_fence_after();

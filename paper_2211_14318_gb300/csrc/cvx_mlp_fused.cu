@@ -193,7 +193,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             // ---- hidden layers: bias, GELU, the next operand
             for (int l = 0; l < 4 && ok; ++l)
                 for (int g = 0; g < ng; ++g) {
-                    if (!(ok = mbar_wait(&d_full[g], ph[g] & 1, kWaitNs))) break;
+                    if (!(ok = mbar_wait_warp(&d_full[g], ph[g] & 1, kWaitNs))) break;
                     ++ph[g];
                     tc_fence_after();
                     const float *bias = sBias + l * kWidth + 64 * part;
@@ -220,7 +220,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                 }
             // ---- outputs
             for (int g = 0; g < ng && ok; ++g) {
-                if (!(ok = mbar_wait(&d_full[g], ph[g] & 1, kWaitNs))) break;
+                if (!(ok = mbar_wait_warp(&d_full[g], ph[g] & 1, kWaitNs))) break;
                 ++ph[g];
                 tc_fence_after();
                 if (part == 0) {

@@ -215,7 +215,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_mlp_train(const MlpTrain f) {
             }
             for (int p = 0; p < 9 && ok; ++p)
                 for (int g = 0; g < ng; ++g) {
-                    if (!(ok = mbar_wait(&d_full[g], ph[g] & 1, kWaitNs))) break;
+                    if (!(ok = mbar_wait_warp(&d_full[g], ph[g] & 1, kWaitNs))) break;
                     ++ph[g];
                     tc_fence_after();
                     const long long m = (long long)(t0 + g * G) * kRows + row;
@@ -444,7 +444,7 @@ __global__ void __launch_bounds__(kDwThreads, 1) k_mlp_dw(const MlpTrain f, int 
         const int quarter = warp & 3, h = (warp - 4) >> 2;
         const int r = kRows * h + 32 * quarter + lane;
         const uint32_t trow = tmem + h * kWidth + ((uint32_t)(32 * quarter) << 16);
-        if (mbar_wait(&done, 0, kWaitNs)) {
+        if (mbar_wait_warp(&done, 0, kWaitNs)) {
             tc_fence_after();
             if (job < 3) {
                 float4 *g = reinterpret_cast<float4 *>(f.dW[job + 1] + (size_t)r * kWidth);

@@ -64,6 +64,13 @@ __device__ __forceinline__ bool mbar_wait(uint64_t *bar, unsigned parity, uint64
         if (global_ns() - t0 > limit_ns) return false;
     return true;
 }
+// The same for a whole warp, whose lanes then all take one branch: each lane
+// reads the clock for itself, so near the limit some lanes can see the phase
+// complete and others give up, and what follows (tcgen05.ld, shuffles) takes
+// whole warps.  True only if every lane saw the phase complete.
+__device__ __forceinline__ bool mbar_wait_warp(uint64_t *bar, unsigned parity, uint64_t limit_ns) {
+    return __all_sync(0xffffffffu, mbar_wait(bar, parity, limit_ns));
+}
 
 // ---------------------------------------------------------------- TMA
 __device__ __forceinline__ void tma_load_2d(void *dst, const CUtensorMap *map, uint64_t *bar,
