@@ -82,6 +82,7 @@ __global__ void __launch_bounds__(256, 1)
             }
         };
         bool ok = true;
+        int issued = 1;
         issue(0);
         for (int c = 0; c < nchunks && ok; ++c) {
             const int s = c % kStages;
@@ -90,6 +91,7 @@ __global__ void __launch_bounds__(256, 1)
                 if (c2 >= kStages) ok = mbar_wait(&bar_mma[s2], ((c2 - kStages) / kStages) & 1, kWaitNs);
                 if (!ok) break;
                 issue(c2);
+                ++issued;
             }
             ok = mbar_wait(&bar_full[s], (c / kStages) & 1, kWaitNs);
             if (!ok) break;
@@ -103,15 +105,15 @@ __global__ void __launch_bounds__(256, 1)
             }
             umma_commit(&bar_mma[s]);
         }
-        if (ok) {
-            umma_commit(&bar_done);
-        } else {
-            s_fail = 1;
+        if (!ok) {
+            *(volatile int *)&s_fail = 1;
             if (ep.err) atomicExch(ep.err, 1);
         }
+        drain_copies(bar_full, kStages, issued, kWaitNs);
+        drain_mmas(&bar_done, kWaitNs);
     }
     __syncwarp();
-    const bool ok = mbar_wait_warp(&bar_done, 0, kWaitNs);
+    const bool ok = mbar_wait_warp(&bar_done, 0, kWaitNs) && *(volatile int *)&s_fail == 0;
     if (!ok && lane == 0 && ep.err) atomicExch(ep.err, 1);
     tc_fence_after();
 
@@ -161,7 +163,7 @@ __global__ void __launch_bounds__(kWsThreads, 1)
         reinterpret_cast<unsigned char *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
     unsigned char *sB = smem;
     unsigned char *sA = smem + (size_t)BN * K * 2;
-    __shared__ __align__(8) uint64_t full[kWsStages], empty[kWsStages], bfull, accf[2], acce[2];
+    __shared__ __align__(8) uint64_t full[kWsStages], empty[kWsStages], bfull, accf[2], acce[2], drain;
     __shared__ uint32_t s_tmem;
 
     const int ntiles = (M + kBM - 1) / kBM;
@@ -174,6 +176,7 @@ __global__ void __launch_bounds__(kWsThreads, 1)
             mbar_init(&empty[i], 1);
         }
         mbar_init(&bfull, 1);
+        mbar_init(&drain, 1);
         for (int i = 0; i < 2; ++i) {
             mbar_init(&accf[i], 1);
             mbar_init(&acce[i], 8);
@@ -204,6 +207,8 @@ __global__ void __launch_bounds__(kWsThreads, 1)
                 }
             }
             if (!ok && ep.err) atomicExch(ep.err, 1);
+            mbar_wait(&bfull, 0, kWaitNs);
+            drain_copies(full, kWsStages, u, kWaitNs);
         }
     } else if (warp == 1) {
         if (lane == 0) {
@@ -233,6 +238,7 @@ __global__ void __launch_bounds__(kWsThreads, 1)
                 umma_commit(&accf[acc]);
             }
             if (!ok && ep.err) atomicExch(ep.err, 1);
+            drain_mmas(&drain, kWaitNs);
         }
     } else if (warp >= 4) {
         const int ew = warp - 4, quarter = ew & 3, half = ew >> 2;

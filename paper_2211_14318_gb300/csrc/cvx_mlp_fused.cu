@@ -50,7 +50,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     unsigned char *sW0 = sB + kRing * kStageBytes;
     unsigned char *sW4 = sW0 + kW0Bytes;
     float *sBias = reinterpret_cast<float *>(sW4 + kW4Bytes);
-    __shared__ __align__(8) uint64_t b_full[kRing], b_empty[kRing], w_full, a_ready[2], d_full[2];
+    __shared__ __align__(8) uint64_t b_full[kRing], b_empty[kRing], w_full, a_ready[2], d_full[2], drain;
     __shared__ uint32_t s_tmem;
 
     const int Mv = f.M_dev ? min(*f.M_dev - f.m_off, f.M) : f.M;
@@ -65,6 +65,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             mbar_init(&b_empty[i], 1);
         }
         mbar_init(&w_full, 1);
+        mbar_init(&drain, 1);
         for (int i = 0; i < 2; ++i) {
             mbar_init(&a_ready[i], 16);
             mbar_init(&d_full[i], 1);
@@ -100,13 +101,9 @@ __global__ void __launch_bounds__(kThreads, 1)
                                       f.W[l] + (size_t)c * kStageK * kWidth, kStageBytes, &b_full[st]);
                         }
                     }
-            if (!ok) {
-                atomicExch(f.err, 1);
-                // the loads in flight land before the CTA ends
-                mbar_wait(&w_full, 0, kWaitNs);
-                for (int i = max(0, u - kRing); i < u; ++i)
-                    mbar_wait(&b_full[i % kRing], (i / kRing) & 1, kWaitNs);
-            }
+            if (!ok) atomicExch(f.err, 1);
+            mbar_wait(&w_full, 0, kWaitNs);
+            drain_copies(b_full, kRing, u, kWaitNs);
         }
     } else if (warp == 1) {
         if (lane == 0) {
@@ -148,6 +145,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                         umma_commit(&d_full[g]);
                     }
             if (!ok) atomicExch(f.err, 1);
+            drain_mmas(&drain, kWaitNs);
         }
     } else if (warp >= 4) {
         // columns 64 part .. 64 part + 63 of the rows of TMEM lanes 32 quarter ..

@@ -63,7 +63,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_mlp_train(const MlpTrain f) {
     unsigned char *sW4 = sW0 + kW0Bytes;       // last layer, forward
     unsigned char *sWt4 = sW4 + kW4Bytes;      // last layer, transposed
     float *sBias = reinterpret_cast<float *>(sWt4 + kW4Bytes);
-    __shared__ __align__(8) uint64_t b_full[kRing], b_empty[kRing], w_full, a_ready[2], d_full[2];
+    __shared__ __align__(8) uint64_t b_full[kRing], b_empty[kRing], w_full, a_ready[2], d_full[2], drain;
     __shared__ uint32_t s_tmem;
     __shared__ float s_db[4][kWidth], s_db4[8];  // bias gradients; the loss in s_db4[7]
 
@@ -77,6 +77,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_mlp_train(const MlpTrain f) {
             mbar_init(&b_empty[i], 1);
         }
         mbar_init(&w_full, 1);
+        mbar_init(&drain, 1);
         for (int i = 0; i < 2; ++i) {
             mbar_init(&a_ready[i], 16);
             mbar_init(&d_full[i], 1);
@@ -119,13 +120,9 @@ __global__ void __launch_bounds__(kThreads, 1) k_mlp_train(const MlpTrain f) {
                         }
                     }
                 }
-            if (!ok) {
-                atomicExch(f.err, 1);
-                // the loads in flight land before the CTA ends
-                mbar_wait(&w_full, 0, kWaitNs);
-                for (int i = max(0, u - kRing); i < u; ++i)
-                    mbar_wait(&b_full[i % kRing], (i / kRing) & 1, kWaitNs);
-            }
+            if (!ok) atomicExch(f.err, 1);
+            mbar_wait(&w_full, 0, kWaitNs);
+            drain_copies(b_full, kRing, u, kWaitNs);
         }
     } else if (warp == 1) {
         if (lane == 0) {
@@ -167,6 +164,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_mlp_train(const MlpTrain f) {
                         umma_commit(&d_full[g]);
                     }
             if (!ok) atomicExch(f.err, 1);
+            drain_mmas(&drain, kWaitNs);
         }
     } else if (warp >= 4) {
         // columns 64 part .. 64 part + 63 of the rows of TMEM lanes 32 quarter ..
@@ -376,7 +374,7 @@ __global__ void __launch_bounds__(kDwThreads, 1) k_mlp_dw(const MlpTrain f, int 
     extern __shared__ unsigned char smem_raw[];
     unsigned char *smem =
         reinterpret_cast<unsigned char *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
-    __shared__ __align__(8) uint64_t full[kDwRing], empty[kDwRing], done;
+    __shared__ __align__(8) uint64_t full[kDwRing], empty[kDwRing], done, drain;
     __shared__ uint32_t s_tmem;
     const int job = blockIdx.y, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int c0 = (int)((long long)chunks * blockIdx.x / gridDim.x);
@@ -393,6 +391,7 @@ __global__ void __launch_bounds__(kDwThreads, 1) k_mlp_dw(const MlpTrain f, int 
             mbar_init(&empty[i], 1);
         }
         mbar_init(&done, 1);
+        mbar_init(&drain, 1);
         fence_mbar_init();
     }
     if (warp == 0) tmem_alloc(&s_tmem, 512);
@@ -413,11 +412,8 @@ __global__ void __launch_bounds__(kDwThreads, 1) k_mlp_dw(const MlpTrain f, int 
                 bulk_load(d, A + (size_t)c * kDwK * kWidth, kDwABytes, &full[st]);
                 bulk_load(d + kDwABytes, B + (size_t)c * kDwK * NB, bbytes, &full[st]);
             }
-            if (!ok) {
-                atomicExch(f.err, 1);
-                for (int i = max(0, u - kDwRing); i < u; ++i)
-                    mbar_wait(&full[i % kDwRing], (i / kDwRing) & 1, kWaitNs);
-            }
+            if (!ok) atomicExch(f.err, 1);
+            drain_copies(full, kDwRing, u, kWaitNs);
         }
     } else if (warp == 1) {
         if (lane == 0) {
@@ -439,6 +435,7 @@ __global__ void __launch_bounds__(kDwThreads, 1) k_mlp_dw(const MlpTrain f, int 
             }
             if (ok) umma_commit(&done);
             else atomicExch(f.err, 1);
+            drain_mmas(&drain, kWaitNs);
         }
     } else if (warp >= 4) {
         const int quarter = warp & 3, h = (warp - 4) >> 2;

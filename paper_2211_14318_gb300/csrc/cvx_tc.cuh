@@ -139,6 +139,23 @@ __device__ __forceinline__ void umma_commit(uint64_t *bar) {
         : "memory");
 }
 
+// A CTA that gives up must not end, nor free its tensor memory, while its own
+// copies and MMAs are in flight: the issuing threads wait for them (each wait
+// bounded) whether they gave up or not; in a run without a time-out all of them
+// are finished by then.
+// Copies: the last use of each stage of a ring of which `issued` uses were
+// issued, use i on barrier i % stages.
+__device__ __forceinline__ void drain_copies(uint64_t *full, int stages, int issued,
+                                             uint64_t limit_ns) {
+    for (int i = max(0, issued - stages); i < issued; ++i)
+        mbar_wait(&full[i % stages], (i / stages) & 1, limit_ns);
+}
+// MMAs of the calling thread, by a barrier of their own.
+__device__ __forceinline__ void drain_mmas(uint64_t *bar, uint64_t limit_ns) {
+    umma_commit(bar);
+    mbar_wait(bar, 0, limit_ns);
+}
+
 // 16 consecutive FP32 columns of this thread's TMEM lane (warp w of the CTA
 // reads lanes 32 (w % 4) .. +31; taddr carries the lane in bits 16..31).
 __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16]) {
