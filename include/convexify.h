@@ -548,7 +548,9 @@ int surrogate_labels(cvx_handle *h, const cvx_params *p, int64_t n, const double
  * |E_pred - V| / (1e-8 + |V|) exceeds gap_tol, where V is the
  * window's node value and E_pred = xi W(F+) + (1 - xi) W(F-) the proposed
  * laminate evaluated exactly (F+ = F + (1 - xi) amp R, F- = F - xi amp R,
- * R = a (x) b of the proposed angles, amp = jump : R).  fell_back (n, DEVICE,
+ * R = a (x) b of the proposed angles, amp = jump : R).  Should a bounded wait
+ * of the network's kernel give up, its nodes and those below them take the
+ * full scan too.  fell_back (n, DEVICE,
  * nullable) = 1 where some node of the point fell back (also status bit
  * CVX_PT_FALLBACK; nodes flagged CVX_NODE_FALLBACK).  Requires weights
  * (surrogate_train / set_weights / load); 0 <= 2 window + 1 <= min(Na, Nb). */

@@ -47,7 +47,11 @@ __global__ void k_feat(const Pipe P, int level, int off, int chunk, const float 
 // Window centre (nearest grid cell of the wrapped angles) and E_pred =
 // xi W(F+) + (1 - xi) W(F-) of the proposed laminate: R = a (x) b of the
 // unrounded angles, amp = jump : R, F+ = F + (1 - xi) amp R, F- = F - xi amp R.
-__global__ void k_decode(const Pipe P, int level, int off, int chunk, const float *out) {
+// Where the network gave up (*err), out holds no proposals: an E_pred of NaN
+// fails the energy gap test under every tolerance, so that the node takes the
+// full scan.
+__global__ void k_decode(const Pipe P, int level, int off, int chunk, const float *out,
+                         const int *err) {
     const int r = blockIdx.x * blockDim.x + threadIdx.x;
     if (r >= chunk) return;
     const int qi = off + r;
@@ -55,6 +59,11 @@ __global__ void k_decode(const Pipe P, int level, int off, int chunk, const floa
     const int p = P.qp[level][qi], hi = P.qh[level][qi];
     const ProbDesc &pd = P.probs[P.pid[p]];
     const cvx_node *nd = node_ptr(pd, p, hi);
+    if (*err) {
+        P.center[qi] = make_int2(0, 0);
+        P.e_pred[qi] = nan("");
+        return;
+    }
     const float *o = out + (long long)r * 7;
     double ta = fmod((double)o[0], kPi), tb = fmod((double)o[1], kPi);
     if (ta < 0.0) ta += kPi;
@@ -286,7 +295,7 @@ int surrogate_propose(cvx_handle *h, const cvx_params *p, int64_t n, const doubl
             CK(cudaGetLastError(), "surrogate_propose/features");
             rc = sur_infer(h, m, nullptr, S.out, s, pp.cnt + l, (int)off);
             if (rc) return rc;
-            k_decode<<<(m + 255) / 256, 256, 0, s>>>(pp, l, (int)off, m, S.out);
+            k_decode<<<(m + 255) / 256, 256, 0, s>>>(pp, l, (int)off, m, S.out, S.err);
             CK(cudaGetLastError(), "surrogate_propose/decode");
         }
         cudaEvent_t *evl = ev.empty() ? nullptr : &ev[2 * per_level * l];
@@ -303,6 +312,8 @@ int surrogate_propose(cvx_handle *h, const cvx_params *p, int64_t n, const doubl
            "surrogate_propose/fallback");
     }
     CK(pipe_end(pp, s), "surrogate_propose");
+    // acted on here: it is not for a later call to report
+    CK(cudaMemsetAsync(S.err, 0, sizeof(int), s), "surrogate_propose");
     if (fell_back) {
         k_fell_back<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(n, status, fell_back);
         CK(cudaGetLastError(), "surrogate_propose");
