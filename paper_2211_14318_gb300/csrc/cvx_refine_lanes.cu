@@ -15,14 +15,19 @@
 //  - a run from an end on the line's edge on which v is concave (and whose
 //    far end lies above the chord) needs none;
 //  - elsewhere every sample whose FP32 value is inconclusive is taken.
-// Samples on or below the chord move the pair to the lowest one of its side
-// (the supporting-slope iteration; ties to the outermost sample, as in
-// Algorithm 1).  The scan's pair is that of FP32 samples, on nearly affine
+// A sample below an end of the pair (v - s x at the chord's slope s; on equal
+// values the outer one) moves that end to the lowest one of its side: the
+// supporting-slope iteration, ties as in Algorithm 1.  A pair is done when all
+// other samples lie strictly above its chord, or when both ends are the lowest
+// of a search in full; samples within rounding of the chord need no more than
+// that.  The scan's pair is that of FP32 samples, on nearly affine
 // lines up to 64 samples off: an end in a convex run first goes to where v has
 // the chord's slope (a Newton step in FP32, twice at most), and a neighbour
 // found on or below the chord is moved to (three times at most) before its
 // side is searched in full.  None of these decides anything: the pair is done
-// when the intervals and samples above say so for its own chord.
+// when the intervals and samples above say so for its own chord.  A candidate
+// that needs too many FP64 samples has its whole line taken by the warp, each
+// sample once (ref_full).
 //
 // The samples to be taken in FP64 queue in shared memory over the warp's 32
 // candidates and are taken 32 at a time, one per lane.  What bounds the
@@ -45,6 +50,19 @@ constexpr int kRefWarps = 4;
 // a load step's proposal windows took 29 FP64 samples beside its chords' ends,
 // with them 2 (k_refine_lanes 15.9 -> 5.2 ms of a step).
 constexpr int kRefJumps = 2, kRefWalks = 3;
+// Candidates per warp at least: eight, but four where lines are longer than
+// this and more than four candidates per node are left, which is so on nearly
+// affine lines, whose searches in full are a serial chain in their warp.  2,000
+// points, 16^2 directions, L = 2049, t_half = 0.01: 10.7 ms with eight, 8.4 with
+// four; a load step's windows, one to two candidates per node, L = 1439: 0.64
+// and 0.78 ms of refinement.
+constexpr int kRefLongL = 512;
+// Half as many FP64 samples, or half the line, and the candidate has its whole
+// line taken.  2,000 points, 16^2 directions, L = 201, t_half = 1e-6 (nearly all
+// samples within rounding of the chord): 58 ms without this limit and with pairs
+// that move on to samples within rounding above their chord, 10 ms so; at half
+// the line alone, L = 33, t_half = 1e-4: 2.8 ms, with 128 at least 2.1.
+constexpr int kRefMany = 128;
 constexpr int kRefRounds = 24;  // chords per candidate before the whole line is taken in FP64
 
 // A lane's candidate as the queue's other lanes need it.
@@ -53,11 +71,17 @@ struct RefLane {
     const ProbDesc *pd;
     long long key[2];  // lowest v - s x (dkey) on or below the chord, left and right
     int k[2];          // its sample
-    int a, m0;
+    int a, m0, L;
 };
 
 __device__ __noinline__ double ref_sample(const RefLane &r, int k) {
     return sample_w64_ek(r.F, r.R, k, r.m0, r.h, r.beta, r.ek, r.pd->mat);
+}
+
+// Key of v - s x at sample k of value v, rounded once everywhere, so that keys
+// of one slope compare.
+__device__ __forceinline__ long long ref_key(double v, double s, int k, int m0) {
+    return dkey(__fma_rn(-s, (double)(k - m0), v));
 }
 
 // Takes queued samples (owner lane << 12 | sample) in FP64, 32 at a time, and
@@ -79,7 +103,7 @@ __device__ __noinline__ int ref_spots(RefLane *rl, int *q, int nq, bool all, int
             const double v = ref_sample(*r, k);
             const double line = r->wa + r->s * (double)(k - r->a);
             low = v == v && !(v > line + 1e-14 * fabs(line));  // NaN: det <= 0, excluded
-            if (low) e = dkey(v - r->s * (double)(k - r->m0));
+            if (low) e = ref_key(v, r->s, k, r->m0);
             ++n_spot;
         }
         const long long old = r->key[side];
@@ -107,19 +131,26 @@ __device__ __noinline__ int ref_spots(RefLane *rl, int *q, int nq, bool all, int
 }
 
 // The whole line in FP64 (warp-wide, for the candidate of one lane): the
-// supporting-slope iteration of bridge64, the samples taken anew in each pass.
+// supporting-slope iteration of bridge64.  Sample k is lane k % 32's k / 32-th,
+// taken once (in local memory: the passes that follow cost two FP64 operations
+// per sample, a sample some forty).
+constexpr int kFullPer = (2079 + 31) / 32;
+
 __device__ __noinline__ void ref_full(const RefLane &r, int L, int lane, int &a, int &b, double &wa,
                                       double &wb) {
-    double s = 0.0;
+    double s = 0.0, v[kFullPer];
+    for (int k = lane, i = 0; k < L; k += 32, ++i) {
+        const double x = k == r.m0 ? INFINITY : ref_sample(r, k);
+        v[i] = x == x ? x : INFINITY;
+    }
+    __syncwarp();
     a = b = -1;
     for (int it = 0; it < 128; ++it) {
         long long bl = kKeyInf, br = kKeyInf;
         int kl = INT_MAX, kr = -1;
-        for (int k = lane; k < L; k += 32) {
-            if (k == r.m0) continue;
-            const double v = ref_sample(r, k);
-            if (!(v < INFINITY)) continue;
-            const long long e = dkey(v - s * (double)(k - r.m0));
+        for (int k = lane, i = 0; k < L; k += 32, ++i) {
+            if (!(v[i] < INFINITY)) continue;
+            const long long e = ref_key(v[i], s, k, r.m0);
             if (k < r.m0) {
                 if (e < bl || (e == bl && k < kl)) {
                     bl = e;
@@ -140,8 +171,8 @@ __device__ __noinline__ void ref_full(const RefLane &r, int L, int lane, int &a,
         if (kl == a && kr == b) return;
         a = kl;
         b = kr;
-        wa = ref_sample(r, a);
-        wb = ref_sample(r, b);
+        wa = __shfl_sync(kFull, v[a >> 5], a & 31);
+        wb = __shfl_sync(kFull, v[b >> 5], b & 31);
         s = (wb - wa) / (double)(b - a);
     }
 }
@@ -170,9 +201,9 @@ __device__ __forceinline__ float tangent_step(const IvLine &l, float t, float h,
 // One warp takes 32 candidates at a time: phase 0 each node's first candidate,
 // phase 1 the others whose lower bound does not exceed the node's first value
 // (see k_refine).  With fewer candidates than lanes the warps take fewer each,
-// but eight at least: a chord's two FP64 samples cost a warp the same for 1 and
-// 32 lanes (an FE step of 20,011 points: 10.80 ms with one, 10.60 with 8,
-// 10.58 with 16, 10.64 with 32).
+// but some at least (kRefLongL): a chord's two FP64 samples cost a warp the same
+// for 1 and 32 lanes (an FE step of 20,011 points: 10.80 ms with one, 10.60 with
+// 8, 10.58 with 16, 10.64 with 32).
 // Measured per call, all launches together, against one warp per candidate
 // with 32 or 64 FP64 samples in two windows and the certificate over every
 // FP32 sample: 1,706,177 candidates at L = 201: 22.3 -> 1.25 ms (one spot
@@ -191,7 +222,8 @@ __global__ void __launch_bounds__(32 * kRefWarps) k_refine_lanes(const Pipe P, i
     const unsigned below = (1u << lane) - 1u;
     const int nwarps = gridDim.x * kRefWarps, gw = blockIdx.x * kRefWarps + warp;
     const int nwork = P.cnt[(P.K + 1) + level];
-    const int bs = min(32, max(8, (nwork + nwarps - 1) / nwarps));
+    const int least = P.stride32 > kRefLongL && nwork > 4 * P.cnt[level] ? 4 : 8;
+    const int bs = min(32, max(least, (nwork + nwarps - 1) / nwarps));
     const int32_t *qp = P.qp[level], *qh = P.qh[level];
     unsigned n_ref = 0, n_full = 0, n_spot = 0;
     long long blk = gw;
@@ -252,6 +284,7 @@ __global__ void __launch_bounds__(32 * kRefWarps) k_refine_lanes(const Pipe P, i
             my.h = ln.h64;
             my.pd = &pd;
             my.m0 = m0;
+            my.L = L;
         }
         const DirLine dl =
             make_dir_line<CVX_ENERGY_NH_DAMAGE>(nc.nl, P.dir32[pd.dir_off + dir]);
@@ -265,6 +298,7 @@ __global__ void __launch_bounds__(32 * kRefWarps) k_refine_lanes(const Pipe P, i
         bool done = !act || slow;
         bool newA = true, newB = true, fullL = false, fullR = false;
         int jumps = 0, walks = 0;  // tangent steps and neighbour moves taken
+        int taken = 0;             // FP64 samples taken beside the chords' ends
         double wa = 0.0, wb = 0.0;
         __syncwarp();
 
@@ -355,6 +389,7 @@ __global__ void __launch_bounds__(32 * kRefWarps) k_refine_lanes(const Pipe P, i
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
                 const unsigned bal = __ballot_sync(kFull, spot[i] >= 0);
+                taken += spot[i] >= 0 ? 1 : 0;
                 if (spot[i] >= 0) q[nq + __popc(bal & below)] = (lane << 12) | spot[i];
                 nq += __popc(bal);
                 __syncwarp();
@@ -392,6 +427,7 @@ __global__ void __launch_bounds__(32 * kRefWarps) k_refine_lanes(const Pipe P, i
                             need = !(__fsub_rn(v[i], Lv) > 1.001f * err);  // else above the chord
                         }
                         const unsigned bal = __ballot_sync(kFull, need);
+                        taken += need ? 1 : 0;
                         if (need) q[nq + __popc(bal & below)] = (lane << 12) | ks;
                         nq += __popc(bal);
                     }
@@ -404,40 +440,47 @@ __global__ void __launch_bounds__(32 * kRefWarps) k_refine_lanes(const Pipe P, i
             // ---- certified, or on to the next chord
             if (!done && !moved) {
                 const bool lowL = my.key[0] < kKeyInf, lowR = my.key[1] < kKeyInf;
-                if (!lowL && !lowR) done = true;
-                // a side searched in full moves to its lowest sample; where only
-                // neighbours were taken, to the lower neighbour a few times, then
-                // the side is searched in full
-                const bool step = walks < kRefWalks;
-                if (lowL || lowR) ++walks;
+                // of the samples on or below the chord, and those within rounding
+                // above it, only one below the pair's end moves it (on equal values
+                // the outermost, as in bridge64)
+                bool betL = false, betR = false;
                 if (lowL) {
-                    if (fullL || step) {
-                        a = my.k[0];
-                        newA = true;
-                    }
-                    fullL = !(fullL || step);
+                    const long long e = ref_key(wa, s, a, m0);
+                    betL = my.key[0] < e || (my.key[0] == e && my.k[0] < a);
                 }
                 if (lowR) {
-                    if (fullR || step) {
-                        b = my.k[1];
-                        newB = true;
-                    }
-                    fullR = !(fullR || step);
+                    const long long e = ref_key(wb, s, b, m0);
+                    betR = my.key[1] < e || (my.key[1] == e && my.k[1] > b);
                 }
-                // the chord changed: start from the neighbours again
-                if (newA || newB) {
-                    fullL = lowL && fullL;
-                    fullR = lowR && fullR;
+                if (!betL && !betR && (fullL || !lowL) && (fullR || !lowR)) {
+                    done = true;
+                } else if (2 * taken > max(my.L, kRefMany)) {
+                    // most of the line is within rounding of its chord: one pass over
+                    // it costs less than further chords
+                    slow = done = true;
+                } else {
+                    // a side searched in full moves to its lowest sample; where only
+                    // neighbours were taken, to the lower neighbour a few times, then
+                    // the side is searched in full
+                    const bool step = walks++ < kRefWalks;
+                    newA = betL && (fullL || step);
+                    newB = betR && (fullR || step);
+                    if (newA) a = my.k[0];
+                    if (newB) b = my.k[1];
+                    // where the chord changed, start from the neighbours again
+                    const bool same = !newA && !newB;
+                    fullL = lowL ? !newA : fullL && same;
+                    fullR = lowR ? !newB : fullR && same;
                 }
             }
             __syncwarp();
         }
         if (!done) slow = true;
         for (unsigned sl = __ballot_sync(kFull, slow); sl; sl &= sl - 1) {
-            const int o = __ffs(sl) - 1, Lo = __shfl_sync(kFull, L, o);
+            const int o = __ffs(sl) - 1;
             int fa, fb;
             double fwa = 0.0, fwb = 0.0;
-            ref_full(rl[o], Lo, lane, fa, fb, fwa, fwb);
+            ref_full(rl[o], rl[o].L, lane, fa, fb, fwa, fwb);
             if (lane == o) {
                 a = fa;
                 b = fb;
