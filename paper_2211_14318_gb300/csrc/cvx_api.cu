@@ -174,10 +174,11 @@ int ensure_dirs(cvx_handle *h, const cvx_params *p, cudaStream_t s) {
         CK(cudaMalloc(&h->d_dir64, sizeof(double) * 4 * D), "direction table");
         h->dir_cap = D;
     }
-    // synchronous copies: the host vectors die at return
-    CK(cudaMemcpy(h->d_dir32, d32.data(), sizeof(float4) * D, cudaMemcpyHostToDevice),
+    // on the stream that reads them next; pageable sources, so they are staged
+    // at return (the host vectors die)
+    CK(cudaMemcpyAsync(h->d_dir32, d32.data(), sizeof(float4) * D, cudaMemcpyHostToDevice, s),
        "direction table");
-    CK(cudaMemcpy(h->d_dir64, d64.data(), sizeof(double) * 4 * D, cudaMemcpyHostToDevice),
+    CK(cudaMemcpyAsync(h->d_dir64, d64.data(), sizeof(double) * 4 * D, cudaMemcpyHostToDevice, s),
        "direction table");
     h->D = D;
     h->dir_custom = p->dirs != nullptr;

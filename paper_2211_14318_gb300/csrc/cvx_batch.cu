@@ -266,9 +266,10 @@ int convexify_batch(cvx_handle *h, int np, const cvx_problem *pr, cvx_stream sv)
                                (float)all64[4 * k + 2], (float)all64[4 * k + 3]);
     CK(cudaMalloc(&plan->d_dir32, sizeof(float4) * Dall), "convexify_batch/directions");
     CK(cudaMalloc(&plan->d_dir64, sizeof(double) * 4 * Dall), "convexify_batch/directions");
-    CK(cudaMemcpy(plan->d_dir32, all32.data(), sizeof(float4) * Dall, cudaMemcpyHostToDevice),
+    // on the stream that reads them next (pageable sources: staged at return)
+    CK(cudaMemcpyAsync(plan->d_dir32, all32.data(), sizeof(float4) * Dall, cudaMemcpyHostToDevice, s),
        "convexify_batch/directions");
-    CK(cudaMemcpy(plan->d_dir64, all64.data(), sizeof(double) * 4 * Dall, cudaMemcpyHostToDevice),
+    CK(cudaMemcpyAsync(plan->d_dir64, all64.data(), sizeof(double) * 4 * Dall, cudaMemcpyHostToDevice, s),
        "convexify_batch/directions");
 
     // launch shape: cached, or timed trials on a sample of the points

@@ -120,6 +120,9 @@ int sur_params(cvx_handle *h) {
         CK(alloc(&S.Wt[l], n), "surrogate");
         CK(cudaMemset(S.Wt[l], 0, sizeof(bf16) * n), "surrogate");
     }
+    // the handle's calls may use any stream, which the legacy stream's fills do
+    // not precede by themselves
+    CK(cudaDeviceSynchronize(), "surrogate");
     return CVX_OK;
 }
 
@@ -273,10 +276,11 @@ int upload_weights(cvx_handle *h, const float *params, const float *mean, const 
         S.scale_h[k] = mean[k];
         S.scale_h[6 + k] = 1.0f / stdv[k];
     }
-    CK(cudaMemcpy(S.scale, S.scale_h, sizeof(float) * 12, cudaMemcpyHostToDevice), "surrogate");
-    CK(cudaMemcpy(S.w, params, sizeof(float) * kSurParams, cudaMemcpyHostToDevice), "surrogate");
-    CK(cudaMemset(S.m, 0, sizeof(float) * kSurParams), "surrogate");
-    CK(cudaMemset(S.v, 0, sizeof(float) * kSurParams), "surrogate");
+    // on the stream that reads them next (pageable sources: staged at return)
+    CK(cudaMemcpyAsync(S.scale, S.scale_h, sizeof(float) * 12, cudaMemcpyHostToDevice, s), "surrogate");
+    CK(cudaMemcpyAsync(S.w, params, sizeof(float) * kSurParams, cudaMemcpyHostToDevice, s), "surrogate");
+    CK(cudaMemsetAsync(S.m, 0, sizeof(float) * kSurParams, s), "surrogate");
+    CK(cudaMemsetAsync(S.v, 0, sizeof(float) * kSurParams, s), "surrogate");
     S.adam_t = 0;
     CK(sur_pack(S, s), "surrogate pack");
     S.has_weights = true;
