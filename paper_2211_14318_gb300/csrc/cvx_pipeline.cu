@@ -1433,7 +1433,14 @@ static cudaError_t launch_scan_t(const Pipe &p, int level, int warps, int grid, 
 // Threads per block of a kernel with one thread per point or node: a warp per
 // block while that leaves SMs without one (the warps of a block share its SM's
 // FP64 pipe, 2 lanes per clock, which is what these kernels wait for).
-static int point_threads(long long n, int threads) { return n <= 32 * 152 ? 32 : threads; }
+static int point_threads(long long n, int threads, int sms) { return n <= 32LL * sms ? 32 : threads; }
+
+static int device_sms() {
+    int dev = 0, sms = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    return sms;
+}
 
 cudaError_t pipe_begin(const Pipe &p, cudaStream_t s) {
     cudaError_t e;
@@ -1464,7 +1471,7 @@ cudaError_t pipe_begin(const Pipe &p, cudaStream_t s) {
             cudaSuccess)
             return e;
     }
-    const int T = point_threads(p.N, 256);
+    const int T = point_threads(p.N, 256, device_sms());
     k_init<<<(unsigned)((p.N + T - 1) / T), T, 0, s>>>(p);
     return cudaGetLastError();
 }
@@ -1472,11 +1479,9 @@ cudaError_t pipe_begin(const Pipe &p, cudaStream_t s) {
 cudaError_t pipe_level(const Pipe &p, int l, int warps, int grid, cudaStream_t s,
                        cudaEvent_t *ev) {
     cudaError_t e;
-    int dev = 0, sms = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    const int sms = device_sms();
     const long long max_nodes = p.N << l;
-    const int T = point_threads(max_nodes, 128);
+    const int T = point_threads(max_nodes, 128, sms);
     const unsigned nb = (unsigned)((max_nodes + T - 1) / T);
     k_nodes<<<nb, T, 0, s>>>(p, l);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
@@ -1514,7 +1519,7 @@ cudaError_t pipe_level(const Pipe &p, int l, int warps, int grid, cudaStream_t s
 }
 
 cudaError_t pipe_end(const Pipe &p, cudaStream_t s) {
-    const int T = point_threads(p.N, kLeafThreads);
+    const int T = point_threads(p.N, kLeafThreads, device_sms());
     k_leaf<<<(unsigned)((p.N + T - 1) / T), T, 0, s>>>(p);
     return cudaGetLastError();
 }
