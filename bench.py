@@ -43,12 +43,13 @@ METRIC = "quadrature points convexified/s (W^R+P) at 1e-6 rel. error, surrogate 
 MAT = dict(mu=1.0, lambda_L=5.0, D_inf=0.99, D0=0.5)
 NX, STRETCH, ANGLES, LINE, DEPTH, T_HALF = 128, 1.3, 64, 1025, 3, 0.5
 # algorithmic FP32 work per valid line sample (energy 22 + hull 8).  The line scan
-# does not take every sample: a part of a line whose bound lies above the minimum
-# looked for is left out, so that "achieved" is the rate of a scan that takes them
-# all (it can exceed the peak); the same holds for the grid's line kernel, which
-# takes no FP64 step where an FP32 bound decides
+# does not take every sample (a part of a line whose bound lies above the minimum
+# looked for is left out), so that a rate counted this way is that of a scan that
+# takes them all and no use of a pipe: it is reported as such, beside the rooflines,
+# which count the instructions that the kernels execute; likewise for the grid's
+# line kernel, which takes no FP64 step where an FP32 bound decides
 FLOP_PER_SAMPLE = 30
-FP32_LANES_PER_SM = 128
+ISSUE_PER_SM = 4  # warp instructions per SM and clock
 
 
 def workload_desc(n):
@@ -213,7 +214,8 @@ class ClockSampler:
 
 
 # ---------------------------------------------------------------- roofline
-def fp32_peak_tflops(torch, dev):
+def issue_peak(torch, dev):
+    """Warp instructions (1e9/s) that the SMs can issue, SMs, clock, its source."""
     props = torch.cuda.get_device_properties(dev)
     mhz = 2070.0
     src = "sm_max_mhz 2070 (nominal)"
@@ -225,7 +227,7 @@ def fp32_peak_tflops(torch, dev):
     except (OSError, ValueError):
         pass
     sms = props.multi_processor_count
-    return sms * FP32_LANES_PER_SM * 2 * mhz * 1e6 / 1e12, sms, mhz, src
+    return sms * ISSUE_PER_SM * mhz / 1e3, sms, mhz, src
 
 
 # the translation unit of k_scan_lanes (the kernel and its launch) and the
@@ -259,18 +261,36 @@ def scan_source_hash(sources=SCAN_SOURCES):
     return h.hexdigest()[:16]
 
 
-def traffic_per_launch(valid_per_launch, name="k_scan_traffic.json", sources=SCAN_SOURCES):
-    """DRAM bytes per launch from the committed ncu summary, scaled to this
-    launch's work; None if the kernel changed since the capture."""
-    path = os.path.join(ROOT, "profiles", name)
+def captured(name, sources=SCAN_SOURCES):
+    """The committed ncu summary of a kernel's launch; None if the kernel changed
+    since the capture."""
     try:
-        t = json.load(open(path))
+        t = json.load(open(os.path.join(ROOT, "profiles", name)))
     except (OSError, ValueError):
         return None
-    if t.get("source_sha") != scan_source_hash(sources):
-        return None
-    per_sample = t["dram_bytes"] / max(1, t["valid_samples"])
-    return per_sample * valid_per_launch
+    return t if t.get("source_sha") == scan_source_hash(sources) else None
+
+
+def roofline_obj(kernel, unit, units, ms, launches, step_ms, peak, sms, mhz, peak_src,
+                 capture=None, sources=SCAN_SOURCES, full_flop=FLOP_PER_SAMPLE):
+    """The kernel's warp instructions per second against what the SMs can issue:
+    instructions per unit of work (a valid line sample, a grid point and
+    direction) from a committed counter capture, times the units and over the
+    time of the timed launches; DRAM bytes per launch likewise.  None where there
+    is no capture of the present kernel."""
+    t = captured(capture, sources) if capture else None
+    per = 1.0 / max(1, t["valid_samples"]) if t else 0.0
+    achieved = t["warp_instructions"] * per * units / (ms / 1e3) / 1e9 if t and ms > 0 else None
+    return {"bound": "alu", "kernel": kernel, "achieved": achieved, "peak": peak,
+            "unit": "1e9 warp instructions/s", "frac": achieved / peak if achieved else None,
+            "traffic": t["dram_bytes"] * per * units / max(1, launches) if t else None,
+            "peak_source": f"{sms} SMs x {ISSUE_PER_SM} issued per clock x {mhz:.0f} MHz ({peak_src})",
+            "counted": (f"executed warp instructions per {unit} of profiles/{capture}" if t else
+                        "no counter capture of this workload with the present kernel"),
+            "every_unit": {"tflops": full_flop * units / (ms / 1e3) / 1e12 if ms > 0 else None,
+                           "flop": full_flop, "per": unit,
+                           "meaning": "the rate of a form that takes every one; not a pipe's use"},
+            "kernel_share_of_step": ms / step_ms if step_ms else None, "launches": launches}
 
 
 # ----------------------------------------------------------------- oracle arm
@@ -421,11 +441,7 @@ def run_ours(a):
                             dist if ws > 1 else None, dev)
     e2e_value = whole_job_rate(n, ws, a.steps, e2e_ms)
 
-    peak, sms, mhz, peak_src = fp32_peak_tflops(torch, dev)
-    flop = FLOP_PER_SAMPLE * st["valid_samples"]
-    achieved = flop / (scan_ms / 1e3) / 1e12 if scan_ms > 0 else None
-    valid_per_launch = st["valid_samples"] / max(1, scan_launches)
-    traffic = traffic_per_launch(valid_per_launch)
+    peak, sms, mhz, peak_src = issue_peak(torch, dev)
 
     if rank == 0:
         cpu = None
@@ -447,14 +463,8 @@ def run_ours(a):
                        "points_per_gpu": n, "angles": [ANGLES, ANGLES], "line_points": LINE,
                        "depth": DEPTH, "l2": "flushed between steps (512 MiB write)",
                        "wall_s_timed_region": wall},
-            "roofline": {"bound": "alu", "kernel": "k_scan", "achieved": achieved,
-                         "peak": peak, "unit": "TFLOP/s",
-                         "frac": (achieved / peak) if achieved else None,
-                         "traffic": traffic,
-                         "peak_source": f"{sms} SMs x {FP32_LANES_PER_SM} FP32 lanes x 2 x {mhz:.0f} MHz ({peak_src})",
-                         "flop_per_valid_sample": FLOP_PER_SAMPLE, "flop_counted": "every valid sample",
-                         "kernel_share_of_step": scan_ms / dev_ms if dev_ms else None,
-                         "launches": scan_launches},
+            "roofline": scan_roofline(st, scan_ms, scan_launches, dev_ms, peak, sms, mhz, peak_src,
+                                      "k_scan_lanes_mesh_traffic.json" if a.nx == NX else None),
             "cpu_baseline": cpu,
             "e2e": {"value": e2e_value, "unit": "points/s",
                     "h2d_bytes_per_step": 2 * n * 4 * 8, "d2h_bytes_per_step": n * 8 + n * 4 * 8},
@@ -572,18 +582,9 @@ def timed_full_scan(cv, p, F, beta, steps, torch):
     return ms, scan_ms, launches, st, out
 
 
-def roofline_obj(st, scan_ms, launches, step_ms, peak, sms, mhz, peak_src, traffic_name=None):
-    flop = FLOP_PER_SAMPLE * st["valid_samples"]
-    achieved = flop / (scan_ms / 1e3) / 1e12 if scan_ms > 0 else None
-    traffic = (traffic_per_launch(st["valid_samples"] / max(1, launches), traffic_name)
-               if traffic_name else None)
-    return {"bound": "alu", "kernel": "k_scan_lanes", "achieved": achieved, "peak": peak,
-            "unit": "TFLOP/s", "frac": (achieved / peak) if achieved else None,
-            "traffic": traffic,
-            "peak_source": f"{sms} SMs x {FP32_LANES_PER_SM} FP32 lanes x 2 x {mhz:.0f} MHz ({peak_src})",
-            "flop_per_valid_sample": FLOP_PER_SAMPLE, "flop_counted": "every valid sample",
-            "kernel_share_of_step": scan_ms / step_ms if step_ms else None,
-            "launches": launches}
+def scan_roofline(st, scan_ms, launches, step_ms, peak, sms, mhz, peak_src, capture=None):
+    return roofline_obj("k_scan_lanes", "valid line sample", st["valid_samples"], scan_ms, launches,
+                        step_ms, peak, sms, mhz, peak_src, capture)
 
 
 def run_loadpath(a):
@@ -709,7 +710,7 @@ def run_loadpath(a):
     else:
         value = whole_job_rate(n, ws, K, t_max)
         e2e_value = whole_job_rate(n, ws, K, e2e_max)
-    peak, sms, mhz, peak_src = fp32_peak_tflops(torch, dev)
+    peak, sms, mhz, peak_src = issue_peak(torch, dev)
 
     if rank == 0:
         # accuracy of the proposed form against the oracle (stored results)
@@ -783,8 +784,8 @@ def run_loadpath(a):
                 "l2": "flushed between steps (512 MiB write)",
                 "timed": "H2D of F excluded from value (included in e2e); proposal + history update",
                 "wall_s_timed_region": wall},
-            "roofline": roofline_obj(st, scan_ms, scan_launches, comp_ms, peak, sms, mhz, peak_src,
-                                     "k_scan_lanes_traffic.json"),
+            "roofline": scan_roofline(st, scan_ms, scan_launches, comp_ms, peak, sms, mhz, peak_src,
+                                      "k_scan_lanes_traffic.json"),
             "cpu_baseline": cpu,
             "e2e": {"value": e2e_value, "unit": "points/s", "h2d_bytes_per_step": n * 4 * 8,
                     "d2h_bytes_per_step": n * 8 + n * 4 * 8},
@@ -834,8 +835,8 @@ def material_points_line(a, cv, api, inputs, torch, dev, peak, sms, mhz, peak_sr
                         f", depth {MP_DEPTH}, full scan"),
            "value": npts * steps / (ms / 1e3), "unit": "points/s", "steps": steps,
            "ms_per_step": ms / steps,
-           "roofline": roofline_obj(st, scan_ms, launches, ms, peak, sms, mhz, peak_src,
-                                    "k_scan_lanes_l201_traffic.json"),
+           "roofline": scan_roofline(st, scan_ms, launches, ms, peak, sms, mhz, peak_src,
+                                     None if doublings else "k_scan_lanes_l201_traffic.json"),
            "stats": st}
     if g is not None and not doublings:
         it = torch.from_numpy(g["idx"]).to(dev)
@@ -871,7 +872,8 @@ def mesh128_line(cv, api, torch, dev, peak, sms, mhz, peak_src, steps):
     ms, scan_ms, launches, st, out = timed_full_scan(cv, p, Fd, bd, steps, torch)
     res = {"workload": workload_desc(F.shape[0]), "value": F.shape[0] * steps / (ms / 1e3),
            "unit": "points/s", "steps": steps, "ms_per_step": ms / steps,
-           "roofline": roofline_obj(st, scan_ms, launches, ms, peak, sms, mhz, peak_src),
+           "roofline": scan_roofline(st, scan_ms, launches, ms, peak, sms, mhz, peak_src,
+                                     "k_scan_lanes_mesh_traffic.json"),
            "stats": st}
     if g is not None:
         it = torch.from_numpy(g["idx"]).to(dev)
@@ -886,7 +888,6 @@ GRID61 = dict(diag=(0.1, 3.4), off=(-2.55, 2.55), delta=(0.15, 0.15), beta=0.06,
 # the strong-scaling study of Sec. 6.4 times a 43,681-point grid (11 x 19 x 19 x 11
 # points) whose bounds are not printed; this one has that shape at delta 0.15
 GRID_SCALING = dict(diag=(0.4, 1.9), off=(-1.35, 1.35), delta=(0.15, 0.15))
-FP64_FMA_PER_SM = 2       # FP64 FMA per SM per clock on GB300 (1.25 TFLOP/s nominal)
 GRID_FLOP_PER_POINT_DIR = 12  # Algorithm 1 (2 predicates x 4) + the chord at the point (4)
 
 
@@ -895,7 +896,7 @@ def global_grid_line(a, cv, api, inputs, torch, dev, sms, mhz, peak_src, runs=10
     """The paper's own algorithm on the grid of its Sec. 6.1 study: 648,025
     grid points, R^1_1, W^0 then Eq. (4.3) until the largest decrease is at
     most 1e-4 (15 steps), timed whole on the device (L2 flushed before each
-    run); the line kernel's roofline against the FP64 pipe; Algorithms 2/3 at
+    run); the line kernel's roofline; Algorithms 2/3 at
     1,048,576 query points; accuracy against the stored oracle results."""
     import numpy as np
 
@@ -937,10 +938,6 @@ def global_grid_line(a, cv, api, inputs, torch, dev, sms, mhz, peak_src, runs=10
     torch.cuda.synchronize()
     lines_ms, launches = cv.scan_timing(reset=True)
     cv.set_profiling(False)
-    flop = GRID_FLOP_PER_POINT_DIR * N * nd * launches
-    peak = sms * FP64_FMA_PER_SM * 2 * mhz * 1e6 / 1e12
-    achieved = flop / (lines_ms / 1e3) / 1e12 if lines_ms > 0 else None
-    traffic = traffic_per_launch(N * nd, "k_grid_lines_traffic.json", GRID_SOURCES)
     res = {"workload": (f"global grid of the Sec. 6.1 NH study: {g.n[0]}x{g.n[1]}x{g.n[2]}x{g.n[3]} "
                         f"= {N} grid points (delta 0.15, diagonal {list(c['diag'])}, off-diagonal "
                         f"{list(c['off'])}), R^1_1 ({nd} directions), beta_k {c['beta']}, "
@@ -948,14 +945,10 @@ def global_grid_line(a, cv, api, inputs, torch, dev, sms, mhz, peak_src, runs=10
            "value": N * K / (t / 1e3), "unit": "grid-point updates/s (points x steps)",
            "steps_to_tol": K, "ms_to_tol": t, "ms_runs": ms,
            "l2": "flushed before each run (256 MiB write); the grid (5.2 MB) fits in L2 within a run",
-           "roofline": {"bound": "alu", "kernel": "k_grid_lines", "achieved": achieved,
-                        "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak if achieved else None,
-                        "traffic": traffic,
-                        "peak_source": (f"{sms} SMs x {FP64_FMA_PER_SM} FP64 FMA x 2 x {mhz:.0f} MHz "
-                                        f"(nominal FP64 rate; {peak_src})"),
-                        "flop_per_point_direction": GRID_FLOP_PER_POINT_DIR,
-                        "kernel_ms_per_launch": lines_ms / max(1, launches),
-                        "kernel_share": lines_ms / t, "launches": launches},
+           "roofline": roofline_obj("k_grid_lines", "grid point and direction", N * nd * launches,
+                                    lines_ms, launches, t, sms * ISSUE_PER_SM * mhz / 1e3, sms, mhz,
+                                    peak_src, "k_grid_lines_traffic.json", GRID_SOURCES,
+                                    GRID_FLOP_PER_POINT_DIR),
            "gpu_launches_per_run": 1 + 2 + c["kmax"] * 3 + 1}
     # Algorithms 2 and 3 at 1,048,576 points of the grid's box
     lo = np.array(g.lo)
@@ -1071,15 +1064,11 @@ def grid_study_line(cv, api, torch, dev, flush, name, sms, mhz, runs=5):
     lines_ms, launches = cv.scan_timing(reset=True)
     cv.set_profiling(False)
     chunks = max(1, launches // K)
-    flop = GRID_FLOP_PER_POINT_DIR * N * nd * K
-    peak = sms * FP64_FMA_PER_SM * 2 * mhz * 1e6 / 1e12
-    achieved = flop / (lines_ms / 1e3) / 1e12 if lines_ms > 0 else None
     res = {"workload": (f"{'STVK study of Sec. 6.1' if name == 'stvk61' else 'nine-dimensional NH study of Sec. 6.8'}: "
                         f"{N} grid points, {nd} directions, tol 1e-4"),
            "value": N * K / (t / 1e3), "unit": "grid-point updates/s (points x steps)",
            "steps_to_tol": K, "ms_to_tol": t,
-           "line_kernel": {"achieved_tflops": achieved, "frac_of_fp64_peak": achieved / peak if achieved else None,
-                           "ms_per_step": lines_ms / K, "launches_per_step": chunks,
+           "line_kernel": {"ms_per_step": lines_ms / K, "launches_per_step": chunks,
                            "share": lines_ms / t}}
     if gold is not None:
         WK = out["W"].cpu().numpy()
@@ -1128,7 +1117,7 @@ def run_grid(a):
     dev = torch.device("cuda:0")
     torch.cuda.set_device(0)
     cv = api.Convexifier(0)
-    _, sms, mhz, peak_src = fp32_peak_tflops(torch, dev)
+    _, sms, mhz, peak_src = issue_peak(torch, dev)
     uuid = getattr(torch.cuda.get_device_properties(dev), "uuid", None)
     clocks = ClockSampler(f"GPU-{uuid}" if uuid is not None else "0")
     clocks.start()
@@ -1467,7 +1456,6 @@ def run_batch(a):
     cv2.close()
     os.remove(cache)
     flop = FLOP_PER_SAMPLE * st["valid_samples"]
-    peak = fp32_peak_tflops(torch, dev)[0]
     line = {
         "metric": "quadrature points convexified/s (W^R+P), batched form",
         "value": total * a.steps / (ms / 1e3), "unit": "points/s", "n_gpus": 1,
@@ -1483,10 +1471,10 @@ def run_batch(a):
                      "default_shape_pts_per_s": total * a.steps / (ms_def / 1e3),
                      "default_shape": list(tune_def[:2]), "from_cache": tune_def[2],
                      "gain": ms_def / ms},
-        "step_flop_rate": {"achieved": flop / (ms / 1e3) / 1e12, "peak": peak, "unit": "TFLOP/s",
-                           "frac": flop / (ms / 1e3) / 1e12 / peak,
-                           "note": "30 FLOP per valid sample over the whole replay (all kernels): "
-                                   "a lower bound of the line scan's own rate"},
+        "every_sample_rate": {"tflops": flop / (ms / 1e3) / 1e12, "flop_per_valid_sample": FLOP_PER_SAMPLE,
+                              "meaning": "the rate of a scan that takes every valid sample, over the "
+                                         "whole replay; the present one leaves most of them out, so "
+                                         "it is not a pipe's use"},
         "stats": st,
     }
     print(json.dumps(line), flush=True)
@@ -1505,7 +1493,7 @@ def run_material_points(a):
     dev = torch.device("cuda:0")
     torch.cuda.set_device(0)
     cv = api.Convexifier(0)
-    peak, sms, mhz, peak_src = fp32_peak_tflops(torch, dev)
+    peak, sms, mhz, peak_src = issue_peak(torch, dev)
     res = material_points_line(a, cv, api, inputs, torch, dev, peak, sms, mhz, peak_src, a.steps)
     res.update(metric="quadrature points convexified/s (W^R+P), full scan", n_gpus=1,
                warmup=2, higher_is_better=True, dtype="f32/f64", data="synthetic")
