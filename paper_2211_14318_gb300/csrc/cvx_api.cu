@@ -457,6 +457,7 @@ int convexify_points(cvx_handle *h, const cvx_params *p, int64_t n, const double
     pp.K = p->depth;
     pp.C = pd.chunks;
     pp.stride32 = pp.stride64 = pd.line.stride;
+    pp.t_half = (float)p->t_half;
     pp.energy = p->energy;
     pp.lanes = lanes ? 1 : 0;
     pp.adaptive = CVX_WINDOW_DOUBLINGS_OF(p->flags);

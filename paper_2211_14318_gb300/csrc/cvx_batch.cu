@@ -122,10 +122,12 @@ int build_layout(cvx_handle *h, int np, const cvx_problem *pr, const std::vector
                  const std::vector<int> &dir_off, const float4 *d32, const double *d64, int warps,
                  int dpi_cap, cudaStream_t s, Layout &lo) {
     int stride = 4;
+    float t_half = 0.0f;
     int K = 0;
     long long N = 0;
     for (int i = 0; i < np; ++i) {
         stride = std::max(stride, line_stride(pr[i].params.line_points));
+        t_half = std::max(t_half, (float)pr[i].params.t_half);
         K = std::max(K, pr[i].params.depth);
         N += n_use[i];
     }
@@ -179,6 +181,7 @@ int build_layout(cvx_handle *h, int np, const cvx_problem *pr, const std::vector
     pp.K = K;
     pp.C = C;
     pp.stride32 = pp.stride64 = stride;
+    pp.t_half = t_half;
     pp.energy = energy;
     pp.lanes = lanes ? 1 : 0;
     pp.adaptive = A;

@@ -143,6 +143,7 @@ struct Pipe {
     int K;               // largest depth
     int C;               // item stride per node (largest chunks)
     int stride32, stride64;
+    float t_half;        // the widest line window of any problem
     int energy;
     int32_t *pid;        // problem of each global point
     int32_t *qp[kMaxDepth], *qh[kMaxDepth];  // node queues per level

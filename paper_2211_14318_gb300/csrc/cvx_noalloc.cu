@@ -197,6 +197,7 @@ extern "C" int convexify_points_static(const cvx_params *p, int64_t n, const dou
     pp.K = K;
     pp.C = chunks;
     pp.stride32 = pp.stride64 = ln.stride;
+    pp.t_half = (float)p->t_half;
     pp.energy = p->energy;
     pp.lanes = lanes ? 1 : 0;
     pipe_layout(pp, ws + o_pipe);

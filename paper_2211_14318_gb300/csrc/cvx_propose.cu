@@ -253,6 +253,7 @@ int surrogate_propose(cvx_handle *h, const cvx_params *p, int64_t n, const doubl
     pp.C = std::max(std::max(pd.chunks, pd.wchunks), mirror ? mwchunks : 0);
     pp.mirror_on = mirror ? 1 : 0;
     pp.stride32 = pp.stride64 = pd.line.stride;
+    pp.t_half = (float)p->t_half;
     pp.energy = p->energy;
     pp.window = 1;
     pp.lanes = lanes ? 1 : 0;

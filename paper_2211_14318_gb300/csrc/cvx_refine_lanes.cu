@@ -51,12 +51,14 @@ constexpr int kRefWarps = 4;
 // with them 2 (k_refine_lanes 15.9 -> 5.2 ms of a step).
 constexpr int kRefJumps = 2, kRefWalks = 3;
 // Candidates per warp at least: eight, but four where lines are longer than
-// this and more than four candidates per node are left, which is so on nearly
-// affine lines, whose searches in full are a serial chain in their warp.  2,000
-// points, 16^2 directions, L = 2049, t_half = 0.01: 10.7 ms with eight, 8.4 with
-// four; a load step's windows, one to two candidates per node, L = 1439: 0.64
-// and 0.78 ms of refinement.
+// kRefLongL in a window narrower than kRefNarrow: lines are nearly affine there,
+// and their searches in full a serial chain in their warp.  2,000 points, 16^2
+// directions, L = 2049, t_half = 0.01: 10.7 ms with eight, 8.4 with four; in
+// windows of 0.5 the FP64 pipe counts, which a half-filled warp loads as much: a
+// mesh of 676 points, 30^2 directions, L = 987: 96 us of refinement with eight,
+// 125 with four.
 constexpr int kRefLongL = 512;
+constexpr float kRefNarrow = 0.03f;
 // Half as many FP64 samples, or half the line, and the candidate has its whole
 // line taken.  2,000 points, 16^2 directions, L = 201, t_half = 1e-6 (nearly all
 // samples within rounding of the chord): 58 ms without this limit and with pairs
@@ -222,7 +224,7 @@ __global__ void __launch_bounds__(32 * kRefWarps) k_refine_lanes(const Pipe P, i
     const unsigned below = (1u << lane) - 1u;
     const int nwarps = gridDim.x * kRefWarps, gw = blockIdx.x * kRefWarps + warp;
     const int nwork = P.cnt[(P.K + 1) + level];
-    const int least = P.stride32 > kRefLongL && nwork > 4 * P.cnt[level] ? 4 : 8;
+    const int least = P.stride32 > kRefLongL && P.t_half < kRefNarrow ? 4 : 8;
     const int bs = min(32, max(least, (nwork + nwarps - 1) / nwarps));
     const int32_t *qp = P.qp[level], *qh = P.qh[level];
     unsigned n_ref = 0, n_full = 0, n_spot = 0;
