@@ -143,10 +143,18 @@ struct LaneTasks {
 // within 2 % of each other).
 constexpr int kOwnMin = 24;
 // Lines of up to this many samples (the longest of a launch) are sampled by
-// their own lanes only: a short line's intervals (6 pairs of samples at most)
-// cost less than their queue.  1,048,576 points, L = 201: 57.3 ms without the
-// queue, 61.0 with it; an FE step at L = 333: 10.7 and 9.9 ms.
-constexpr int kOwnMaxL = 256;
+// their own lanes only: a short line's few intervals of few samples cost less
+// than their queue.  With doubled windows (P.adaptive) the lines of a warp differ
+// more in their intervals, and the queue gains sooner.  Time with the queue over
+// time without, at L = 201 / 265 / 333 / 513 / 769 / 1025 / 2049:
+//   points (16 x 16 angles)         1.08 / 1.06 / 1.04 / 1.04 / 1.00 / 0.97 / 0.87
+//   an FE step's, window fixed         - / 1.07 / 1.06 / 1.05 / 1.03 / 1.00 / 0.93
+//   a load step's proposal windows     - / 1.05 / 1.05 / 1.04 / 1.02 / 1.01 / 0.96
+//   a mesh (64 x 64)                   - / 1.02 / 0.99 / 0.97 / 0.97 / 0.95 / 0.85
+//   an FE step, up to 3 doublings   1.03 / 0.96 / 0.93 / 0.88 / 0.87 / 0.84 / -
+// The fixed windows cross between 320 (mesh) and 1,100 samples (proposals); at
+// 400 none of them is more than 1 % off its better side below, 5 % above.
+constexpr int kOwnMaxL = 400, kOwnMaxLDoubled = 256;
 constexpr unsigned long long kSideNone = ~0ull;
 
 // Smaller value first, then the lower pair; -0 and +0 are equal.
@@ -932,7 +940,7 @@ cudaError_t launch_scan_lanes(const Pipe &p, int level, int sms, cudaStream_t s)
     static int bpsm = 0;
     if (!bpsm) bpsm = lane_scan_blocks_per_sm();
     if (bpsm < 1) return cudaErrorInvalidConfiguration;
-    if (p.stride32 > kOwnMaxL)
+    if (p.stride32 > (p.adaptive ? kOwnMaxLDoubled : kOwnMaxL))
         k_scan_lanes<true><<<sms * bpsm, 32 * kLaneWarps, 0, s>>>(p, level);
     else
         k_scan_lanes<false><<<sms * bpsm, 32 * kLaneWarps, 0, s>>>(p, level);
