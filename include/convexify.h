@@ -432,7 +432,7 @@ int cvx_grid_convexify(cvx_handle *h, const cvx_params *p, const cvx_grid *g, do
  * made the forest.  0 <= K <= 64.  The trees are tabulated per grid point and
  * order first (K sweeps over the grid); workspace: two tables of one record
  * per grid point (W, P, leaf count; with A its upper triangle): 64 bytes for
- * d = 2 and 96 for d = 3, with A 128 and 448. */
+ * d = 2 and 96 for d = 3, with A 128 and 448; and two of one byte per point. */
 int cvx_grid_query(cvx_handle *h, const cvx_params *p, const cvx_grid *g, double beta_k,
                    int32_t det_rule, int32_t nd, const int32_t *off, int32_t K, const double *WK,
                    const int32_t *forest, int64_t n, const double *F, double *W_interp,
